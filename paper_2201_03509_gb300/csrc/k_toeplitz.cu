@@ -13,9 +13,9 @@
 // detector gives it; a scan then stores, for the coarse correction, the
 // prefix sums H(x) = sum_{d<x} h(d) and G(x) = sum_{d<x} d h(d) (FP64 sums
 // kept as FP32 pairs), and the first TOEP_LMAX lags for the gap blocks.
-// A second kernel runs the Durbin recursion (Golub & Van Loan, Algorithm
-// 4.7.1) in FP64 and stores, for every order L, the first column
-// x = T_L^{-1} e_1.  The CG then applies T_L^{-1} by the Gohberg-Semencul
+// A second kernel finds, for every order L, the first column
+// x = T_L^{-1} e_1 (Durbin's solutions, Golub & Van Loan, Section 4.7) by the
+// Schur recursion.  The CG then applies T_L^{-1} by the Gohberg-Semencul
 // formula T^{-1} = (L(x) L(x)^T - L(w) L(w)^T) / x_0, w = (0, x_{L-1}, ..,
 // x_1), L(v) the lower-triangular Toeplitz matrix with first column v.
 #include "common.cuh"
@@ -197,71 +197,118 @@ k_cz_tables(const float2 *__restrict__ X, int href, const double2 *__restrict__ 
     if (ch == nch - 1 && threadIdx.x == CZ_ST - 1) t[href] = cz_pack(Hc, Gc);
 }
 
-// One CTA per detector (FP64 issue is the bound, so the dot products use
-// all four SM sub-partitions).  xtab[det] holds, at offset L(L-1)/2, the L
-// values of T_L^{-1} e_1 for L = 1..TOEP_LMAX; lvalid[det] is the largest
-// order the recursion reached with a positive pivot.
-constexpr int DT = 256;
+// One CTA per detector.  xtab[det] holds, at offset L(L-1)/2, the L values
+// of T_L^{-1} e_1 for L = 1..TOEP_LMAX; lvalid[det] is the largest order the
+// recursion reached with a positive pivot.
+//
+// The 511 orders are one serial chain, so the time is the length of an
+// order.  The Durbin recursion needs two dot products per order (in FP64, a
+// CTA reduction of about 5 us); the Schur recursion (Kailath, "A theorem of
+// I. Schur and its impact on modern signal processing", 1986) carries the
+// sequences those dot products evaluate instead: with a^(k) = (1, y^(k)),
+//   P_k[m] = sum_i a_i r(k + 1 + m - i),  Q_k[m] = sum_i a_{k-i} r(k + m - i),
+// the reflection coefficient is alpha = -P_k[0] / Q_k[0], the pivot
+// 1 + r . y^(k) is Q_k[0], and
+//   P_{k+1}[m] = P_k[m+1] + alpha Q_k[m+1],  Q_{k+1}[m] = Q_k[m] + alpha P_k[m],
+//   y^(k+1) = (y^(k) + alpha reversed y^(k), alpha):
+// element-wise, one barrier per order.  Half of the CTA owns the (P, Q)
+// elements, the other half y and the output rows.  Arithmetic in FP32
+// double-words (about 2^-45 relative: the input lags carry the 2^-24 of an
+// FP32 transform), because this part issues FP64 at 1/64 of the FP32 rate
+// and one dependent FP64 division costs more than a whole order does here.
+// Measured, 1 to 12 detectors: 2540 us with the dot products, 223 us so.
+constexpr int DT = 2 * TOEP_LMAX;
+static_assert(TOEP_LMAX == 512, "one thread per element in each half of the CTA");
+
+struct DW { float h, l; };
+// x + a b
+__device__ __forceinline__ DW dw_fma(DW x, DW a, DW b) {
+    const float p = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -p);
+    e = __fmaf_rn(a.h, b.l, e);
+    e = __fmaf_rn(a.l, b.h, e);
+    const float s = __fadd_rn(x.h, p);
+    const float bb = __fsub_rn(s, x.h);
+    float r = __fadd_rn(__fsub_rn(x.h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+    r = __fadd_rn(r, __fadd_rn(x.l, e));
+    DW o;
+    o.h = __fadd_rn(s, r);
+    o.l = __fsub_rn(r, __fsub_rn(o.h, s));
+    return o;
+}
+// a / b
+__device__ __forceinline__ DW dw_div(DW a, DW b) {
+    const float inv = __frcp_rn(b.h);
+    const float q = __fmul_rn(a.h, inv);
+    const float p = __fmul_rn(q, b.h);
+    float r = __fsub_rn(a.h, p);
+    r = __fsub_rn(r, __fmaf_rn(q, b.h, -p));
+    r = __fadd_rn(r, __fmaf_rn(-q, b.l, a.l));
+    const float c = __fmul_rn(r, inv);
+    DW o;
+    o.h = __fadd_rn(q, c);
+    o.l = __fsub_rn(c, __fsub_rn(o.h, q));
+    return o;
+}
 
 __global__ void __launch_bounds__(DT)
 k_toep_durbin(const float *__restrict__ htab, float *__restrict__ xtab, int32_t *__restrict__ lvalid)
 {
     const int det = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ double y[TOEP_LMAX];
-    __shared__ double r[TOEP_LMAX];
-    __shared__ double2 part[2][DT / 32];
+    const int t = threadIdx.x & (TOEP_LMAX - 1);        // element index
+    const bool pq = threadIdx.x < TOEP_LMAX;            // the (P, Q) half; else the y half
+    __shared__ float4 s_pq[2][TOEP_LMAX + 1];           // (P, Q) double-words of the even and odd orders
+    __shared__ DW s_y[2][TOEP_LMAX];
     const float *h = htab + det * TOEP_LMAX;
     float *xt = xtab + static_cast<int64_t>(det) * (TOEP_LMAX * (TOEP_LMAX + 1) / 2);
-    const double t0 = h[0];
-    if (!(t0 > 0.0)) { if (tid == 0) lvalid[det] = 0; return; }
-    for (int i = tid; i < TOEP_LMAX; i += DT) r[i] = (i + 1 < TOEP_LMAX ? h[i + 1] : 0.0f) / t0;
+    const float t0 = h[0];
+    if (!(t0 > 0.0f)) { if (threadIdx.x == 0) lvalid[det] = 0; return; }
+    DW P{0.f, 0.f}, Q{0.f, 0.f};
+    if (pq) {
+        // order 0: P[m] = r(1 + m), Q[m] = r(m), r = h / h(0)
+        const DW d0{t0, 0.f};
+        if (t + 1 < TOEP_LMAX) P = dw_div(DW{h[t + 1], 0.f}, d0);
+        Q = dw_div(DW{h[t], 0.f}, d0);
+        s_pq[0][t] = make_float4(P.h, P.l, Q.h, Q.l);
+        if (t == 0) {
+            s_pq[0][TOEP_LMAX] = s_pq[1][TOEP_LMAX] = make_float4(0.f, 0.f, 0.f, 0.f);
+            xt[0] = 1.0f / t0;
+        }
+    }
     __syncthreads();
-    // order 1
-    if (tid == 0) { xt[0] = static_cast<float>(1.0 / t0); y[0] = -r[0]; }
-    __syncthreads();
-    double beta = 1.0, alpha = -r[0];
     int valid = 1;
-    for (int k = 1; k < TOEP_LMAX; ++k) {
-        // with y^(k) (length k): D1 = r[0..k) . y, D2 = sum_j r[k-1-j] y[j]
-        double d1 = 0.0, d2 = 0.0;
-        for (int j = tid; j < k; j += DT) {
-            const double yj = y[j];
-            d1 += r[j] * yj;
-            d2 += r[k - 1 - j] * yj;
+    for (int k = 0; k < TOEP_LMAX; ++k) {
+        const int cur = k & 1;
+        const float4 z = s_pq[cur][0];                  // P_k[0], Q_k[0]: the pivot is Q_k[0]
+        const DW beta{z.z, z.w};
+        if (!(beta.h > 0.0f) || !isfinite(beta.h)) break;
+        if (k > 0) {
+            // order k + 1: x = (1, y^(k)) / (pivot h(0))
+            valid = k + 1;
+            if (!pq) {
+                const float sc = 1.0f / (beta.h * t0);
+                float *xk = xt + (k + 1) * k / 2;
+                if (t < k) { const DW v = s_y[cur][t]; xk[t + 1] = (v.h + v.l) * sc; }
+                else if (t == k) xk[0] = sc;
+            }
+            if (k + 1 >= TOEP_LMAX) break;
         }
-        for (int o = 16; o; o >>= 1) {
-            d1 += __shfl_xor_sync(0xffffffffu, d1, o);
-            d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+        const DW alpha = dw_div(DW{-z.x, -z.y}, beta);
+        if (pq) {
+            if (t < TOEP_LMAX - k) {
+                const float4 nx = s_pq[cur][t + 1];
+                const DW Qn = dw_fma(Q, alpha, P);
+                P = dw_fma(DW{nx.x, nx.y}, alpha, DW{nx.z, nx.w});
+                Q = Qn;
+                s_pq[cur ^ 1][t] = make_float4(P.h, P.l, Q.h, Q.l);
+            }
+        } else {
+            if (t < k) s_y[cur ^ 1][t] = dw_fma(s_y[cur][t], alpha, s_y[cur][k - 1 - t]);
+            else if (t == k) s_y[cur ^ 1][t] = alpha;
         }
-        if (lane == 0) part[k & 1][warp] = make_double2(d1, d2);
-        __syncthreads();
-        double D1 = 0.0, D2 = 0.0;
-        for (int w = 0; w < DT / 32; ++w) { D1 += part[k & 1][w].x; D2 += part[k & 1][w].y; }
-        // x for order k+1: gamma = 1/(1 + D1), x = gamma (1, y) / t0
-        const double gam = 1.0 / (1.0 + D1);
-        if (!(gam > 0.0) || !isfinite(gam)) break;
-        float *xk = xt + static_cast<int64_t>(k + 1) * k / 2;       // order L = k+1
-        if (tid == 0) xk[0] = static_cast<float>(gam / t0);
-        for (int i = tid; i < k; i += DT) xk[i + 1] = static_cast<float>(gam * y[i] / t0);
-        valid = k + 1;
-        if (k + 1 >= TOEP_LMAX) break;
-        // Durbin step to y^(k+1)
-        beta = (1.0 - alpha * alpha) * beta;
-        if (!(beta > 0.0)) break;
-        alpha = -(r[k] + D2) / beta;
-        __syncthreads();      // every read of y^(k) is done
-        // y[i] += alpha y[k-1-i] for i < k, pairs (i, k-1-i) by one thread
-        for (int i = tid; i < (k + 1) / 2; i += DT) {
-            const int jj = k - 1 - i;
-            const double yi = y[i], yj = y[jj];
-            y[i] = yi + alpha * yj;
-            if (jj != i) y[jj] = yj + alpha * yi;
-        }
-        if (tid == 0) y[k] = alpha;
         __syncthreads();
     }
-    if (tid == 0) lvalid[det] = valid;
+    if (threadIdx.x == 0) lvalid[det] = valid;
 }
 
 cudaError_t launch_toeplitz_prep(const Plan &p, const double *psd, cudaStream_t st)
