@@ -224,8 +224,8 @@ enum {
     TOD_KT_GAIN_ROWS,         /* k_gain_rows */
     TOD_KT_GAIN_COLSINV,      /* k_gain_colsinv */
     TOD_KT_GAIN_FIN,          /* k_gain_fin */
-    TOD_KT_TOEP_KERNEL,       /* the gap kernel h(d) and its prefix sums: k_cz_fill, the k_cz_fft
-                                 passes (log2 of twice the reference length, halved, rounded up),
+    TOD_KT_TOEP_KERNEL,       /* the gap kernel h(d) and its prefix sums: the k_cz_fft passes
+                                 (log2 of twice the reference length over 7, rounded up),
                                  k_cz_sums, k_cz_tables */
     TOD_KT_TOEP_DURBIN,       /* k_toep_durbin */
     TOD_KT_NC_FLAG_COUNT,     /* k_nc_flag_count */
@@ -386,7 +386,7 @@ tod_status tod_sample_ncorr(tod_plan *p, const float *d, const float *s,
  *   tod_ncorr_prepare builds, from psd (double[ndet][3], device), the
  *   per-detector gap preconditioner tables the plan holds (the Toeplitz
  *   autocovariance of the CG operator at every lag of a power-of-two
- *   reference length, by one FFT per detector, its prefix sums for the
+ *   reference length, by one FFT per two detectors, its prefix sums for the
  *   coarse correction, and the Durbin solutions of its first 512 lags),
  *   overwriting the previous ones.
  *   tod_sample_ncorr_prepared is tod_sample_ncorr (same arguments, results

@@ -872,7 +872,7 @@ tod_status tod_plan_create(tod_plan **out, const tod_band_desc *band)
         p->cz_href = 1024;
         while (p->cz_href < maxlen) p->cz_href *= 2;
         const size_t M2 = 2 * static_cast<size_t>(p->cz_href);
-        if ((e = dev_upload(*p, p->czfft, static_cast<float2 *>(nullptr), 2 * static_cast<size_t>(p->ndet) * M2)))
+        if ((e = dev_upload(*p, p->czfft, static_cast<float2 *>(nullptr), 2 * static_cast<size_t>((p->ndet + 1) / 2) * M2)))
             return fail(e);
         if ((e = dev_upload(*p, p->cztab, static_cast<float4 *>(nullptr),
                             static_cast<size_t>(p->ndet) * (static_cast<size_t>(p->cz_href) + 1))))
@@ -887,8 +887,6 @@ tod_status tod_plan_create(tod_plan **out, const tod_band_desc *band)
             return fail(e);
         if ((e = dev_upload(*p, p->czl, static_cast<float *>(nullptr),
                             static_cast<size_t>(p->nq) * 2 * TX_CBMAX * (TX_CZB + 1))))
-            return fail(e);
-        if ((e = dev_upload(*p, p->htab, static_cast<float *>(nullptr), static_cast<size_t>(p->ndet) * TOEP_LMAX)))
             return fail(e);
         if ((e = dev_upload(*p, p->xtab, static_cast<float *>(nullptr),
                             static_cast<size_t>(p->ndet) * (TOEP_LMAX * (TOEP_LMAX + 1) / 2))))

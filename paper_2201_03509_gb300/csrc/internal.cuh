@@ -121,14 +121,13 @@ struct Plan {
     int64_t *tile_t0 = nullptr;
     float2 *trig = nullptr;          // [TOD_N_PSI] (cos 2psi, sin 2psi) at bin centres, FP32
     // correlated-noise preconditioner (k_toeplitz.cu)
-    float *htab = nullptr;           // [ndet][TOEP_LMAX] gap-kernel h(d)
     float *xtab = nullptr;           // [ndet][TOEP_LMAX (TOEP_LMAX+1)/2] T_L^{-1} e_1 per order
     int32_t *lvalid = nullptr;       // [ndet]
     // coarse correction: the kernel h(d) at every lag below cz_href (a power
     // of two >= the longest detscan), from one FFT of length 2 cz_href per
-    // detector, and its prefix sums
+    // two detectors, and its prefix sums
     int32_t cz_href = 0;
-    float2 *czfft = nullptr;         // [2][ndet][2 cz_href] FFT work
+    float2 *czfft = nullptr;         // [2][(ndet + 1)/2][2 cz_href] FFT work, then the kernels
     float4 *cztab = nullptr;         // [ndet][cz_href + 1] (H, G) as FP32 pairs: H(x) = sum_{d<x} h(d), G: d h(d)
     int32_t *gbpos = nullptr;        // [nq][TX_GBMAX] first sample (within the detscan) of each block
     float *czsz = nullptr;           // [czcap][TX_CZJ] S Z entries by flagged rank

@@ -9,192 +9,277 @@
 // be symmetric positive definite, and a kernel shared by all detscans of a
 // detector is close enough), at every lag d < H at once: h(d) is the real
 // part of the length-2H DFT of the even sequence a_k = gamma_k (k < H),
-// a_{2H-k} = gamma_k, a_H = 0, divided by 2H.  One FP32 Stockham FFT per
-// detector gives it; a scan then stores, for the coarse correction, the
-// prefix sums H(x) = sum_{d<x} h(d) and G(x) = sum_{d<x} d h(d) (FP64 sums
-// kept as FP32 pairs), and the first TOEP_LMAX lags for the gap blocks.
+// a_{2H-k} = gamma_k, a_H = 0, divided by 2H.  The transform of a real even
+// sequence is real, so one complex FP32 FFT serves two detectors (one in the
+// real, one in the imaginary part).  A scan then stores, for the coarse
+// correction, the prefix sums H(x) = sum_{d<x} h(d) and G(x) = sum_{d<x} d h(d)
+// (FP32 double-words); the gap blocks take the first TOEP_LMAX lags.
 // A second kernel finds, for every order L, the first column
 // x = T_L^{-1} e_1 (Durbin's solutions, Golub & Van Loan, Section 4.7) by the
 // Schur recursion.  The CG then applies T_L^{-1} by the Gohberg-Semencul
 // formula T^{-1} = (L(x) L(x)^T - L(w) L(w)^T) / x_0, w = (0, x_{L-1}, ..,
 // x_1), L(v) the lower-triangular Toeplitz matrix with first column v.
 #include "common.cuh"
+#include "fft_reg.cuh"
 #include "internal.cuh"
 
 namespace tg {
 
-constexpr int CZ_FT = 256;      // threads per CTA of the fill and FFT passes
-constexpr int CZ_ST = 256;      // threads of the prefix-table kernels
+constexpr int CZ_T = 256;       // threads per CTA of the FFT passes and the scans
+constexpr int CZ_C = 32;        // columns (consecutive j) of an FFT tile
+constexpr int CZ_PER = 8;       // lags per thread of the scans
+constexpr int CZ_CHUNK = CZ_T * CZ_PER;
 
-// a_k for k < 2H (gamma at f_k = k f_samp / (2H); a_0 = a_H = 0)
-__global__ void __launch_bounds__(CZ_FT)
-k_cz_fill(const double *__restrict__ psd, int href, double fsamp, float2 *__restrict__ a)
-{
-    const int det = blockIdx.y;
-    const int M = 2 * href;
-    const int k = blockIdx.x * CZ_FT + threadIdx.x;
-    if (k >= M) return;
-    const double sig0 = psd[3 * det], fk = psd[3 * det + 1], al = psd[3 * det + 2];
-    const float s2 = static_cast<float>(sig0 * sig0);
-    const float fscale = static_cast<float>(fsamp / (2.0 * href * fk));
-    const float mal = static_cast<float>(-al);
-    const int kk = k <= href ? k : M - k;
-    float g = 0.f;
-    if (kk > 0 && kk < href) {
-        const float r = exp2f(mal * log2f(static_cast<float>(kk) * fscale));
-        g = s2 / (1.0f + 1.0f / r);           // sigma0^2 r / (1 + r), also for r = 0 or inf
-    }
-    a[static_cast<int64_t>(det) * M + k] = make_float2(g, 0.f);
+// FP32 double-word (head + tail, |tail| <= ulp(head)/2): about 2^-45 relative
+// per operation, at the FP32 rate (FP64 issues at 1/64 of it on this part).
+struct DW { float h, l; };
+__device__ __forceinline__ DW dw_renorm(float s, float r) {
+    DW o;
+    o.h = __fadd_rn(s, r);
+    o.l = __fsub_rn(r, __fsub_rn(o.h, s));
+    return o;
+}
+// x + (p + e), e small against p
+__device__ __forceinline__ DW dw_add2(DW x, float p, float e) {
+    const float s = __fadd_rn(x.h, p);
+    const float bb = __fsub_rn(s, x.h);
+    float r = __fadd_rn(__fsub_rn(x.h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+    r = __fadd_rn(r, __fadd_rn(x.l, e));
+    return dw_renorm(s, r);
+}
+__device__ __forceinline__ DW dw_add(DW x, DW y) { return dw_add2(x, y.h, y.l); }
+// x + a b
+__device__ __forceinline__ DW dw_fma(DW x, DW a, DW b) {
+    const float p = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -p);
+    e = __fmaf_rn(a.h, b.l, e);
+    e = __fmaf_rn(a.l, b.h, e);
+    return dw_add2(x, p, e);
+}
+// a / b
+__device__ __forceinline__ DW dw_div(DW a, DW b) {
+    const float inv = __frcp_rn(b.h);
+    const float q = __fmul_rn(a.h, inv);
+    const float p = __fmul_rn(q, b.h);
+    float r = __fsub_rn(a.h, p);
+    r = __fsub_rn(r, __fmaf_rn(q, b.h, -p));
+    r = __fadd_rn(r, __fmaf_rn(-q, b.l, a.l));
+    return dw_renorm(q, __fmul_rn(r, inv));
 }
 
-// One radix-R Stockham pass (forward DFT) over every detector's length-M
-// sequence, Ns points of each sub-transform already done (Ns, M powers of
-// two).  Thread j < M/R reads x[j + r M/R], twiddles by exp(-2 pi i r k /
-// (Ns R)), k = j mod Ns, and writes the R outputs to (j - k) R + k + r Ns.
-template <int R>
-__global__ void __launch_bounds__(CZ_FT)
-k_cz_fft(const float2 *__restrict__ src, float2 *__restrict__ dst, int M, int Ns)
+// gamma at mode k of the length-2H sequence (f_k = k f_samp / (2H); a_0 = a_H = 0)
+struct CzDet { float s2, fscale, mal; };
+__device__ __forceinline__ float cz_gamma(const CzDet &c, int k, int href) {
+    const int kk = k <= href ? k : 2 * href - k;
+    if (kk == 0 || kk >= href) return 0.f;
+    const float r = exp2f(c.mal * log2f(static_cast<float>(kk) * c.fscale));
+    return c.s2 / (1.0f + 1.0f / r);          // sigma0^2 r / (1 + r), also for r = 0 or inf
+}
+
+// One radix-R Stockham pass (R = 8 A, forward DFT) over the length-M sequence
+// of every detector pair, Ns points of each sub-transform done (powers of
+// two).  Point j < M/R reads x[j + r M/R], twiddles by exp(-2 pi i r k /
+// (Ns R)), k = j mod Ns, and writes output r' to (j - k) R + k + r' Ns.
+// A CTA takes CZ_C consecutive j: the R-point DFTs are A-point DFTs of the
+// rows r = 8 n1 + n2 in registers, a table twiddle, one exchange through
+// shared memory, and 8-point DFTs over n2.  FIRST evaluates gamma in place
+// of a load (and writes through shared memory, since its outputs of one j
+// are consecutive); LAST keeps the lags d < H only, real part to the first
+// detector's kernel, imaginary part to the second's.
+// Every radix-R pass reads and writes the sequence once, so R up to 128
+// takes three passes where radix 4 took ten; per point one sincospif in
+// eight instead of three in four.  Bound: L2 bandwidth and the gamma
+// evaluations.  Fill, FFT and tables of 12 detectors, H = 262144: 1022 us by
+// radix-4 passes per detector and FP64 scans, 151 us so; of 2 detectors,
+// H = 32768: 166 us, 37 us.
+template <int A, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(CZ_T)
+k_cz_fft(const float2 *__restrict__ src, float2 *__restrict__ dst, const double *__restrict__ psd, int ndet, int href,
+         double fsamp, int Ns, float *__restrict__ hout)
 {
-    const int det = blockIdx.y;
-    const int MR = M / R;
-    const int j = blockIdx.x * CZ_FT + threadIdx.x;
-    if (j >= MR) return;
-    const float2 *x = src + static_cast<int64_t>(det) * M;
-    float2 *y = dst + static_cast<int64_t>(det) * M;
-    const int k = j & (Ns - 1);
-    float2 v[R];
+    constexpr int R = 8 * A;
+    constexpr int IT = (A * CZ_C + CZ_T - 1) / CZ_T;
+    __shared__ float2 t[R * (CZ_C + 1)];
+    __shared__ float2 wt[R];                   // W_R^{n2 k1} at n2 A + k1
+    __shared__ CzDet s_det[2];
+    const int pair = blockIdx.y, M = 2 * href, MR = M / R;
+    const int j0 = blockIdx.x * CZ_C;
+    if (threadIdx.x < R) {
+        const int n2 = threadIdx.x / A, k1 = threadIdx.x % A;
+        float sn, cs;
+        sincospif(-2.0f * static_cast<float>(n2 * k1) / static_cast<float>(R), &sn, &cs);
+        wt[threadIdx.x] = make_float2(cs, sn);
+    }
+    if (FIRST && threadIdx.x < 2) {
+        const int det = min(2 * pair + static_cast<int>(threadIdx.x), ndet - 1);
+        const double sig0 = psd[3 * det], fk = psd[3 * det + 1];
+        s_det[threadIdx.x] = CzDet{static_cast<float>(sig0 * sig0), static_cast<float>(fsamp / (2.0 * href * fk)),
+                                   static_cast<float>(-psd[3 * det + 2])};
+    }
+    __syncthreads();
+    {
+        const int c = threadIdx.x & (CZ_C - 1), n2 = threadIdx.x / CZ_C;
+        const int j = j0 + c;
+        float2 v[A];
+        if (FIRST) {
+            const CzDet d0 = s_det[0], d1 = s_det[1];
+            const bool two = 2 * pair + 1 < ndet;
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = x[j + r * MR];
-    if (Ns > 1) {
+            for (int n1 = 0; n1 < A; ++n1) {
+                const int k = j + (8 * n1 + n2) * MR;
+                v[n1] = make_float2(cz_gamma(d0, k, href), two ? cz_gamma(d1, k, href) : 0.f);
+            }
+        } else {
+            const float2 *x = src + static_cast<int64_t>(pair) * M;
 #pragma unroll
-        for (int r = 1; r < R; ++r) {
-            float sn, cs;
-            sincospif(-2.0f * static_cast<float>(r * k) / static_cast<float>(Ns * R), &sn, &cs);
-            v[r] = make_float2(v[r].x * cs - v[r].y * sn, v[r].x * sn + v[r].y * cs);
+            for (int n1 = 0; n1 < A; ++n1) v[n1] = x[j + (8 * n1 + n2) * MR];
+            // W^{r k}, r = 8 n1 + n2: the factors of n2 and of each bit of n1
+            const int k = j & (Ns - 1);
+            const float inv = -2.0f / (static_cast<float>(Ns) * static_cast<float>(R));     // a power of two
+            float2 w[A];
+            {
+                float sn, cs;
+                sincospif(static_cast<float>(n2 * k) * inv, &sn, &cs);
+                w[0] = make_float2(cs, sn);
+            }
+#pragma unroll
+            for (int b = 1; b < A; b <<= 1) {
+                float sn, cs;
+                sincospif(static_cast<float>(8 * b * k) * inv, &sn, &cs);
+#pragma unroll
+                for (int n1 = 0; n1 < b; ++n1) w[n1 + b] = vmul(w[n1], make_float2(cs, sn));
+            }
+#pragma unroll
+            for (int n1 = 0; n1 < A; ++n1) v[n1] = vmul(v[n1], w[n1]);
+        }
+        RDft<A, false, float2>::run(v);
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) t[(n2 * A + k1) * CZ_C + c] = vmul(v[k1], wt[n2 * A + k1]);
+    }
+    __syncthreads();
+    float2 u[IT][8];
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        const int w = threadIdx.x + i * CZ_T, c = w & (CZ_C - 1), k1 = w / CZ_C;
+        if (k1 >= A) continue;
+#pragma unroll
+        for (int n2 = 0; n2 < 8; ++n2) u[i][n2] = t[(n2 * A + k1) * CZ_C + c];
+        RDft<8, false, float2>::run(u[i]);
+    }
+    if (FIRST) __syncthreads();                // t is reused for the outputs
+    float2 *y = dst + static_cast<int64_t>(pair) * M;
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        const int w = threadIdx.x + i * CZ_T, c = w & (CZ_C - 1), k1 = w / CZ_C;
+        if (k1 >= A) continue;
+        const int j = j0 + c, k = j & (Ns - 1);
+#pragma unroll
+        for (int k2 = 0; k2 < 8; ++k2) {
+            const int r = k1 + A * k2;
+            if (FIRST) {
+                t[c * (R + 1) + r] = u[i][k2];
+            } else if (LAST) {
+                const int d = j + r * Ns;      // Ns = M/R: j < Ns
+                if (d < href) {
+                    const float inv = 1.0f / static_cast<float>(M);              // a power of two
+                    hout[static_cast<int64_t>(2 * pair) * href + d] = u[i][k2].x * inv;
+                    if (2 * pair + 1 < ndet) hout[static_cast<int64_t>(2 * pair + 1) * href + d] = u[i][k2].y * inv;
+                }
+            } else {
+                y[(j - k) * R + k + r * Ns] = u[i][k2];
+            }
         }
     }
-    float2 o[R];
-    if constexpr (R == 2) {
-        o[0] = make_float2(v[0].x + v[1].x, v[0].y + v[1].y);
-        o[1] = make_float2(v[0].x - v[1].x, v[0].y - v[1].y);
-    } else {
-        const float2 a0 = make_float2(v[0].x + v[2].x, v[0].y + v[2].y);
-        const float2 a1 = make_float2(v[0].x - v[2].x, v[0].y - v[2].y);
-        const float2 a2 = make_float2(v[1].x + v[3].x, v[1].y + v[3].y);
-        const float2 a3 = make_float2(v[1].y - v[3].y, v[3].x - v[1].x);     // (v1 - v3) (-i)
-        o[0] = make_float2(a0.x + a2.x, a0.y + a2.y);
-        o[1] = make_float2(a1.x + a3.x, a1.y + a3.y);
-        o[2] = make_float2(a0.x - a2.x, a0.y - a2.y);
-        o[3] = make_float2(a1.x - a3.x, a1.y - a3.y);
-    }
-    const int base = (j - k) * R + k;
-#pragma unroll
-    for (int r = 0; r < R; ++r) y[base + r * Ns] = o[r];
-}
-
-__device__ __forceinline__ float4 cz_pack(double H, double G) {
-    const float hh = __double2float_rn(H), gh = __double2float_rn(G);
-    return make_float4(hh, __double2float_rn(H - static_cast<double>(hh)), gh,
-                       __double2float_rn(G - static_cast<double>(gh)));
-}
-
-// h(d) = Re X_d / 2H for d < H; tab[x] = (H(x), G(x)) for x <= H (FP64 sums
-// of the FP32 h values, as FP32 pairs); htab = the first TOEP_LMAX lags.
-// The lags of a detector are cut into chunks of CZ_ST threads x cz_per(H)
-// lags, one CTA each: k_cz_sums adds up every chunk, k_cz_tables scans
-// within its chunk from the sum of the chunks before it.
-__host__ __device__ __forceinline__ int cz_per(int href) { return href >= 64 * CZ_ST ? 64 : href / CZ_ST; }
-
-__device__ __forceinline__ void cz_stretch(const float2 *__restrict__ x, int d0, int per, float inv, double &sh,
-                                           double &sg) {
-    sh = 0.0;
-    sg = 0.0;
-    for (int i = 0; i < per; ++i) {
-        const double h = static_cast<double>(x[d0 + i].x * inv);
-        sh += h;
-        sg += static_cast<double>(d0 + i) * h;
+    if (FIRST) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < R * CZ_C; e += CZ_T) y[j0 * R + e] = t[(e / R) * (R + 1) + (e & (R - 1))];
     }
 }
 
-__global__ void __launch_bounds__(CZ_ST)
-k_cz_sums(const float2 *__restrict__ X, int href, double2 *__restrict__ csum)
-{
-    const int det = blockIdx.y, nch = gridDim.x;
-    const int per = cz_per(href);
-    const float2 *x = X + static_cast<int64_t>(det) * 2 * href;
-    const float inv = 1.0f / static_cast<float>(2 * href);      // exact: a power of two
-    double sh, sg;
-    cz_stretch(x, (blockIdx.x * CZ_ST + threadIdx.x) * per, per, inv, sh, sg);
-    for (int o = 16; o; o >>= 1) {
-        sh += __shfl_xor_sync(0xffffffffu, sh, o);
-        sg += __shfl_xor_sync(0xffffffffu, sg, o);
-    }
-    __shared__ double wh[CZ_ST / 32], wg[CZ_ST / 32];
+// tab[x] = (H(x), G(x)) for x <= H as double-words.  The lags of a detector
+// are cut into chunks of CZ_CHUNK, one CTA each: k_cz_sums adds up every
+// chunk, k_cz_tables scans within its chunk from the sum of the chunks
+// before it.  Fixed order of the sums throughout.
+struct HG { DW h, g; };
+__device__ __forceinline__ HG hg_zero() { return HG{{0.f, 0.f}, {0.f, 0.f}}; }
+__device__ __forceinline__ HG hg_add(const HG &a, const HG &b) { return HG{dw_add(a.h, b.h), dw_add(a.g, b.g)}; }
+__device__ __forceinline__ void hg_lag(HG &a, float h, int d) {
+    const float fd = static_cast<float>(d);                 // d < 2^24: exact
+    const float p = __fmul_rn(fd, h);
+    a.h = dw_add2(a.h, h, 0.f);
+    a.g = dw_add2(a.g, p, __fmaf_rn(fd, h, -p));
+}
+__device__ __forceinline__ HG hg_shfl_up(const HG &a, int o) {
+    return HG{{__shfl_up_sync(0xffffffffu, a.h.h, o), __shfl_up_sync(0xffffffffu, a.h.l, o)},
+              {__shfl_up_sync(0xffffffffu, a.g.h, o), __shfl_up_sync(0xffffffffu, a.g.l, o)}};
+}
+// Exclusive scan of one value per thread over the CTA (the total in *tot)
+__device__ __forceinline__ HG hg_exscan(const HG &own, HG *s_w, HG *tot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) { wh[warp] = sh; wg[warp] = sg; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double th = 0.0, tg_ = 0.0;
-        for (int w = 0; w < CZ_ST / 32; ++w) { th += wh[w]; tg_ += wg[w]; }
-        csum[det * nch + blockIdx.x] = make_double2(th, tg_);
-    }
-}
-
-__global__ void __launch_bounds__(CZ_ST)
-k_cz_tables(const float2 *__restrict__ X, int href, const double2 *__restrict__ csum, float *__restrict__ htab,
-            float4 *__restrict__ tab)
-{
-    const int det = blockIdx.y, ch = blockIdx.x, nch = gridDim.x;
-    const int per = cz_per(href);
-    const float2 *x = X + static_cast<int64_t>(det) * 2 * href;
-    float4 *t = tab + static_cast<int64_t>(det) * (href + 1);
-    const float inv = 1.0f / static_cast<float>(2 * href);
-    const int d0 = (ch * CZ_ST + threadIdx.x) * per;
-    double sh, sg;
-    cz_stretch(x, d0, per, inv, sh, sg);
-    // exclusive scan of (sh, sg) over the CTA, offset by the earlier chunks
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double ih = sh, ig = sg;
+    HG inc = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const double uh = __shfl_up_sync(0xffffffffu, ih, o), ug = __shfl_up_sync(0xffffffffu, ig, o);
-        if (lane >= o) { ih += uh; ig += ug; }
+        const HG up = hg_shfl_up(inc, o);
+        if (lane >= o) inc = hg_add(up, inc);
     }
-    __shared__ double wh[CZ_ST / 32], wg[CZ_ST / 32];
-    __shared__ double base[2];
-    if (lane == 31) { wh[warp] = ih; wg[warp] = ig; }
-    if (threadIdx.x == 0) {
-        double bh = 0.0, bg = 0.0;
-        for (int c = 0; c < ch; ++c) { const double2 v = csum[det * nch + c]; bh += v.x; bg += v.y; }
-        base[0] = bh;
-        base[1] = bg;
-    }
+    HG ex = hg_shfl_up(inc, 1);
+    if (lane == 0) ex = hg_zero();
+    if (lane == 31) s_w[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-        constexpr int NW = CZ_ST / 32;
-        const double ownh = lane < NW ? wh[lane] : 0.0, owng = lane < NW ? wg[lane] : 0.0;
-        double vh = ownh, vg = owng;
+    HG base = hg_zero(), all = hg_zero();
+    for (int w = 0; w < CZ_T / 32; ++w) {
+        if (w == warp) base = all;
+        all = hg_add(all, s_w[w]);
+    }
+    *tot = all;
+    __syncthreads();
+    return hg_add(base, ex);
+}
+
+__global__ void __launch_bounds__(CZ_T)
+k_cz_sums(const float *__restrict__ hk, int href, float4 *__restrict__ csum)
+{
+    __shared__ HG s_w[CZ_T / 32];
+    const int det = blockIdx.y, d0 = blockIdx.x * CZ_CHUNK + threadIdx.x * CZ_PER;
+    const float *h = hk + static_cast<int64_t>(det) * href;
+    HG s = hg_zero(), tot;
+    if (d0 < href) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double uh = __shfl_up_sync(0xffffffffu, vh, o), ug = __shfl_up_sync(0xffffffffu, vg, o);
-            if (lane >= o) { vh += uh; vg += ug; }
-        }
-        if (lane < NW) {
-            wh[lane] = vh - ownh;              // exclusive over the warps
-            wg[lane] = vg - owng;
-        }
+        for (int i = 0; i < CZ_PER; ++i) hg_lag(s, h[d0 + i], d0 + i);
     }
-    __syncthreads();
-    double Hc = base[0] + wh[warp] + (ih - sh), Gc = base[1] + wg[warp] + (ig - sg);
-    for (int i = 0; i < per; ++i) {
-        const int d = d0 + i;
-        const float h32 = x[d].x * inv;
-        if (d < TOEP_LMAX) htab[det * TOEP_LMAX + d] = h32;
-        t[d] = cz_pack(Hc, Gc);
-        Hc += static_cast<double>(h32);
-        Gc += static_cast<double>(d) * static_cast<double>(h32);
+    hg_exscan(s, s_w, &tot);
+    if (threadIdx.x == 0) csum[det * gridDim.x + blockIdx.x] = make_float4(tot.h.h, tot.h.l, tot.g.h, tot.g.l);
+}
+
+__global__ void __launch_bounds__(CZ_T)
+k_cz_tables(const float *__restrict__ hk, int href, const float4 *__restrict__ csum, float4 *__restrict__ tab)
+{
+    __shared__ HG s_w[CZ_T / 32];
+    const int det = blockIdx.y, ch = blockIdx.x, nch = gridDim.x;
+    const int d0 = ch * CZ_CHUNK + threadIdx.x * CZ_PER;
+    const float *h = hk + static_cast<int64_t>(det) * href;
+    float4 *t = tab + static_cast<int64_t>(det) * (href + 1);
+    // the chunks before this one
+    HG b = hg_zero(), base, tot;
+    for (int c = threadIdx.x; c < ch; c += CZ_T) {
+        const float4 v = csum[det * nch + c];
+        b = hg_add(b, HG{{v.x, v.y}, {v.z, v.w}});
     }
-    if (ch == nch - 1 && threadIdx.x == CZ_ST - 1) t[href] = cz_pack(Hc, Gc);
+    hg_exscan(b, s_w, &base);
+    float x[CZ_PER];
+    HG s = hg_zero();
+    if (d0 < href) {
+#pragma unroll
+        for (int i = 0; i < CZ_PER; ++i) { x[i] = h[d0 + i]; hg_lag(s, x[i], d0 + i); }
+    }
+    HG run = hg_add(base, hg_exscan(s, s_w, &tot));
+    if (d0 >= href) return;
+#pragma unroll
+    for (int i = 0; i < CZ_PER; ++i) {
+        t[d0 + i] = make_float4(run.h.h, run.h.l, run.g.h, run.g.l);
+        hg_lag(run, x[i], d0 + i);
+    }
+    if (d0 + CZ_PER == href) t[href] = make_float4(run.h.h, run.h.l, run.g.h, run.g.l);
 }
 
 // One CTA per detector.  xtab[det] holds, at offset L(L-1)/2, the L values
@@ -220,46 +305,15 @@ k_cz_tables(const float2 *__restrict__ X, int href, const double2 *__restrict__ 
 constexpr int DT = 2 * TOEP_LMAX;
 static_assert(TOEP_LMAX == 512, "one thread per element in each half of the CTA");
 
-struct DW { float h, l; };
-// x + a b
-__device__ __forceinline__ DW dw_fma(DW x, DW a, DW b) {
-    const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, e);
-    e = __fmaf_rn(a.l, b.h, e);
-    const float s = __fadd_rn(x.h, p);
-    const float bb = __fsub_rn(s, x.h);
-    float r = __fadd_rn(__fsub_rn(x.h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    r = __fadd_rn(r, __fadd_rn(x.l, e));
-    DW o;
-    o.h = __fadd_rn(s, r);
-    o.l = __fsub_rn(r, __fsub_rn(o.h, s));
-    return o;
-}
-// a / b
-__device__ __forceinline__ DW dw_div(DW a, DW b) {
-    const float inv = __frcp_rn(b.h);
-    const float q = __fmul_rn(a.h, inv);
-    const float p = __fmul_rn(q, b.h);
-    float r = __fsub_rn(a.h, p);
-    r = __fsub_rn(r, __fmaf_rn(q, b.h, -p));
-    r = __fadd_rn(r, __fmaf_rn(-q, b.l, a.l));
-    const float c = __fmul_rn(r, inv);
-    DW o;
-    o.h = __fadd_rn(q, c);
-    o.l = __fsub_rn(c, __fsub_rn(o.h, q));
-    return o;
-}
-
 __global__ void __launch_bounds__(DT)
-k_toep_durbin(const float *__restrict__ htab, float *__restrict__ xtab, int32_t *__restrict__ lvalid)
+k_toep_durbin(const float *__restrict__ hk, int href, float *__restrict__ xtab, int32_t *__restrict__ lvalid)
 {
     const int det = blockIdx.x;
     const int t = threadIdx.x & (TOEP_LMAX - 1);        // element index
     const bool pq = threadIdx.x < TOEP_LMAX;            // the (P, Q) half; else the y half
     __shared__ float4 s_pq[2][TOEP_LMAX + 1];           // (P, Q) double-words of the even and odd orders
     __shared__ DW s_y[2][TOEP_LMAX];
-    const float *h = htab + det * TOEP_LMAX;
+    const float *h = hk + static_cast<int64_t>(det) * href;
     float *xt = xtab + static_cast<int64_t>(det) * (TOEP_LMAX * (TOEP_LMAX + 1) / 2);
     const float t0 = h[0];
     if (!(t0 > 0.0f)) { if (threadIdx.x == 0) lvalid[det] = 0; return; }
@@ -311,44 +365,58 @@ k_toep_durbin(const float *__restrict__ htab, float *__restrict__ xtab, int32_t 
     if (threadIdx.x == 0) lvalid[det] = valid;
 }
 
-cudaError_t launch_toeplitz_prep(const Plan &p, const double *psd, cudaStream_t st)
+template <bool FIRST, bool LAST>
+static void cz_fft_pass(const Plan &p, int lgR, const float2 *src, float2 *dst, const double *psd, int Ns, float *h,
+                        cudaStream_t st)
 {
     const int M = 2 * p.cz_href;
-    float2 *buf[2] = {p.czfft, p.czfft + static_cast<int64_t>(p.ndet) * M};
-    {
-        KTIME(TOD_KT_TOEP_KERNEL);
-        k_cz_fill<<<dim3((M + CZ_FT - 1) / CZ_FT, p.ndet), CZ_FT, 0, st>>>(psd, p.cz_href, p.fsamp, buf[0]);
+    const dim3 grid(M >> (lgR + 5), (p.ndet + 1) / 2);
+    static_assert(CZ_C == 32, "grid");
+    KTIME(TOD_KT_TOEP_KERNEL);
+    switch (lgR) {
+    case 5: k_cz_fft<4, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, h); break;
+    case 6: k_cz_fft<8, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, h); break;
+    default: k_cz_fft<16, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, h); break;
     }
-    int cur = 0, Ns = 1, lg = 0;
+}
+
+cudaError_t launch_toeplitz_prep(const Plan &p, const double *psd, cudaStream_t st)
+{
+    // passes of radix 32, 64 or 128, as equal as log2(M) allows (M >= 2048:
+    // two passes at least; every factor has at least five bits)
+    const int M = 2 * p.cz_href;
+    int lg = 0;
     while ((1 << lg) < M) ++lg;
-    if (lg & 1) {
-        KTIME(TOD_KT_TOEP_KERNEL);
-        k_cz_fft<2><<<dim3((M / 2 + CZ_FT - 1) / CZ_FT, p.ndet), CZ_FT, 0, st>>>(buf[cur], buf[cur ^ 1], M, Ns);
+    const int np = (lg + 6) / 7;
+    const int64_t half = static_cast<int64_t>((p.ndet + 1) / 2) * M;
+    float2 *buf[2] = {p.czfft, p.czfft + half};
+    int cur = 0, Ns = 1;
+    for (int i = 0; i < np; ++i) {
+        const int lgR = (lg + np - 1 - i) / np;
+        // the last pass leaves the kernels (FP32) where its output would go
+        float *h = reinterpret_cast<float *>(buf[cur ^ 1]);
+        if (i == 0) cz_fft_pass<true, false>(p, lgR, nullptr, buf[cur ^ 1], psd, Ns, nullptr, st);
+        else if (i + 1 < np) cz_fft_pass<false, false>(p, lgR, buf[cur], buf[cur ^ 1], psd, Ns, nullptr, st);
+        else cz_fft_pass<false, true>(p, lgR, buf[cur], nullptr, psd, Ns, h, st);
         cur ^= 1;
-        Ns *= 2;
+        Ns <<= lgR;
     }
-    while (Ns < M) {
-        KTIME(TOD_KT_TOEP_KERNEL);
-        k_cz_fft<4><<<dim3((M / 4 + CZ_FT - 1) / CZ_FT, p.ndet), CZ_FT, 0, st>>>(buf[cur], buf[cur ^ 1], M, Ns);
-        cur ^= 1;
-        Ns *= 4;
-    }
-    // chunk sums into the other FFT buffer (free after the last pass)
-    const int nch = p.cz_href / (CZ_ST * cz_per(p.cz_href));
-    double2 *csum = reinterpret_cast<double2 *>(buf[cur ^ 1]);
+    const float *h = reinterpret_cast<const float *>(buf[cur]);
+    float4 *csum = reinterpret_cast<float4 *>(buf[cur ^ 1]);        // the last pass's input is free
+    const int nch = (p.cz_href + CZ_CHUNK - 1) / CZ_CHUNK;
     {
         KTIME(TOD_KT_TOEP_KERNEL);
-        k_cz_sums<<<dim3(nch, p.ndet), CZ_ST, 0, st>>>(buf[cur], p.cz_href, csum);
+        k_cz_sums<<<dim3(nch, p.ndet), CZ_T, 0, st>>>(h, p.cz_href, csum);
     }
     {
         KTIME(TOD_KT_TOEP_KERNEL);
-        k_cz_tables<<<dim3(nch, p.ndet), CZ_ST, 0, st>>>(buf[cur], p.cz_href, csum, p.htab, p.cztab);
+        k_cz_tables<<<dim3(nch, p.ndet), CZ_T, 0, st>>>(h, p.cz_href, csum, p.cztab);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     {
         KTIME(TOD_KT_TOEP_DURBIN);
-        k_toep_durbin<<<p.ndet, DT, 0, st>>>(p.htab, p.xtab, p.lvalid);
+        k_toep_durbin<<<p.ndet, DT, 0, st>>>(h, p.cz_href, p.xtab, p.lvalid);
     }
     return cudaGetLastError();
 }

@@ -45,3 +45,39 @@ def test_single_gap_inverse(fknee, alpha):
                                      oracle.omega1(SEED, BAND, q, IT, n), oracle.omega2(SEED, BAND, q, IT, n))
         assert np.linalg.norm(x[sl] - ref) < 1e-5 * np.linalg.norm(ref), (L, its[q])
         assert 1 <= its[q] <= 8, (L, its[q])
+
+
+@pytest.mark.parametrize("length", [1024, 1030, 4096, 9000, 40000, 140000])
+def test_kernel_of_every_detector(length):
+    """Three detectors (one pair of a transform and one alone) of different
+    spectra at reference lengths of two to three transform passes: each
+    detector's own inverse serves its gap (the bound of the test above)."""
+    torch = pytest.importorskip("torch")
+    import paper_2201_03509_gb300 as tg
+    from gpu_workload import Workload
+    cfg = synth.scaled(synth.CONFIGS["tiny"], ndet=3, nscan=2, len_lo=length, len_hi=length, fsamp=78.8,
+                       fknee_lo=0.02, fknee_hi=2.0, alpha_lo=-2.0, alpha_hi=-1.0, sigma0_jitter=0.2)
+    wl = Workload(cfg)
+    L = min(500, length // 10)
+    f = np.zeros(wl.N, bool)
+    for q in range(wl.nq):
+        a = int(wl.off[q]) + length // 3
+        f[a:a + L] = True
+    flags = torch.from_numpy(tg.pack_flags(f).view(np.int32)).to(wl.dev)
+    gain = torch.ones(wl.nq, dtype=torch.float64, device=wl.dev)
+    x = torch.zeros(wl.N, dtype=torch.float32, device=wl.dev)
+    its = torch.zeros(wl.nq, dtype=torch.int32, device=wl.dev)
+    for levels in (tg.PREC_BLOCKS, tg.PREC_TWO_LEVEL):
+        wl.plan.set_preconditioner(levels)
+        wl.plan.sample_ncorr(wl.t_d, wl.t_s, gain, flags, wl.t_psd, tg.Rng(SEED, BAND, IT), tg.MODE_DRAW, x, its,
+                             cg_tol=1e-7)
+        wl.plan.status()
+        assert 1 <= int(its.min()) and int(its.max()) <= 8, (levels, its.tolist())
+    x = x.cpu().numpy().astype(np.float64)
+    for q in (0, 2, 4):
+        sl = wl.sl(q)
+        n = sl.stop - sl.start
+        ref, _ = oracle.sample_ncorr(wl.d32[sl].astype(np.float64), wl.s32[sl].astype(np.float64), 1.0,
+                                     (~f[sl]).astype(np.float64), *wl.band.psd[wl.det(q)], cfg.fsamp,
+                                     oracle.omega1(SEED, BAND, q, IT, n), oracle.omega2(SEED, BAND, q, IT, n))
+        assert np.linalg.norm(x[sl] - ref) < 1e-5 * np.linalg.norm(ref), q
