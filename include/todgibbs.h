@@ -179,7 +179,7 @@ tod_status tod_plan_status(tod_plan *p, int32_t *detscan_status);
 /* Launch schedule of the transform stages (gain, n_corr):
  * TOD_SCHED_PERSISTENT (default): every pass of a stage is one launch over
  * the tiles of all detscans (the n_corr draw: a fixed sequence of pass
- * launches, its CG iterations past the eighth in one cooperative launch);
+ * launches, its CG iterations past the third in one cooperative launch);
  * TOD_SCHED_PER_SCAN: the same kernels launched once per detscan (the
  * plain per-scan path, kept for comparison).  Results are identical: each
  * detscan's arithmetic does not depend on the others or on the launch. */
@@ -229,7 +229,7 @@ enum {
                                  k_cz_sums, k_cz_tables */
     TOD_KT_TOEP_DURBIN,       /* k_toep_durbin */
     TOD_KT_NC_FLAG_COUNT,     /* k_nc_flag_count */
-    TOD_KT_NC_FLAG_SCAN,      /* k_nc_flag_scan */
+    TOD_KT_NC_FLAG_SCAN,      /* none (the prefix of the chunk counts is part of k_nc_flag_write) */
     TOD_KT_NC_FLAG_WRITE,     /* k_nc_flag_write */
     TOD_KT_NC_INDEX,          /* k_nc_index */
     TOD_KT_NC_COARSE,         /* k_nc_coarse (the coarse correction of the preconditioner) */
@@ -241,12 +241,12 @@ enum {
     TOD_KT_NC_FILTER,         /* k_nc_filter of a CG iteration */
     TOD_KT_NC_GATHER,         /* k_nc_gather of a CG iteration */
     TOD_KT_NC_UPDATE,         /* k_nc_update */
-    TOD_KT_NC_LIST,           /* k_nc_list (the detscans a CG pass works on) */
+    TOD_KT_NC_LIST,           /* none (the list of iterating detscans is part of k_nc_cg_init, k_nc_update, k_nc_tail) */
     TOD_KT_NC_TAIL,           /* k_nc_tail (cooperative: the remaining CG iterations) */
     TOD_KT_NC_SCATTER_FINAL,  /* k_nc_scatter of the correction x = x0 + B^-1 E y */
     TOD_KT_NC_FILTER_FINAL,   /* k_nc_filter of the correction */
     TOD_KT_NC_GATHER_FINAL,   /* k_nc_gather of the correction */
-    TOD_KT_NC_FINISH,         /* k_nc_finish */
+    TOD_KT_NC_FINISH,         /* none (the iteration counts are part of k_nc_tail) */
     TOD_KT_BIN,               /* k_bin */
     TOD_KT_REDUCE,            /* k_reduce */
     TOD_KT_COMBINE,           /* k_combine */

@@ -860,7 +860,7 @@ tod_status tod_plan_create(tod_plan **out, const tod_band_desc *band)
         p->cgcap = std::max<int64_t>(p->N / 16, 2 * static_cast<int64_t>(maxlen));
         if ((e = dev_upload(*p, p->cgv, static_cast<float *>(nullptr), static_cast<size_t>(5 * p->cgcap))))
             return fail(e);
-        if ((e = dev_upload(*p, p->cg_count, static_cast<int32_t *>(nullptr), 2))) return fail(e);
+        if ((e = dev_upload(*p, p->cg_count, static_cast<int32_t *>(nullptr), 3))) return fail(e);
         if ((e = dev_upload(*p, p->nclist, static_cast<int32_t *>(nullptr), 3 * static_cast<size_t>(p->nq) + 3)))
             return fail(e);
         if ((e = dev_upload(*p, p->chi2_dpsd, static_cast<double *>(nullptr), 3 * static_cast<size_t>(p->nq))))

@@ -1067,7 +1067,8 @@ __device__ int3 cta_exscan3(int3 v, int3 *s_w, int3 &total)
 }
 
 // Flagged-sample prefix over the range's flag words, in chunks of words per
-// CTA: count (chunk totals), scan (one thread), write (per-word prefix).
+// CTA: count (chunk totals), then write (the per-word prefix from the totals
+// of the chunks before).
 struct FlagChunk {
     int64_t w_lo, nw, c0, c1, t0, per, obase, oend;
 };
@@ -1105,16 +1106,26 @@ __device__ void nc_flag_count(const NcorrTx &a, NcShared &S)
 __device__ void nc_flag_write(const NcorrTx &a, NcShared &S)
 {
     const FlagChunk f = flag_chunk(a);
+    // the chunks before this one: at most a grid's worth of counts, summed by
+    // the CTA (a serial scan of them by one thread took 20-50 us)
+    long long before = 0;
+    for (int c = threadIdx.x; c < static_cast<int>(blockIdx.x); c += TX_T) before += __ldg(a.chunk + c);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    __shared__ long long s_before[TX_T / 32];
+    if ((threadIdx.x & 31) == 0) s_before[threadIdx.x >> 5] = before;
     int mine = 0;
     for (int64_t i = f.t0; i < min(f.c1, f.t0 + f.per); ++i) mine += __popc(flag_word(a, f, i));
     int3 tot3;
-    const int3 ex = cta_exscan3(make_int3(mine, 0, 0), S.scan, tot3);
-    int64_t run = a.chunk[blockIdx.x] + ex.x;
+    const int3 ex = cta_exscan3(make_int3(mine, 0, 0), S.scan, tot3);       // barriers: s_before is complete
+    int64_t run = ex.x;
+#pragma unroll
+    for (int w = 0; w < TX_T / 32; ++w) run += s_before[w];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) a.wpre[f.nw] = run + tot3.x;
     for (int64_t i = f.t0; i < min(f.c1, f.t0 + f.per); ++i) {
         a.wpre[i] = run;
         run += __popc(flag_word(a, f, i));
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) a.wpre[f.nw] = a.chunk[gridDim.x];
 }
 
 // Phase 2 (per detscan): flagged count and rank offset, CG mode, and the
@@ -2044,7 +2055,7 @@ __device__ __forceinline__ void nc_items(const NcorrTx &a, TxCtx &X, bool rows, 
 
 // The list of the launch range's detscans in CG mode `want` (ascending),
 // with exclusive running counts of their column and row items.  One CTA
-// (any multiple of 32 threads up to 1024) builds it.
+// builds it (modes read past L1: other CTAs of the launch have written them).
 __device__ void nc_build_list(const NcorrTx &a, int want)
 {
     __shared__ int s_w[32][3];
@@ -2055,7 +2066,7 @@ __device__ void nc_build_list(const NcorrTx &a, int want)
     int32_t *lq = nl_q(a), *lc = nl_col(a), *lr = nl_row(a);
     for (int c0 = a.q0; c0 < a.q1; c0 += blockDim.x) {
         const int q = c0 + threadIdx.x;
-        const bool in = q < a.q1 && a.cgs[q].mode == want;
+        const bool in = q < a.q1 && __ldcg(&a.cgs[q].mode) == want;
         int v[3] = {in ? 1 : 0, in ? a.col_off[q + 1] - a.col_off[q] : 0, in ? a.row_off[q + 1] - a.row_off[q] : 0};
         int x[3];
 #pragma unroll
@@ -2092,10 +2103,22 @@ __device__ void nc_build_list(const NcorrTx &a, int want)
         lr[s_base[0]] = s_base[2];
     }
 }
-__global__ void __launch_bounds__(1024) k_nc_list(NcorrTx a, int want, int par)
+// Called by every CTA at the end of a launch that set the detscans' modes: the
+// last one to arrive builds the list of those still iterating (a launch of
+// its own for the list cost 3 us an iteration; count[2] counts arrivals).
+__device__ void nc_list_by_last(const NcorrTx &a)
 {
-    if (par >= 0 && *reinterpret_cast<volatile const int32_t *>(a.count + par) == 0) return;
-    nc_build_list(a, want);
+    __shared__ int s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(a.count + 2, 1) == static_cast<int>(gridDim.x) - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    if (threadIdx.x == 0) a.count[2] = 0;
+    nc_build_list(a, CG_ACTIVE);
 }
 
 // The listed detscans' column (or row) items, a contiguous share per CTA:
@@ -2130,13 +2153,6 @@ __global__ void __launch_bounds__(TX_T) k_nc_flag_count(NcorrTx a)
     __shared__ NcShared S;
     nc_flag_count(a, S);
 }
-__global__ void k_nc_flag_scan(NcorrTx a, int G)
-{
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    int64_t acc = 0;
-    for (int c = 0; c < G; ++c) { const int64_t v = a.chunk[c]; a.chunk[c] = acc; acc += v; }
-    a.chunk[G] = acc;
-}
 __global__ void __launch_bounds__(TX_T) k_nc_flag_write(NcorrTx a)
 {
     __shared__ NcShared S;
@@ -2145,7 +2161,7 @@ __global__ void __launch_bounds__(TX_T) k_nc_flag_write(NcorrTx a)
 __global__ void __launch_bounds__(TX_T) k_nc_index(NcorrTx a)
 {
     __shared__ NcShared S;
-    if (blockIdx.x == 0 && threadIdx.x == 0) { a.count[0] = 0; a.count[1] = 0; }
+    if (blockIdx.x == 0 && threadIdx.x == 0) { a.count[0] = 0; a.count[1] = 0; a.count[2] = 0; }
     for (int q = a.q0 + blockIdx.x; q < a.q1; q += gridDim.x) {
         nc_detscan_index(a, S, q);
         __syncthreads();
@@ -2186,6 +2202,7 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_cg_init(NcorrTx a)
         __syncthreads();
         nc_cg_init(a, S, q, reinterpret_cast<float *>(tx_smem));
     }
+    nc_list_by_last(a);
 }
 // One CG iteration (parity par: count[par] active detscans going in, the
 // update counts into count[par ^ 1]), or with FINAL the correction B^{-1} E y.
@@ -2237,21 +2254,21 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_update(NcorrTx a, int par)
     __shared__ NcShared S;
     if (*reinterpret_cast<volatile const int32_t *>(a.count + par) == 0) return;
     nc_update_listed(a, S, reinterpret_cast<float *>(tx_smem), a.count + (par ^ 1));
+    nc_list_by_last(a);
 }
-// The iterations left after the launched ones, in one cooperative launch:
-// the passes over the listed detscans with grid barriers between them, the
-// list rebuilt by CTA 0 after each update.
-__global__ void __launch_bounds__(TX_T, 2) k_nc_tail(NcorrTx a, int par)
+// The iterations left after the launched ones, in one cooperative launch at
+// the passes' own occupancy: the passes over the listed detscans with grid
+// barriers between them, the list rebuilt by CTA 0 after each update.  Then
+// the list of the detscans that ran the CG (for the correction), the
+// iteration counts, and the status of detscans left at x0 for want of CG room.
+__global__ void __launch_bounds__(TX_T, 3) k_nc_tail(NcorrTx a, int par)
 {
     extern __shared__ __align__(16) float2 tx_smem[];
     __shared__ NcShared S;
     cgrp::grid_group grid = cgrp::this_grid();
     const CgVec V = cg_vecs(a);
     int cur = -1;
-    for (;;) {
-        if (*reinterpret_cast<volatile const int32_t *>(a.count + par) == 0) break;
-        if (blockIdx.x == 0) nc_build_list(a, CG_ACTIVE);
-        grid.sync();
+    while (*reinterpret_cast<volatile const int32_t *>(a.count + par) != 0) {
         if (blockIdx.x == 0 && threadIdx.x == 0) a.count[par ^ 1] = 0;
         nc_list_items(a, S.X, false, cur, [&] { nc_scatter_cols(a, S.X, tx_smem, tx_smem + TX_TILE, V.p); });
         grid.sync();
@@ -2262,16 +2279,15 @@ __global__ void __launch_bounds__(TX_T, 2) k_nc_tail(NcorrTx a, int par)
         nc_update_listed(a, S, reinterpret_cast<float *>(tx_smem), a.count + (par ^ 1));
         grid.sync();
         par ^= 1;
+        if (*reinterpret_cast<volatile const int32_t *>(a.count + par) == 0) break;
+        if (blockIdx.x == 0) nc_build_list(a, CG_ACTIVE);
+        grid.sync();
     }
-}
-// Iteration counts; detscans left at x0 for want of CG room are reported.
-__global__ void k_nc_finish(NcorrTx a)
-{
-    const int q = a.q0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= a.q1) return;
-    const CgState cs = a.cgs[q];
-    if (a.iters) a.iters[q] = cs.it;
-    if (cs.mode == CG_OVER) set_status(a.status, q, TOD_ERR_NOT_CONVERGED);
+    if (blockIdx.x == 0) nc_build_list(a, CG_DONE);
+    for (int q = a.q0 + blockIdx.x * TX_T + threadIdx.x; q < a.q1; q += gridDim.x * TX_T) {
+        if (a.iters) a.iters[q] = __ldcg(&a.cgs[q].it);
+        if (__ldcg(&a.cgs[q].mode) == CG_OVER) set_status(a.status, q, TOD_ERR_NOT_CONVERGED);
+    }
 }
 
 // ===========================================================================
@@ -2280,7 +2296,13 @@ __global__ void k_nc_finish(NcorrTx a)
 static size_t tx_smem_bytes(bool fp64) { return (fp64 ? sizeof(double2) : sizeof(float2)) * 2 * TX_TILE; }
 constexpr size_t kGbBytes = (5 * TX_GBCAP + CZ_FLOATS) * sizeof(float);   // preconditioner staging
 static_assert(kGbBytes <= sizeof(float2) * 2 * TX_TILE, "the preconditioner staging fits the tile buffers");
-constexpr int NC_LAUNCHED_ITERS = 8;                                // CG iterations as separate launches
+// CG iterations as separate launches.  The two-level preconditioner takes 2.1
+// on average and 4 to 5 at most on the 30 to 70 GHz bands; the rest runs in
+// the cooperative tail, whose grid barriers cost what a launch does.  Launches
+// past the last iteration return at once but cost 2 us each (four an
+// iteration), and the tail costs as much as they do: three launched
+// iterations leave it the few stragglers.
+constexpr int NC_LAUNCHED_ITERS = 3;
 
 template <class K>
 static cudaError_t smem_attr(K k, size_t bytes) {
@@ -2444,15 +2466,11 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
     const int ncol = p.h_col_off[q1] - p.h_col_off[q0], nrow = p.h_row_off[q1] - p.h_row_off[q0];
     const int gc = std::min(grid_for(p, ncol), grid), gr = std::min(grid_for(p, nrow), grid);
     const int gq = std::min(nq, std::max(1, grid));
-    // flag index (the chunked scan uses the same grid for count and write)
+    // flag index (count and write use the same grid)
     const int gf = std::max(1, std::min(p.pass_grid, grid));
     {
         KTIME(TOD_KT_NC_FLAG_COUNT);
         k_nc_flag_count<<<gf, TX_T, 0, st>>>(a);
-    }
-    {
-        KTIME(TOD_KT_NC_FLAG_SCAN);
-        k_nc_flag_scan<<<1, 1, 0, st>>>(a, gf);
     }
     {
         KTIME(TOD_KT_NC_FLAG_WRITE);
@@ -2485,10 +2503,6 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
         k_nc_cg_init<<<gq, TX_T, sgb, st>>>(a);
     }
     int par = 0;
-    {
-        KTIME(TOD_KT_NC_LIST);
-        k_nc_list<<<1, 1024, 0, st>>>(a, CG_ACTIVE, par);
-    }
     for (int it = 0; it < NC_LAUNCHED_ITERS; ++it, par ^= 1) {
         {
             KTIME(TOD_KT_NC_SCATTER);
@@ -2506,10 +2520,6 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
             KTIME(TOD_KT_NC_UPDATE);
             k_nc_update<<<gq, TX_T, sgb, st>>>(a, par);
         }
-        {
-            KTIME(TOD_KT_NC_LIST);
-            k_nc_list<<<1, 1024, 0, st>>>(a, CG_ACTIVE, par ^ 1);
-        }
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -2521,10 +2531,6 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
                                         dim3(std::max(1, std::min(grid, p.coop_grid))), dim3(TX_T), args, sgb, st);
     }
     if (e != cudaSuccess) return e;
-    {
-        KTIME(TOD_KT_NC_LIST);
-        k_nc_list<<<1, 1024, 0, st>>>(a, CG_DONE, -1);
-    }
     // x = x0 + B^{-1} E y for every detscan that ran the CG
     {
         KTIME(TOD_KT_NC_SCATTER_FINAL);
@@ -2537,10 +2543,6 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
     {
         KTIME(TOD_KT_NC_GATHER_FINAL);
         k_nc_gather<true><<<gc, TX_T, s32, st>>>(a, 0);
-    }
-    {
-        KTIME(TOD_KT_NC_FINISH);
-        k_nc_finish<<<(nq + 255) / 256, 256, 0, st>>>(a);
     }
     return cudaGetLastError();
 }

@@ -210,11 +210,11 @@ class GibbsTODStep:
         self._mark_d_done(stream)
 
     # decode x2, project, gain (scalars, three passes, draw), n_corr (flag
-    # index 4, coarse correction, right-hand side 3, CG start and its list,
-    # 8 launched CG iterations x (3 passes, update, list), cooperative tail,
-    # list, correction 3, finish), bin + reduce, solve; plus the
-    # preconditioner preparation (Plan.toeplitz_prep_launches)
-    LAUNCHES_PER_STEP = 2 + 1 + 5 + (4 + 1 + 3 + 2 + 8 * 5 + 1 + 1 + 3 + 1) + 2 + 1
+    # index 3, coarse correction, right-hand side 3, CG start, 3 launched CG
+    # iterations x (3 passes, update), cooperative tail, correction 3), bin +
+    # reduce, solve; plus the preconditioner preparation
+    # (Plan.toeplitz_prep_launches)
+    LAUNCHES_PER_STEP = 2 + 1 + 5 + (3 + 1 + 3 + 1 + 3 * 4 + 1 + 3) + 2 + 1
     DATA_LAUNCHES = 2       # with data_streams: decode of the TOD and of the flags
 
     @property
