@@ -250,23 +250,46 @@ int64_t fft_length_impl(int64_t n)
     return best;
 }
 
-// Stockham radices of a sub-transform of length L: repeatedly the largest
-// register DFT up to rmax (16, 10, 9, 8, 6, 5, 4, 3, 2) that divides what is
-// left (empty for L = 1).  A thread of the in-place passes holds the inputs
-// of ceil(16/R) butterflies: at most 20 values with these radices.
+// Stockham radices of a sub-transform of length L, from 10, 9, 8, 6, 5, 4, 3, 2
+// up to rmax (and TX_RMAX): the product with the least cost per value, a pass
+// costing its shared-memory round trip, twiddle and indexing (about 9
+// instructions a value pair) plus its butterfly; smaller radices first
+// (empty for L = 1, or when L has a prime factor above rmax).
 std::vector<int8_t> radix_plan(int L, int rmax)
 {
-    static const int kRadix[] = {16, 10, 9, 8, 6, 5, 4, 3, 2};
-    std::vector<int8_t> r;
-    while (L > 1) {
-        int pick = 0;
-        for (int R : kRadix)
-            if (R <= rmax && L % R == 0) { pick = R; break; }
-        if (!pick) { r.clear(); return r; }
-        r.push_back(static_cast<int8_t>(pick));
-        L /= pick;
+    static const int kRadix[] = {10, 9, 8, 6, 5, 4, 3, 2};
+    static const double kCost[] = {6.0, 5.6, 3.6, 3.8, 4.0, 2.0, 2.7, 1.0};
+    static const double kPass = 9.0;
+    // plans depend on (L, rmax) alone: remembered across lengths and calls
+    static std::mutex mu;
+    static std::map<std::pair<int, int>, std::vector<int8_t>> seen;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = seen.find(std::make_pair(L, rmax));
+        if (it != seen.end()) return it->second;
     }
-    std::reverse(r.begin(), r.end());
+    std::map<int, std::pair<double, int>> best;           // length -> (cost, first radix)
+    const std::function<double(int)> cost = [&](int l) -> double {
+        if (l == 1) return 0.0;
+        const auto it = best.find(l);
+        if (it != best.end()) return it->second.first;
+        double c = 1e30;
+        int pick = 0;
+        for (int i = 0; i < 8; ++i) {
+            const int R = kRadix[i];
+            if (R > std::min(rmax, TX_RMAX) || l % R) continue;
+            const double t = kPass + kCost[i] + cost(l / R);
+            if (t < c) { c = t; pick = R; }
+        }
+        best[l] = std::make_pair(c, pick);
+        return c;
+    };
+    std::vector<int8_t> r;
+    if (L > 1 && cost(L) < 1e30)
+        for (int l = L; l > 1; l /= best[l].second) r.push_back(static_cast<int8_t>(best[l].second));
+    std::sort(r.begin(), r.end());
+    std::lock_guard<std::mutex> lk(mu);
+    seen[std::make_pair(L, rmax)] = r;
     return r;
 }
 
@@ -283,64 +306,64 @@ void fill_stages(DctStage *st, const std::vector<int8_t> &r, int L)
 }
 
 // Column pairs per column tile: the largest power of two (at most 64, so
-// that the 2 TP columns divide the CTA's threads) with 2 TP m1 <= TX_TILE,
-// capped by tile_pairs when given.
+// that it divides the CTA's threads) with TP m1 <= TX_PAIRS, capped by
+// tile_pairs when given.
 int tile_width(int P2, int m1, int tile_pairs)
 {
-    int cap = std::min(64, TX_TILE / (2 * m1));
+    int cap = std::min(64, TX_PAIRS / m1);
     if (tile_pairs > 0) cap = std::min(cap, tile_pairs);
     int tp = 1;
     while (2 * tp <= cap && tp < P2) tp *= 2;
     return tp;
 }
 
-// Shared-memory bank conflicts of the row FFTs of a row tile with nslot
-// rows at stride m2p: butterfly w of a Stockham pass (radix R after Ns
-// points) works on row w mod nslot, index j = w / nslot, reading elements
+// Shared-memory bank conflicts of the row FFTs of a row tile with TR row
+// pairs at stride m2p: butterfly w of a Stockham pass (radix R after Ns
+// points) works on pair w mod TR, index j = w / TR, reading elements
 // j + r L/R and writing (j / Ns) Ns R + j mod Ns + r Ns.  Returned: the mean
-// number of extra 8-byte wavefronts per half-warp access, over the first
-// eight warps' first two reads and writes of every pass.
-double row_bank_cost(int m2, int m2p, int nslot, const std::vector<int8_t> &radices)
+// number of extra wavefronts per quarter-warp access (eight threads' 16-byte
+// elements fill the 32 banks once), over the first eight warps' first two
+// reads and writes of every pass.
+double row_bank_cost(int m2, int m2p, int TR, const std::vector<int8_t> &radices)
 {
     int Ns = 1;
     double extra = 0.0;
     int count = 0;
     for (int R : radices) {
-        const int LR = m2 / R, total = nslot * LR;
-        for (int w0 = 0; w0 < std::min(total, TX_T); w0 += 32)
-            for (int half = 0; half < 32; half += 16)
-                for (int rd = 0; rd < 2; ++rd)
-                    for (int r = 0; r < 2; ++r) {
-                        int hits[16] = {0};
-                        int used = 0, worst = 0;
-                        for (int i = 0; i < 16; ++i) {
-                            const int w = w0 + half + i;
-                            if (w >= total) break;
-                            const int j = w / nslot, vec = w - j * nslot;
-                            int e;
-                            if (rd) e = j + r * LR;
-                            else { const int jq = j / Ns, k = j - jq * Ns; e = jq * Ns * R + k + r * Ns; }
-                            const int b = (vec * m2p + e) & 15;
-                            worst = std::max(worst, ++hits[b]);
-                            ++used;
-                        }
-                        if (used) { extra += worst - 1; ++count; }
+        const int LR = m2 / R, total = TR * LR;
+        for (int w0 = 0; w0 < std::min(total, TX_T); w0 += 8)
+            for (int rd = 0; rd < 2; ++rd)
+                for (int r = 0; r < 2; ++r) {
+                    int hits[8] = {0};
+                    int used = 0, worst = 0;
+                    for (int i = 0; i < 8; ++i) {
+                        const int w = w0 + i;
+                        if (w >= total) break;
+                        const int j = w / TR, vec = w - j * TR;
+                        int e;
+                        if (rd) e = j + r * LR;
+                        else { const int jq = j / Ns, k = j - jq * Ns; e = jq * Ns * R + k + r * Ns; }
+                        const int b = (vec * m2p + e) & 7;
+                        worst = std::max(worst, ++hits[b]);
+                        ++used;
                     }
+                    if (used) { extra += worst - 1; ++count; }
+                }
         Ns *= R;
     }
     return count ? extra / count : 0.0;
 }
 
 // Row tile shape for row FFTs of length m2: TR row pairs, a power of two
-// (so a warp's butterflies spread evenly over the rows), and the row
-// stride m2p in [m2, m2 + 16] with the fewest bank conflicts; more row
-// pairs win unless they cost more than a quarter wavefront per access.
+// (so a warp's butterflies spread evenly over them), and the pair stride m2p
+// in [m2, m2 + 8] with the fewest bank conflicts; more row pairs win unless
+// they cost more than a quarter wavefront per access.
 void row_shape(int m2, int P1, const std::vector<int8_t> &radices, int &TR, int &m2p)
 {
-    // the shape depends on (m2, P1 up to 64) alone: remembered across lengths
+    // the shape depends on (m2, P1 up to 65, radices): remembered across lengths
     static std::mutex mu;
-    static std::map<std::pair<int, int>, std::pair<int, int>> seen;
-    const std::pair<int, int> key(m2, std::min(P1, 65));
+    static std::map<std::pair<std::pair<int, int>, std::vector<int8_t>>, std::pair<int, int>> seen;
+    const auto key = std::make_pair(std::make_pair(m2, std::min(P1, 65)), radices);
     {
         std::lock_guard<std::mutex> lk(mu);
         const auto it = seen.find(key);
@@ -348,11 +371,11 @@ void row_shape(int m2, int P1, const std::vector<int8_t> &radices, int &TR, int 
     }
     double best = 1e30;
     TR = 1;
-    m2p = m2 | 1;
-    for (int tr = 1; tr <= 64 && 2 * tr * m2 <= TX_TILE; tr *= 2) {
+    m2p = m2;
+    for (int tr = 1; tr <= 64 && tr * m2 <= TX_PAIRS; tr *= 2) {
         if (tr > 1 && tr / 2 >= P1) break;          // more row pairs than the transform has
-        for (int p = m2; p <= m2 + 16 && 2 * tr * p <= TX_TILE; ++p) {
-            const double score = row_bank_cost(m2, p, 2 * tr, radices) - 0.25 * std::log2(static_cast<double>(tr));
+        for (int p = m2; p <= m2 + 8 && tr * p <= TX_PAIRS; ++p) {
+            const double score = row_bank_cost(m2, p, tr, radices) - 0.25 * std::log2(static_cast<double>(tr));
             if (score < best - 1e-12) { best = score; TR = tr; m2p = p; }
         }
     }
@@ -361,8 +384,8 @@ void row_shape(int m2, int P1, const std::vector<int8_t> &radices, int &TR, int 
 }
 
 // Split m = n/2 = m1 x m2 for the multi-pass transform.  A column tile holds
-// m1 rows of 2 TP columns and a row tile 2 TR rows of m2 (made odd), each at
-// most TX_TILE values.  Wide column tiles (TP up to 16: sample runs of 64
+// m1 rows of TP column pairs and a row tile TR row pairs of m2, each at
+// most TX_PAIRS pairs of values.  Wide column tiles (TP up to 16: sample runs of 64
 // floats) and several row pairs (TR up to 4: fewer Philox blocks per mode)
 // score highest, then m2 / m1 nearest 2.5.  tile_pairs > 0 caps TP.
 bool choose_tx_split(int n, int rmax, int tile_pairs, TxLen &out)
@@ -378,7 +401,7 @@ bool choose_tx_split(int n, int rmax, int tile_pairs, TxLen &out)
         if (r1.size() > TX_MAXR || r2.size() > TX_MAXR) continue;
         const int m2p = m2 | 1;
         if (2 * m1 > TX_TILE || 2 * m2p > TX_TILE) continue;
-        const int P1 = m1 / 2 + 1, P2 = (m2 + 1) / 2;
+        const int P1 = (m1 + 1) / 2, P2 = (m2 + 1) / 2;
         const int TP = tile_width(P2, m1, tile_pairs);
         const int TR = std::min(P1, TX_TILE / (2 * m2p));
         const double score = std::min(TP, 16) / 16.0 + std::min(TR, 4) / 4.0 -
@@ -390,7 +413,7 @@ bool choose_tx_split(int n, int rmax, int tile_pairs, TxLen &out)
     const auto r1 = radix_plan(m1, rmax), r2 = radix_plan(m2, rmax);
     std::memset(&out, 0, sizeof(out));
     out.n = n; out.m = m; out.m1 = m1; out.m2 = m2;
-    out.P1 = m1 / 2 + 1;
+    out.P1 = (m1 + 1) / 2;
     out.P2 = (m2 + 1) / 2;
     out.TP = tile_width(out.P2, m1, tile_pairs);
     row_shape(m2, out.P1, r2, out.TR, out.m2p);
@@ -398,16 +421,11 @@ bool choose_tx_split(int n, int rmax, int tile_pairs, TxLen &out)
     out.nr2 = static_cast<int32_t>(r2.size());
     fill_stages(out.s1, r1, m1);
     fill_stages(out.s2, r2, m2);
-    out.f_m2 = make_fastdiv(static_cast<uint32_t>(m2));
-    out.f_W = make_fastdiv(static_cast<uint32_t>(2 * out.TP));
     out.lgW = 0;
-    while ((2 << out.lgW) <= 2 * out.TP) ++out.lgW;
+    while ((2 << out.lgW) <= out.TP) ++out.lgW;
     out.lgS = 0;
-    while ((2 << out.lgS) <= 2 * out.TR) ++out.lgS;
-    out.f_2TR = make_fastdiv(static_cast<uint32_t>(2 * out.TR));
-    out.sq_fwd = std::sqrt(2.0 / n);
+    while ((2 << out.lgS) <= out.TR) ++out.lgS;
     out.s0_fwd = 1.0 / std::sqrt(static_cast<double>(n));
-    out.sq_inv = std::sqrt(0.5 * n) / m;
     out.s0_inv = std::sqrt(static_cast<double>(n)) / m;
     return true;
 }
@@ -794,25 +812,38 @@ tod_status tod_plan_create(tod_plan **out, const tod_band_desc *band)
             if (!choose_tx_split(n, rmax, tile_pairs, L)) { free_plan(p); return TOD_ERR_ARG; }
             tl.push_back(L);
         }
-        // twiddle block per length, FP64-generated: W_m1^i (m1), W_m2^i (m2),
-        // W_4n^{k1} (m1), W_4n^{m1 k2} (m2), W_4n^{5 k1} (m1),
-        // W_4n^{5 m1 k2} (m2), W_m^{64 i} (m/64 + 1), W_m^i (64)
+        // twiddle block per length, FP64-generated: W_m1^i (m1) and W_m2^i
+        // (m2), each part in both lanes of a pair; then plain complex values
+        // hq W_4n^{k1} (m1), W_4n^{m1 k2} (m2), hq W_4n^{5 k1} (m1),
+        // W_4n^{5 m1 k2} (m2), W_m^{64 i} (m/64 + 1), W_m^i (64), with
+        // hq = 1/(2 sqrt(m)) the scale of the real split
         std::vector<double2> tw;
-        const auto push_w = [&](int64_t Lp, int64_t i) {
+        const auto unit = [&](int64_t Lp, int64_t i) {
             const double ang = -2.0 * kPi * static_cast<double>(i % Lp) / static_cast<double>(Lp);
-            tw.push_back(make_double2(std::cos(ang), std::sin(ang)));
+            return make_double2(std::cos(ang), std::sin(ang));
+        };
+        const auto push_w = [&](int64_t Lp, int64_t i, double sc) {
+            const double2 w = unit(Lp, i);
+            tw.push_back(make_double2(sc * w.x, sc * w.y));
+        };
+        const auto push_pair = [&](int64_t Lp, int64_t i) {
+            const double2 w = unit(Lp, i);
+            tw.push_back(make_double2(w.x, w.x));
+            tw.push_back(make_double2(w.y, w.y));
         };
         for (auto &L : tl) {
+            if (tw.size() & 1) tw.push_back(make_double2(0.0, 0.0));       // pairs are read as 16-byte words
             L.twb = static_cast<int64_t>(tw.size());
             const int64_t n4 = 4 * static_cast<int64_t>(L.n);
-            for (int i = 0; i < L.m1; ++i) push_w(L.m1, i);
-            for (int i = 0; i < L.m2; ++i) push_w(L.m2, i);
-            for (int i = 0; i < L.m1; ++i) push_w(n4, i);
-            for (int i = 0; i < L.m2; ++i) push_w(n4, static_cast<int64_t>(L.m1) * i);
-            for (int i = 0; i < L.m1; ++i) push_w(n4, 5 * static_cast<int64_t>(i));
-            for (int i = 0; i < L.m2; ++i) push_w(n4, 5 * static_cast<int64_t>(L.m1) * i);
-            for (int i = 0; i <= L.m / 64; ++i) push_w(L.m, 64 * static_cast<int64_t>(i));
-            for (int i = 0; i < 64; ++i) push_w(L.m, i);
+            const double hq = 0.5 / std::sqrt(static_cast<double>(L.m));
+            for (int i = 0; i < L.m1; ++i) push_pair(L.m1, i);
+            for (int i = 0; i < L.m2; ++i) push_pair(L.m2, i);
+            for (int i = 0; i < L.m1; ++i) push_w(n4, i, hq);
+            for (int i = 0; i < L.m2; ++i) push_w(n4, static_cast<int64_t>(L.m1) * i, 1.0);
+            for (int i = 0; i < L.m1; ++i) push_w(n4, 5 * static_cast<int64_t>(i), hq);
+            for (int i = 0; i < L.m2; ++i) push_w(n4, 5 * static_cast<int64_t>(L.m1) * i, 1.0);
+            for (int i = 0; i <= L.m / 64; ++i) push_w(L.m, 64 * static_cast<int64_t>(i), 1.0);
+            for (int i = 0; i < 64; ++i) push_w(L.m, i, 1.0);
         }
         std::vector<float2> tw32(tw.size());
         for (size_t i = 0; i < tw.size(); ++i)

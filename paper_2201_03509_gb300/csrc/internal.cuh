@@ -49,13 +49,15 @@ struct DctStage {
 // ---------------------------------------------------------------------------
 // Multi-pass batched DCT-II (k_tx.cu).  A length-n transform is an m = n/2
 // complex FFT split m = m1 x m2: a column pass (FFTs of length m1 over
-// tiles of column pairs {c, m2-1-c}, four-step twiddle, written row-major
-// to an intermediate in memory), a row pass (FFTs of length m2 over tiles of
+// tiles of column pairs {c, m2-1-c}, four-step twiddle, written to an
+// intermediate in memory), a row pass (FFTs of length m2 over tiles of
 // row pairs {k1, m1-k1}, where the real split and any per-mode filter run,
 // then the inverse row FFTs), and an inverse column pass.
 // ---------------------------------------------------------------------------
 constexpr int TX_T = 256;             // threads per CTA of the pass kernels
 constexpr int TX_TILE = 4096;         // complex values per tile buffer (two buffers per CTA)
+constexpr int TX_PAIRS = TX_TILE / 2;  // as pairs of complex values (fft_reg.cuh)
+constexpr int TX_RMAX = 10;           // largest Stockham radix of the pair butterflies
 constexpr int TX_MAXR = 20;           // radix stages per sub-transform
 constexpr int TX_GBMAX = 256;         // preconditioner gap blocks per detscan
 constexpr int TX_GBCAP = 2048;        // padded preconditioner elements staged per round
@@ -69,14 +71,12 @@ constexpr int TX_CBMAX = 64;                      // most blocks of a detscan wi
 
 struct alignas(16) TxLen {
     int32_t n, m, m1, m2, m2p;        // m2p: row stride of a row tile (>= m2, chosen against bank conflicts)
-    int32_t P1, P2;                   // row pairs m1/2 + 1, column pairs (m2 + 1)/2
+    int32_t P1, P2;                   // row pairs (m1 + 1)/2, column pairs (m2 + 1)/2
     int32_t TP, TR;                   // column pairs per column tile, row pairs per row tile
     int32_t nr1, nr2;                 // radix stages of the column and row FFTs
-    int16_t lgW, lgS;                 // log2 of the column tile's 2 TP columns and the row tile's 2 TR rows
+    int16_t lgW, lgS;                 // log2 of TP and TR
     int64_t twb;                      // offset of this length's twiddle block
-    FastDiv f_m2, f_W, f_2TR;         // divisions by m2, 2 TP, 2 TR
-    int32_t pad1;
-    double sq_fwd, s0_fwd, sq_inv, s0_inv;   // real-split scales
+    double s0_fwd, s0_inv;            // real-split scales of slot 0
     DctStage s1[TX_MAXR], s2[TX_MAXR];
 };
 

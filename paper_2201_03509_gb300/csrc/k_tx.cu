@@ -7,7 +7,7 @@
 // x_{2n-1-2i} (i >= m) (Makhoul 1980), plus a real split.  The FFT is
 // four-step, m = m1 x m2, with j = j1 m2 + j2 and k = k1 + m1 k2:
 //   column pass: for a tile of column pairs {c, m2-1-c}: FFTs of length m1
-//     along j1, times W_m^{c k1}, written row-major to the intermediate Y;
+//     along j1, times W_m^{c k1}, written to the intermediate Y;
 //     z_j and z_{m-1-j} together are the four samples x_{4j..4j+3}, so the
 //     tile reads and writes whole runs of samples;
 //   row pass: for a tile of row pairs {k1, m1-k1}: FFTs of length m2 along
@@ -15,8 +15,11 @@
 //     coefficients (X_k, X_{n-k}) (slot 0: (X_0, X_m)), a per-mode filter,
 //     the inverse split and inverse FFTs, written back to Y;
 //   inverse column pass: times W_m^{-c k1}, inverse FFTs, samples out.
-// Every tile is independent: a CTA holds one tile in shared memory, passes
-// are separate grid-wide phases, and the intermediate goes through L2/HBM.
+// The two members of a pair are the two lanes of every value the passes
+// compute with (fft_reg.cuh): one packed FP32 instruction, one 16-byte
+// shared-memory access and one twiddle for both.  Every tile is independent:
+// a CTA holds one tile in shared memory, passes are separate grid-wide
+// phases, and the intermediate goes through L2/HBM.
 #include <cooperative_groups.h>
 #include "fft_reg.cuh"
 
@@ -99,15 +102,6 @@ __global__ void k_det_scalars(const double *__restrict__ psd, const double *__re
     if (q < q1) det_scalars_q(psd, gain, off, ndet, fsamp, q, qsc);
 }
 
-// This CTA's contiguous share [i0, i1) of nitems work items: consecutive
-// items of a CTA are mostly tiles of one detscan (same length: the plan
-// copy and the twiddles stay hot).
-__device__ __forceinline__ void cta_share(int nitems, int &i0, int &i1) {
-    const int per = (nitems + gridDim.x - 1) / gridDim.x;
-    i0 = min(nitems, static_cast<int>(blockIdx.x) * per);
-    i1 = min(nitems, i0 + per);
-}
-
 // The SFU's approximate base-2 logarithm and exponential and reciprocal
 // (PTX lg2/ex2/rcp.approx: absolute error about 2^-22 in the logarithm,
 // relative about 2^-22 in the others).  Used for the per-mode noise weights,
@@ -134,45 +128,37 @@ __device__ __forceinline__ float tx_fpow(int k, float fscale, float alpha) {
     return sfu_ex2(alpha * sfu_lg2(static_cast<float>(k) * fscale));
 }
 
-// twiddle block of a length: W_m1^i, W_m2^i, W_4n^{k1}, W_4n^{m1 k2},
-// W_4n^{5 k1}, W_4n^{5 m1 k2}, W_m^{64 i}, W_m^i (i < 64)
+// twiddle block of a length: W_m1^i and W_m2^i (both lanes of a pair), then
+// plain complex values: hq W_4n^{k1}, W_4n^{m1 k2}, hq W_4n^{5 k1},
+// W_4n^{5 m1 k2} (hq = 1/(2 sqrt(m)): the real split's scale, the same both
+// ways), W_m^{64 i}, W_m^i (i < 64)
+template <class V> struct PairOf;
+template <> struct PairOf<CF2> { typedef float2 Z; };
+template <> struct PairOf<CD2> { typedef double2 Z; };
+__device__ __forceinline__ float2 zmul(float2 a, float2 b) {
+    return make_float2(fmaf(-a.y, b.y, a.x * b.x), fmaf(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ double2 zmul(double2 a, double2 b) {
+    return make_double2(fma(-a.y, b.y, a.x * b.x), fma(a.x, b.y, a.y * b.x));
+}
+template <class V, class Z> __device__ __forceinline__ V vtwo(Z a, Z b) {
+    return vmake<V>(pset(a.x, b.x), pset(a.y, b.y));
+}
 template <class V> struct TwB {
-    const V *tw1, *tw2, *sa1, *sb1, *sa5, *sb5, *t4hi, *t4lo;
-    __device__ __forceinline__ TwB(const V *base, const TxLen &L) {
-        tw1 = base;
+    typedef typename PairOf<V>::Z Z;
+    const V *tw1, *tw2;
+    const Z *sa1, *sb1, *sa5, *sb5, *t4hi, *t4lo;
+    __device__ __forceinline__ TwB(const Z *base, const TxLen &L) {
+        tw1 = reinterpret_cast<const V *>(base);
         tw2 = tw1 + L.m1;
-        sa1 = tw2 + L.m2;
+        sa1 = reinterpret_cast<const Z *>(tw2 + L.m2);
         sb1 = sa1 + L.m1;
         sa5 = sb1 + L.m2;
         sb5 = sa5 + L.m1;
         t4hi = sb5 + L.m2;
         t4lo = t4hi + L.m / 64 + 1;
     }
-    __device__ __forceinline__ V w4(int r) const { return vmul(vld(t4hi + (r >> 6)), vld(t4lo + (r & 63))); }
-};
-
-// ---------------------------------------------------------------------------
-// column tiles: pairs p in [p0, p0 + np), tile column lc = side * TP + i
-// (side 0: column p0 + i; side 1: column m2-1-p0-i, absent when it is the
-// middle column already held by side 0); element (j1, lc) at j1 * W + lc.
-// ---------------------------------------------------------------------------
-struct ColGeo {
-    int n, m, m1, m2, P2, TP, W, p0, np, m1h;
-    __device__ __forceinline__ ColGeo(const TxLen &L, int blk) {
-        n = L.n; m = L.m; m1 = L.m1; m2 = L.m2; P2 = L.P2; TP = L.TP; W = 2 * L.TP;
-        p0 = blk * TP;
-        np = min(TP, P2 - p0);
-        m1h = (m1 + 1) >> 1;
-    }
-    __device__ __forceinline__ int col(int lc) const {     // -1: no column
-        const int side = lc >= TP, i = lc - side * TP;
-        if (i >= np) return -1;
-        const int p = p0 + i;
-        if (!side) return p;
-        const int c = m2 - 1 - p;
-        return c == p ? -1 : c;
-    }
-    __device__ __forceinline__ int lcol(int c) const { return c < P2 ? c - p0 : TP + (m2 - 1 - c - p0); }
+    __device__ __forceinline__ Z w4(int r) const { return zmul(vld(t4hi + (r >> 6)), vld(t4lo + (r & 63))); }
 };
 
 // flagged-sample mask (bit u: sample t + u) of samples t..t+cnt-1, cnt <= 4
@@ -185,7 +171,7 @@ __device__ __forceinline__ uint32_t flag_bits(const uint32_t *__restrict__ fl, i
 }
 
 // The four samples of unit j (x_{4j..4j+3}; two at the centre j = m-1-j):
-// load them as z_j = (x0, x2), z_{m-1-j} = (x3, x1).
+// z_j = (x0, x2), z_{m-1-j} = (x3, x1).
 __device__ __forceinline__ float4 ld4(const float *__restrict__ x, int64_t t, bool centre) {
     const float2 a = __ldg(reinterpret_cast<const float2 *>(x + t));
     if (centre) return make_float4(a.x, a.y, 0.f, 0.f);
@@ -196,90 +182,126 @@ __device__ __forceinline__ float4 ld4(const float *__restrict__ x, int64_t t, bo
 // Asynchronous global -> shared copies (cp.async, Ampere and later): every
 // copy of a tile is in flight at once; cp_wait ends them (a barrier must
 // follow before other threads read the tile).
-__device__ __forceinline__ void cp_async(float2 *dst, const float2 *src) {
+__device__ __forceinline__ void cp_async(PF *dst, const float2 *src) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async(double2 *dst, const double2 *src) {
+__device__ __forceinline__ void cp_async(PD *dst, const double2 *src) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-constexpr int TX_UNR = 4;     // units per thread whose loads are issued together
+// ---------------------------------------------------------------------------
+// The intermediate Y of a detscan (m complex values): row pairs {p, m1 - p}
+// (p = 0: rows 0 and m1/2), two planes of m2 values each: the pair's real
+// parts (re_a, re_b), then its imaginary parts.  With m1 odd row 0 has no
+// partner: it is stored last, as plain complex values.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int y_plane(int m1, int p) { return (m1 & 1) ? 2 * (p - 1) : 2 * p; }
 
-// Column tiles have 2 TP = W columns with W a power of two dividing TX_T:
-// thread t keeps column lc = t mod W and takes rows t / W, t / W + TX_T / W,
-// ..., so a column's index arithmetic is done once per thread.
+// ---------------------------------------------------------------------------
+// column tiles: column pairs {c, m2-1-c}, c in [p0, p0 + np); the pair's two
+// columns are the two lanes; element (j1, i) at j1 TP + i.  TP is a power of
+// two dividing TX_T: thread t keeps pair t mod TP and takes rows r0 = t / TP,
+// r0 + rstep, .. (at most TX_ROWS of the m1/2 rows, since TP m1 <= TX_TILE/2).
+// Unit j = j1 m2 + c holds z_j and its mirror z_{m-1-j}, which lies in the
+// other lane at row m1-1-j1: the two units of row j1 fill both lanes of the
+// elements j1 and m1-1-j1.
+// ---------------------------------------------------------------------------
+constexpr int TX_ROWS = 4;
 struct ColThread {
-    int lc, c, r0, rstep, cpart, lpart;   // own column, its index, first row, row step; partner column and slot
-    __device__ __forceinline__ ColThread(const ColGeo &G) {
-        lc = threadIdx.x & (G.W - 1);
-        r0 = threadIdx.x / G.W;
-        rstep = TX_T / G.W;
-        c = G.col(lc);
-        cpart = c < 0 ? -1 : G.m2 - 1 - c;
-        lpart = c < 0 ? -1 : G.lcol(cpart);
+    int m, m1, m2, TP, np, i, c, c2, r0, rstep, m1h;
+    __device__ __forceinline__ ColThread(const TxLen &L, int blk) {
+        m = L.m; m1 = L.m1; m2 = L.m2; TP = L.TP;
+        const int p0 = blk * TP;
+        np = min(TP, L.P2 - p0);
+        i = threadIdx.x & (TP - 1);
+        r0 = threadIdx.x >> L.lgW;
+        rstep = TX_T >> L.lgW;
+        c = i < np ? p0 + i : -1;          // -1: no column
+        c2 = m2 - 1 - c;
+        m1h = (m1 + 1) >> 1;
     }
+    __device__ __forceinline__ int row(int r) const { return r0 + r * rstep; }
+    __device__ __forceinline__ bool mid(int j1) const { return 2 * j1 == m1 - 1; }
+    __device__ __forceinline__ bool centre(int j1) const { return mid(j1) && c == c2; }
+    __device__ __forceinline__ bool second(int j1) const { return !mid(j1) && c != c2; }   // unit (j1, c2) too
 };
 
 // The flag bits of a thread's units, loaded ahead of the transform (all
-// loads in flight together): bit 4i + u is sample u of the thread's i-th
-// unit (rows r0, r0 + rstep, ..; at most TX_TILE / 512 <= 8 units).  Zero
-// without flags (fl null) or for a thread without a column.
-__device__ __forceinline__ uint32_t unit_flags(const ColGeo &G, const ColThread &C, const uint32_t *__restrict__ fl,
-                                               int64_t o)
+// loads in flight together): nibble 2r + u is unit u (column c, c2) of the
+// thread's r-th row.  Zero without flags (fl null) or without a column.
+__device__ __forceinline__ uint32_t unit_flags(const ColThread &C, const uint32_t *__restrict__ fl, int64_t o)
 {
     uint32_t nib = 0;
     if (!fl || C.c < 0) return nib;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int j1 = C.r0 + i * C.rstep;
-        const int j = j1 * G.m2 + C.c;
-        if (j1 < G.m1h && j <= G.m - 1 - j)
-            nib |= flag_bits(fl, o + 4 * static_cast<int64_t>(j), j == G.m - 1 - j ? 2 : 4) << (4 * i);
+    for (int r = 0; r < TX_ROWS; ++r) {
+        const int j1 = C.row(r);
+        if (j1 >= C.m1h) continue;
+        const int64_t t = o + 4 * static_cast<int64_t>(j1 * C.m2);
+        nib |= flag_bits(fl, t + 4 * C.c, C.centre(j1) ? 2 : 4) << (8 * r);
+        if (C.second(j1)) nib |= flag_bits(fl, t + 4 * C.c2, 4) << (8 * r + 4);
     }
     return nib;
 }
 
-// Forward column pass.  For every unit j <= m-1-j of the tile (the four
-// samples x_{4j..4j+3}, two at the centre j = m-1-j): D = ld(j, centre, fb)
-// issues the unit's loads (TX_UNR units per thread at a time; fb: the
-// unit's flag bits, from fl at sample o + 4j, read ahead), then
-// put(D, ea, eb, j, jm, tile, fb) writes z_j at tile element ea = (j1, lc) and
-// z_{m-1-j} at eb = (m1-1-j1, lcol(m2-1-c)).  pre(tile) runs first (after the columns a
-// ragged tile lacks are zeroed), with a barrier before the units.  Then
-// the column FFTs, the twiddle, and the tile out to Y.
-template <class V, class Pre, class Ld, class Put>
-__device__ __forceinline__ void col_forward(const TxCtx &X, V *b0, V *b1, V *__restrict__ Y, const V *__restrict__ twb,
-                                            const uint32_t *__restrict__ fl, Pre pre, Ld ld, Put put)
+// Forward column pass.  D = ld(j, centre, fb) issues a unit's loads (UNR rows
+// per thread at a time; fb: the unit's flag bits, from fl at sample o + 4j,
+// read ahead), val(D, j, centre, fb, wa, wb, v) gives its samples
+// v[0..3] (two at the centre).  With NORM, pre(tile) first fills the tile
+// and wa, wb are the tile's values at z_j and z_{m-1-j}.  Then the column
+// FFTs, the four-step twiddle W_m^{c k1}, and the tile out to Y.
+template <bool NORM, int UNR, class V, class Pre, class Ld, class Val>
+__device__ __forceinline__ void col_forward(const TxCtx &X, V *b0, V *b1, typename PairOf<V>::Z *__restrict__ Y,
+                                            const typename PairOf<V>::Z *__restrict__ twb,
+                                            const uint32_t *__restrict__ fl, Pre pre, Ld ld, Val val)
 {
-    const ColGeo G(X.L, X.blk);
-    const ColThread C(G);
-    const int W = G.W, m1 = G.m1, m2 = G.m2;
+    typedef typename PairOf<V>::Z Z;
+    typedef typename VecT<V>::S S;
+    const ColThread C(X.L, X.blk);
+    const int m1 = C.m1, m2 = C.m2, TP = C.TP;
     if (C.c < 0)
-        for (int j1 = C.r0; j1 < m1; j1 += C.rstep) b0[j1 * W + C.lc] = vzero<V>();
+        for (int j1 = C.r0; j1 < m1; j1 += C.rstep) sst(b0 + j1 * TP + C.i, vzero<V>());
     pre(b0);
-    const uint32_t fnib = unit_flags(G, C, fl, X.o);
-    __syncthreads();
+    const uint32_t fnib = unit_flags(C, fl, X.o);
+    if (NORM) __syncthreads();
     if (C.c >= 0) {
-        for (int j10 = C.r0, i0 = 0; j10 < G.m1h; j10 += TX_UNR * C.rstep, i0 += TX_UNR) {
-            decltype(ld(0, false, 0u)) D[TX_UNR];
-            bool ok[TX_UNR];
 #pragma unroll
-            for (int k = 0; k < TX_UNR; ++k) {
-                const int j1 = j10 + k * C.rstep;
-                const int j = j1 * m2 + C.c;
-                ok[k] = j1 < G.m1h && j <= G.m - 1 - j;
-                if (ok[k]) D[k] = ld(j, j == G.m - 1 - j, (fnib >> (4 * (i0 + k))) & 15u);
+        for (int r1 = 0; r1 < TX_ROWS; r1 += UNR) {
+            decltype(ld(0, false, 0u)) D[UNR][2];
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                const int j1 = C.row(r1 + u);
+                if (j1 >= C.m1h) continue;
+                const uint32_t fb = fnib >> (8 * (r1 + u));
+                D[u][0] = ld(j1 * m2 + C.c, C.centre(j1), fb & 15u);
+                if (C.second(j1)) D[u][1] = ld(j1 * m2 + C.c2, false, (fb >> 4) & 15u);
             }
 #pragma unroll
-            for (int k = 0; k < TX_UNR; ++k) {
-                if (!ok[k]) continue;
-                const int j1 = j10 + k * C.rstep;
-                const int j = j1 * m2 + C.c;
-                put(D[k], j1 * W + C.lc, (m1 - 1 - j1) * W + C.lpart, j, G.m - 1 - j, b0,
-                    (fnib >> (4 * (i0 + k))) & 15u);
+            for (int u = 0; u < UNR; ++u) {
+                const int j1 = C.row(r1 + u);
+                if (j1 >= C.m1h) continue;
+                const uint32_t fb = fnib >> (8 * (r1 + u));
+                V *ea = b0 + j1 * TP + C.i, *eb = b0 + (m1 - 1 - j1) * TP + C.i;
+                V na = vzero<V>(), nb = na;
+                if (NORM) { na = sld(ea); nb = sld(eb); }
+                S va[4], vb[4];
+                val(D[u][0], j1 * m2 + C.c, C.centre(j1), fb & 15u, Z{na.x.a, na.y.a}, Z{nb.x.b, nb.y.b}, va);
+                if (C.mid(j1)) {
+                    sst(ea, C.c == C.c2 ? vmake<V>(pset(va[0], va[0]), pset(va[1], va[1]))
+                                        : vmake<V>(pset(va[0], va[3]), pset(va[2], va[1])));
+                    continue;
+                }
+                if (C.c == C.c2) {
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) vb[s] = va[s];
+                } else {
+                    val(D[u][1], j1 * m2 + C.c2, false, (fb >> 4) & 15u, Z{na.x.b, na.y.b}, Z{nb.x.a, nb.y.a}, vb);
+                }
+                sst(ea, vmake<V>(pset(va[0], vb[0]), pset(va[2], vb[2])));
+                sst(eb, vmake<V>(pset(vb[3], va[3]), pset(vb[1], va[1])));
             }
         }
     }
@@ -287,154 +309,183 @@ __device__ __forceinline__ void col_forward(const TxCtx &X, V *b0, V *b1, V *__r
     const TwB<V> T(twb, X.L);
     V *R = sp_transform<false, TX_T, true>(b0, b1, m1, X.L.s1, X.L.nr1, X.L.lgW, 0, T.tw1);
     if (C.c < 0) return;
-    V *Yq = Y + X.yb + C.c;
-    // W_m^{c k1} from the table at the first row of every TX_UNR rows, then
-    // by steps of W_m^{c rstep} (at most TX_UNR - 1 products from an exact value)
-    const V wstep = C.rstep < m1 ? T.w4(C.c * C.rstep) : vzero<V>();
-    for (int k10 = C.r0; k10 < m1; k10 += TX_UNR * C.rstep) {
-        V w = T.w4(C.c * k10);
+    Z *Yq = Y + X.yb;
+    // W_m^{c p} from the table at the thread's first row, then by steps of
+    // W_m^{c rstep} (at most three products); row m1 - p takes W_m2^c conj(W_m^{c p})
+    const V wc = vtwo<V>(Z{vld(T.tw2 + C.c).x.a, vld(T.tw2 + C.c).y.a}, Z{vld(T.tw2 + C.c2).x.a, vld(T.tw2 + C.c2).y.a});
+    V w = C.r0 < m1 ? vtwo<V>(T.w4(C.c * C.r0), T.w4(C.c2 * C.r0)) : vzero<V>();
+    const V wstep = C.rstep < m1 ? vtwo<V>(T.w4(C.c * C.rstep), T.w4(C.c2 * C.rstep)) : vzero<V>();
 #pragma unroll
-        for (int k = 0; k < TX_UNR; ++k) {
-            const int k1 = k10 + k * C.rstep;
-            if (k1 < m1) Yq[static_cast<int64_t>(k1) * m2] = vmul(R[k1 * W + C.lc], w);
-            if (k + 1 < TX_UNR) w = vmul(w, wstep);
+    for (int r = 0; r < TX_ROWS; ++r) {
+        const int p = C.row(r);
+        if (p >= C.m1h) break;
+        const V za = vmul(sld(R + p * TP + C.i), w);
+        if (p == 0 && (m1 & 1)) {
+            Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
+            y[C.c] = Z{za.x.a, za.y.a};
+            if (C.c2 != C.c) y[C.c2] = Z{za.x.b, za.y.b};
+        } else {
+            const int pr = p ? m1 - p : m1 >> 1;
+            const V wr = p ? vmul<true>(wc, w) : vtwo<V>(T.w4(C.c * pr), T.w4(C.c2 * pr));
+            const V zb = vmul(sld(R + pr * TP + C.i), wr);
+            Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
+            y[C.c] = Z{za.x.a, zb.x.a};
+            y[m2 + C.c] = Z{za.y.a, zb.y.a};
+            if (C.c2 != C.c) {
+                y[C.c2] = Z{za.x.b, zb.x.b};
+                y[m2 + C.c2] = Z{za.y.b, zb.y.b};
+            }
         }
+        w = vmul(w, wstep);
     }
 }
 
-// Inverse column pass: the tile's Y values copied in asynchronously,
-// twiddled in place, inverse FFT of the columns; then for every unit
-// j <= m-1-j: D = ld(j, centre, fb) (issued TX_UNR units at a time) and
-// out(D, ea, eb, j, jm, tile, fb) with ea, eb, fb as for the forward pass
-// (the flag bits are read while the tile loads).
-template <class V, class Ld, class Out>
-__device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1, const V *__restrict__ Y,
-                                            const V *__restrict__ twb, const uint32_t *__restrict__ fl, Ld ld,
-                                            Out out)
+// Inverse column pass: the tile's Y values (every load of a thread in
+// flight), the conjugate twiddle, inverse FFT of the columns; then for every
+// unit D = ld(j, centre, fb) (UNR rows issued at a time) and
+// out(D, j, centre, v, fb) with v its samples (the flag bits are read while
+// the tile loads).
+template <int UNR, class V, class Ld, class Out>
+__device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
+                                            const typename PairOf<V>::Z *__restrict__ Y,
+                                            const typename PairOf<V>::Z *__restrict__ twb,
+                                            const uint32_t *__restrict__ fl, Ld ld, Out out)
 {
-    const ColGeo G(X.L, X.blk);
-    const ColThread C(G);
-    const int W = G.W, m1 = G.m1, m2 = G.m2;
+    typedef typename PairOf<V>::Z Z;
+    typedef typename VecT<V>::S S;
+    const ColThread C(X.L, X.blk);
+    const int m1 = C.m1, m2 = C.m2, TP = C.TP;
     const TwB<V> T(twb, X.L);
     uint32_t fnib = 0;
     if (C.c < 0) {
-        for (int k1 = C.r0; k1 < m1; k1 += C.rstep) b0[k1 * W + C.lc] = vzero<V>();
+        for (int k1 = C.r0; k1 < m1; k1 += C.rstep) sst(b0 + k1 * TP + C.i, vzero<V>());
     } else {
-        const V *Yq = Y + X.yb + C.c;
-        for (int k1 = C.r0; k1 < m1; k1 += C.rstep) cp_async(b0 + k1 * W + C.lc, Yq + static_cast<int64_t>(k1) * m2);
-        fnib = unit_flags(G, C, fl, X.o);
-        cp_wait();
-        // the conjugate four-step twiddle, stepped as in the forward pass
-        const V wstep = C.rstep < m1 ? T.w4(C.c * C.rstep) : vzero<V>();
-        for (int k10 = C.r0; k10 < m1; k10 += TX_UNR * C.rstep) {
-            V w = T.w4(C.c * k10);
+        const Z *Yq = Y + X.yb;
+        Z A[TX_ROWS][4];
 #pragma unroll
-            for (int k = 0; k < TX_UNR; ++k) {
-                const int k1 = k10 + k * C.rstep;
-                if (k1 < m1) b0[k1 * W + C.lc] = vmulc(b0[k1 * W + C.lc], w);
-                if (k + 1 < TX_UNR) w = vmul(w, wstep);
+        for (int r = 0; r < TX_ROWS; ++r) {
+            const int p = C.row(r);
+            if (p >= C.m1h) break;
+            if (p == 0 && (m1 & 1)) {
+                const Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
+                A[r][0] = y[C.c];
+                A[r][1] = y[C.c2];
+            } else {
+                const Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
+                A[r][0] = y[C.c];
+                A[r][1] = y[C.c2];
+                A[r][2] = y[m2 + C.c];
+                A[r][3] = y[m2 + C.c2];
             }
+        }
+        fnib = unit_flags(C, fl, X.o);
+        const V wc = vtwo<V>(Z{vld(T.tw2 + C.c).x.a, vld(T.tw2 + C.c).y.a},
+                             Z{vld(T.tw2 + C.c2).x.a, vld(T.tw2 + C.c2).y.a});
+        V w = C.r0 < m1 ? vtwo<V>(T.w4(C.c * C.r0), T.w4(C.c2 * C.r0)) : vzero<V>();
+        const V wstep = C.rstep < m1 ? vtwo<V>(T.w4(C.c * C.rstep), T.w4(C.c2 * C.rstep)) : vzero<V>();
+#pragma unroll
+        for (int r = 0; r < TX_ROWS; ++r) {
+            const int p = C.row(r);
+            if (p >= C.m1h) break;
+            if (p == 0 && (m1 & 1)) {
+                sst(b0 + C.i, vmul<true>(vtwo<V>(A[r][0], A[r][1]), w));
+            } else {
+                const int pr = p ? m1 - p : m1 >> 1;
+                const V wr = p ? vmul<true>(wc, w) : vtwo<V>(T.w4(C.c * pr), T.w4(C.c2 * pr));
+                const V za = vmake<V>(pset(A[r][0].x, A[r][1].x), pset(A[r][2].x, A[r][3].x));
+                const V zb = vmake<V>(pset(A[r][0].y, A[r][1].y), pset(A[r][2].y, A[r][3].y));
+                sst(b0 + p * TP + C.i, vmul<true>(za, w));
+                sst(b0 + pr * TP + C.i, vmul<true>(zb, wr));
+            }
+            w = vmul(w, wstep);
         }
     }
     __syncthreads();
     V *R = sp_transform<true, TX_T, true>(b0, b1, m1, X.L.s1, X.L.nr1, X.L.lgW, 0, T.tw1);
     if (C.c < 0) return;
-    for (int j10 = C.r0, i0 = 0; j10 < G.m1h; j10 += TX_UNR * C.rstep, i0 += TX_UNR) {
-        decltype(ld(0, false, 0u)) D[TX_UNR];
-        bool ok[TX_UNR];
 #pragma unroll
-        for (int k = 0; k < TX_UNR; ++k) {
-            const int j1 = j10 + k * C.rstep;
-            const int j = j1 * m2 + C.c;
-            ok[k] = j1 < G.m1h && j <= G.m - 1 - j;
-            if (ok[k]) D[k] = ld(j, j == G.m - 1 - j, (fnib >> (4 * (i0 + k))) & 15u);
+    for (int r1 = 0; r1 < TX_ROWS; r1 += UNR) {
+        decltype(ld(0, false, 0u)) D[UNR][2];
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            const int j1 = C.row(r1 + u);
+            if (j1 >= C.m1h) continue;
+            const uint32_t fb = fnib >> (8 * (r1 + u));
+            D[u][0] = ld(j1 * m2 + C.c, C.centre(j1), fb & 15u);
+            if (C.second(j1)) D[u][1] = ld(j1 * m2 + C.c2, false, (fb >> 4) & 15u);
         }
 #pragma unroll
-        for (int k = 0; k < TX_UNR; ++k) {
-            if (!ok[k]) continue;
-            const int j1 = j10 + k * C.rstep;
-            const int j = j1 * m2 + C.c;
-            out(D[k], j1 * W + C.lc, (m1 - 1 - j1) * W + C.lpart, j, G.m - 1 - j, R, (fnib >> (4 * (i0 + k))) & 15u);
+        for (int u = 0; u < UNR; ++u) {
+            const int j1 = C.row(r1 + u);
+            if (j1 >= C.m1h) continue;
+            const uint32_t fb = fnib >> (8 * (r1 + u));
+            const V ea = sld(R + j1 * TP + C.i), eb = sld(R + (m1 - 1 - j1) * TP + C.i);
+            if (C.centre(j1)) {
+                const S v[4] = {ea.x.a, ea.y.a, S(0), S(0)};
+                out(D[u][0], j1 * m2 + C.c, true, v, fb & 15u);
+            } else {
+                const S v[4] = {ea.x.a, eb.y.b, ea.y.a, eb.x.b};
+                out(D[u][0], j1 * m2 + C.c, false, v, fb & 15u);
+            }
+            if (C.second(j1)) {
+                const S v[4] = {ea.x.b, eb.y.a, ea.y.b, eb.x.a};
+                out(D[u][1], j1 * m2 + C.c2, false, v, (fb >> 4) & 15u);
+            }
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// row tiles: row pairs p in [r0, r0 + nr); slot 2i is row r0 + i, slot
-// 2i+1 row m1 - r0 - i (unused when that row is the same, or r0 + i = 0);
-// element (slot, k2) at slot * m2p + k2.
+// row tiles: row pairs p in [r0, r0 + nr); the pair's rows are the two lanes
+// (lane a: row p; lane b: row m1 - p, or m1/2 for p = 0, absent when m1 is
+// odd); element (p, k2) at (p - r0) m2p + k2.
+//
+// Row pass.  The tile's rows in from Y, forward row FFTs, then pre(nubuf)
+// (NORM: a second tile-sized buffer filled with a value per mode; a barrier
+// follows), the real split, Y' = f(k0, k1, mask, Y, nu) for the packed slots
+// of modes k0, k1 (lanes; Y = (X_k, X_{n-k}), or (X_0, X_m) for k = 0; mask
+// bit l: lane l holds a mode not met before, for sums; nu the second buffer's
+// values), the inverse split, inverse row FFTs, and the rows back to Y.
+//
+// Split: with e1 = W_4n^k, e5 = W_4n^{5k} and Za = Z_k, Zb = Z_{m-k},
+//   P = e1 (Za + conj Zb), Q = e5 (-i)(Za - conj Zb),
+//   Y_k = hq conj(P + Q), Y_{m-k} = hq e^{i pi/4} (P - Q)
+// (the twiddles of m - k are those of k rotated by e^{-i pi/4}); the inverse
+// runs it backwards with the same factors.  Mode m - k of row p lies in
+// row m1 - p at m2 - 1 - k2, the other lane of that element, so one thread
+// takes elements k2 and m2 - 1 - k2 together: lane a the pair based in row p,
+// lane b the pair based in row m1 - p.  Rows 0 and m1/2 pair with themselves
+// (p = 0).  The conjugates of P and Q are carried, so no sign is flipped.
 // ---------------------------------------------------------------------------
-struct RowGeo {
-    int n, m, m1, m2, m2p, r0, nr, TR;
-    __device__ __forceinline__ RowGeo(const TxLen &L, int blk) {
-        n = L.n; m = L.m; m1 = L.m1; m2 = L.m2; m2p = L.m2p; TR = L.TR;
-        r0 = blk * TR;
-        nr = min(TR, L.P1 - r0);
-    }
-    __device__ __forceinline__ int row(int slot) const {   // -1: unused
-        const int i = slot >> 1;
-        if (i >= nr) return -1;
-        const int p = r0 + i;
-        if (!(slot & 1)) return p;
-        const int r = m1 - p;
-        return (p == 0 || r == p) ? -1 : r;
-    }
-};
-
-// The split's twiddles of mode k: e1 = W_4n^k, e5 = W_4n^{5k} (for
-// k = k1 + m1 k2 the products of a per-row and a per-column table entry).
-template <class V> struct SplitTw { V e1, e5; };
-// Packed orthonormal coefficients of slot k from Z_k, Z_{m-k} (forward
-// half-split): W = e^{-i pi k/2n} A + e^{-i 5 pi k/2n} B.
-template <class V>
-__device__ __forceinline__ V split_f(const SplitTw<V> &w, V a, V b, typename VecT<V>::S sq) {
-    typedef typename VecT<V>::S S;
-    const V cb = vconj(b);
-    const V A = vscale(vadd(a, cb), static_cast<S>(0.5));
-    const V d = vsub(a, cb);
-    const V Bv = vmake<V>(static_cast<S>(0.5) * d.y, static_cast<S>(-0.5) * d.x);
-    const V Wv = vadd(vmul(w.e1, A), vmul(w.e5, Bv));
-    return vmake<V>(sq * Wv.x, -sq * Wv.y);
-}
-// Z_k from the packed slots k and m-k (inverse half-split; sq includes 1/m).
-template <class V>
-__device__ __forceinline__ V split_i(const SplitTw<V> &wk, const SplitTw<V> &wp, V yk, V yp,
-                                     typename VecT<V>::S sq) {
-    typedef typename VecT<V>::S S;
-    const V Vk = vscale(vmulc(vconj(yk), wk.e1), sq);
-    const V Vp = vscale(vmulc(vconj(yp), wp.e1), sq);
-    const V cVp = vconj(Vp);
-    const V A = vscale(vadd(Vk, cVp), static_cast<S>(0.5));
-    const V e4 = vmulc(wk.e5, wk.e1);                                   // W_4n^{4k} = e^{-2 pi i k/n}
-    const V Bv = vscale(vmulc(vsub(Vk, cVp), e4), static_cast<S>(0.5));
-    return vmake<V>(A.x - Bv.y, A.y + Bv.x);
-}
-
-// Row pass.  Loads the tile's rows from Y, forward row FFTs, then
-// pre(nubuf) (a second tile-sized buffer, or null when pre needs none; a
-// barrier follows), then for every packed slot:
-// Y' = f(e, k, Y) (e: tile element, k: slot, Y = (X_k, X_{n-k}) or (X_0, X_m));
-// with INV_BACK the inverse split and inverse row FFTs follow and the rows go
-// back to Y.  Rows are taken one at a time (their index is uniform over
-// the CTA), the threads over k2.
-template <class V, bool INV_BACK, class Pre, class F>
-__device__ __forceinline__ void row_pass(const TxCtx &X, V *b0, V *b1, V *__restrict__ Y, const V *__restrict__ twb,
-                                         Pre pre, F f)
+template <bool NORM, class V, class Pre, class F>
+__device__ __forceinline__ void row_pass(const TxCtx &X, V *b0, V *b1, typename PairOf<V>::Z *__restrict__ Y,
+                                         const typename PairOf<V>::Z *__restrict__ twb, Pre pre, F f)
 {
+    typedef typename PairOf<V>::Z Z;
     typedef typename VecT<V>::S S;
-    const RowGeo G(X.L, X.blk);
-    const int m1 = G.m1, m2 = G.m2, m2p = G.m2p;
-    const int nslot = 2 * G.TR;
+    typedef typename VecT<V>::C C;
+    const int m = X.L.m, m1 = X.L.m1, m2 = X.L.m2, m2p = X.L.m2p, TR = X.L.TR;
+    const int p0 = X.blk * TR, nr = min(TR, X.L.P1 - p0);
+    const bool odd = m1 & 1;
     const int tid = threadIdx.x;
-    V *Yq = Y + X.yb;
-    for (int sl = 0; sl < nslot; ++sl) {
-        const int r = G.row(sl);
-        V *dst = b0 + sl * m2p;
-        if (r < 0) {
-            for (int k2 = tid; k2 < m2; k2 += TX_T) dst[k2] = vzero<V>();
+    Z *Yq = Y + X.yb;
+    for (int pl = 0; pl < TR; ++pl) {
+        const int p = p0 + pl;
+        V *dst = b0 + pl * m2p;
+        if (pl >= nr) {
+            for (int k2 = tid; k2 < m2; k2 += TX_T) sst(dst + k2, vzero<V>());
+        } else if (odd && p == 0) {
+            const Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
+            for (int k2 = tid; k2 < m2; k2 += TX_T) {
+                const Z z = y[k2];
+                sst(dst + k2, vmake<V>(pset(z.x, S(0)), pset(z.y, S(0))));
+            }
         } else {
-            const V *src = Yq + static_cast<int64_t>(r) * m2;
-            for (int k2 = tid; k2 < m2; k2 += TX_T) cp_async(dst + k2, src + k2);
+            const Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
+            for (int k2 = tid; k2 < m2; k2 += TX_T) {
+                cp_async(&dst[k2].x, y + k2);
+                cp_async(&dst[k2].y, y + m2 + k2);
+            }
         }
     }
     cp_wait();
@@ -442,78 +493,88 @@ __device__ __forceinline__ void row_pass(const TxCtx &X, V *b0, V *b1, V *__rest
     const TwB<V> T(twb, X.L);
     V *R = sp_transform<false, TX_T, false>(b0, b1, m2, X.L.s2, X.L.nr2, X.L.lgS, m2p, T.tw2);
     V *Fr = R == b0 ? b1 : b0;
-    pre(Fr);
-    __syncthreads();
-    const S sqf = static_cast<S>(X.L.sq_fwd), s0f = static_cast<S>(X.L.s0_fwd);
-    const S sqi = static_cast<S>(X.L.sq_inv), s0i = static_cast<S>(X.L.s0_inv);
-    for (int pl = 0; pl < G.nr; ++pl) {
-        const int p = G.r0 + pl;
-        const bool mid = 2 * p == m1;                 // the row pairs with itself
-        // elements (pl, k2) for k2 < cnt; each pairs with mode m - k
-        const int cnt = (p == 0) ? (m2 / 2 + 1) : (mid ? (m2 + 1) / 2 : m2);
-        const int rowa = 2 * pl * m2p, rowb = (p == 0 || mid) ? rowa : rowa + m2p;
-        const V a1 = vld(T.sa1 + p), a5 = vld(T.sa5 + p);
+    if (NORM) {
+        pre(Fr);
+        __syncthreads();
+    }
+    const C h = pdup<C>(static_cast<S>(0.70710678118654752440));
+    for (int pl = 0; pl < nr; ++pl) {
+        const int p = p0 + pl;
+        const int ra = p, rb = p ? m1 - p : (odd ? 0 : m1 >> 1);
+        V *t = R + pl * m2p, *nt = Fr + pl * m2p;
+        const V A1 = vtwo<V>(vld(T.sa1 + ra), vld(T.sa1 + rb)), A5 = vtwo<V>(vld(T.sa5 + ra), vld(T.sa5 + rb));
+        const int cnt = p ? (m2 + 1) >> 1 : (m2 >> 1) + 1;
         for (int k2 = tid; k2 < cnt; k2 += TX_T) {
-            const int q2 = (p == 0) ? (k2 == 0 ? 0 : m2 - k2) : m2 - 1 - k2;
-            const int ia = rowa + k2, ib = rowb + q2;
-            const V Za = R[ia], Zb = R[ib];
-            const int ka = p + m1 * k2;
-            if (ka == 0) {
-                V Yv = vmake<V>((Za.x + Za.y) * s0f, (Za.x - Za.y) * s0f);
-                Yv = f(ia, 0, Yv);
-                if (INV_BACK) {
-                    const S V0 = Yv.x * s0i, Vm = Yv.y * s0i;
-                    R[ia] = vmake<V>(static_cast<S>(0.5) * (V0 + Vm), static_cast<S>(0.5) * (V0 - Vm));
+            const int q = m2 - 1 - k2;                       // partner element (p = 0: lane b)
+            const int q0 = k2 ? m2 - k2 : 0;                 // p = 0: lane a's partner
+            int mb = 3, mp = 3;
+            V Za = sld(t + k2), Zb, nua = vzero<V>(), nub = nua;
+            if (p) {
+                Zb = vswap(sld(t + q));
+                if (NORM) { nua = sld(nt + k2); nub = vswap(sld(nt + q)); }
+                if (q == k2) mb = mp = 1;
+            } else {
+                const int qb = max(q, 0);
+                Zb = vmake<V>(pset(t[q0].x.a, t[qb].x.b), pset(t[q0].y.a, t[qb].y.b));
+                if (NORM) {
+                    nua = sld(nt + k2);
+                    nub = vmake<V>(pset(nt[q0].x.a, nt[qb].x.b), pset(nt[q0].y.a, nt[qb].y.b));
                 }
-                continue;
+                mb = 1 | ((!odd && k2 <= q) ? 2 : 0);
+                mp = ((k2 && q0 != k2) ? 1 : 0) | ((!odd && k2 < q) ? 2 : 0);
             }
-            SplitTw<V> wa;
-            wa.e1 = vmul(a1, vld(T.sb1 + k2));
-            wa.e5 = vmul(a5, vld(T.sb5 + k2));
-            if (ib == ia) {                           // the mode pairs with itself
-                V Ya = split_f(wa, Za, Zb, sqf);
-                Ya = f(ia, ka, Ya);
-                if (INV_BACK) R[ia] = split_i(wa, wa, Ya, Ya, sqi);
-                continue;
+            const Z s1 = vld(T.sb1 + k2), s5 = vld(T.sb5 + k2);
+            const V e1 = vmul(A1, vtwo<V>(s1, s1)), e5 = vmul(A5, vtwo<V>(s5, s5));
+            const V cP = vmul<true>(vmake<V>(padd(Za.x, Zb.x), psub(Zb.y, Za.y)), e1);
+            const V cQ = vmul<true>(vmake<V>(padd(Za.y, Zb.y), psub(Za.x, Zb.x)), e5);
+            V Ya = vadd(cP, cQ);
+            const V cm = vsub(cP, cQ);
+            V Yb = vmake<V>(pmul(h, padd(cm.x, cm.y)), pmul(h, psub(cm.x, cm.y)));
+            const int k0 = ra + m1 * k2, k1 = rb + m1 * k2;
+            if (k0 == 0) {
+                const S s0f = static_cast<S>(X.L.s0_fwd);
+                Ya.x.a = (Za.x.a + Za.y.a) * s0f;
+                Ya.y.a = (Za.x.a - Za.y.a) * s0f;
             }
-            // Both slots of the pair at once (modes k and m - k, whose split
-            // twiddles are e1' = w conj(e1), e5' = -w conj(e5), w = e^{-i pi/4}):
-            // with P = e1 (Za + conj Zb), Q = e5 (-i)(Za - conj Zb),
-            // Y_k = (sq/2) conj(P + Q) and Y_{m-k} = (sq/2) conj(w) (P - Q).
-            const V sum = vmake<V>(Za.x + Zb.x, Za.y - Zb.y), dif = vmake<V>(Za.x - Zb.x, Za.y + Zb.y);
-            const V P = vmul(wa.e1, sum), Q = vmul(wa.e5, vmake<V>(dif.y, -dif.x));
-            const S hq = static_cast<S>(0.5) * sqf;
-            const S h = static_cast<S>(0.70710678118654752440);
-            const V pm = vsub(P, Q);
-            V Ya = vmake<V>(hq * (P.x + Q.x), -hq * (P.y + Q.y));
-            V Yb = vmake<V>(hq * h * (pm.x - pm.y), hq * h * (pm.x + pm.y));
-            Ya = f(ia, ka, Ya);
-            Yb = f(ib, G.m - ka, Yb);
-            if (INV_BACK) {
-                // U_a = (sqi/2) conj(Y_k) conj(e1), U_b = (sqi/2) conj(Y_{m-k}) conj(w) e1;
-                // S = U_a + conj(U_b), G = (U_a - conj(U_b)) conj(e4), e4 = e5 conj(e1);
-                // Z_k = S + i G, Z_{m-k} = conj(S) + i conj(G)
-                const S hi = static_cast<S>(0.5) * sqi;
-                const V Ua = vscale(vmulc(vconj(Ya), wa.e1), hi);
-                const V cb = vmul(vconj(Yb), wa.e1);
-                const V Ub = vscale(vmake<V>(h * (cb.x - cb.y), h * (cb.x + cb.y)), hi);
-                const V Sv = vmake<V>(Ua.x + Ub.x, Ua.y - Ub.y);
-                const V Dv = vmake<V>(Ua.x - Ub.x, Ua.y + Ub.y);
-                const V Gv = vmulc(Dv, vmulc(wa.e5, wa.e1));
-                R[ia] = vmake<V>(Sv.x - Gv.y, Sv.y + Gv.x);
-                R[ib] = vmake<V>(Sv.x + Gv.y, Gv.x - Sv.y);
+            Ya = f(k0, k1, mb, Ya, nua);
+            Yb = f(m - k0, m - k1, mp, Yb, nub);
+            const V cn = vmake<V>(pmul(h, padd(Yb.x, Yb.y)), pmul(h, psub(Yb.x, Yb.y)));
+            const V cs = vmul(vadd(Ya, cn), e1), cd = vmul(vsub(Ya, cn), e5);
+            Za = vmake<V>(padd(cs.x, cd.y), psub(cd.x, cs.y));
+            Zb = vmake<V>(psub(cs.x, cd.y), padd(cd.x, cs.y));
+            if (p) {
+                sst(t + k2, Za);
+                if (q != k2) sst(t + q, vswap(Zb));
+            } else {
+                if (k2 == 0) {
+                    const S s0i = static_cast<S>(X.L.s0_inv), v0 = Ya.x.a * s0i, vm = Ya.y.a * s0i;
+                    Za.x.a = static_cast<S>(0.5) * (v0 + vm);
+                    Za.y.a = static_cast<S>(0.5) * (v0 - vm);
+                }
+                t[k2].x.a = Za.x.a;
+                t[k2].y.a = Za.y.a;
+                if (mp & 1) { t[q0].x.a = Zb.x.a; t[q0].y.a = Zb.y.a; }
+                if (mb & 2) { t[k2].x.b = Za.x.b; t[k2].y.b = Za.y.b; }
+                if (mp & 2) { t[q].x.b = Zb.x.b; t[q].y.b = Zb.y.b; }
             }
         }
     }
-    if (!INV_BACK) return;
     __syncthreads();
-    V *Ri = sp_transform<true, TX_T, false>(R, Fr, m2, X.L.s2, X.L.nr2, X.L.lgS, m2p, T.tw2);
-    for (int sl = 0; sl < nslot; ++sl) {
-        const int r = G.row(sl);
-        if (r < 0) continue;
-        const V *src = Ri + sl * m2p;
-        V *dst = Yq + static_cast<int64_t>(r) * m2;
-        for (int k2 = tid; k2 < m2; k2 += TX_T) dst[k2] = src[k2];
+    const V *Ri = sp_transform<true, TX_T, false>(R, Fr, m2, X.L.s2, X.L.nr2, X.L.lgS, m2p, T.tw2);
+    for (int pl = 0; pl < nr; ++pl) {
+        const int p = p0 + pl;
+        const V *src = Ri + pl * m2p;
+        if (odd && p == 0) {
+            Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
+            for (int k2 = tid; k2 < m2; k2 += TX_T) y[k2] = Z{src[k2].x.a, src[k2].y.a};
+        } else {
+            Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
+            for (int k2 = tid; k2 < m2; k2 += TX_T) {
+                const V v = sld(src + k2);
+                y[k2] = Z{v.x.a, v.x.b};
+                y[m2 + k2] = Z{v.y.a, v.y.b};
+            }
+        }
     }
 }
 
@@ -596,54 +657,72 @@ struct GainTx {
     const float4 *qsc;            // per-detscan FP32 scalars of the call
 };
 
+// A pair of FP32 double-word accumulators (one per lane)
+struct PAcc { PF s, c; };
+__device__ __forceinline__ PAcc pacc_zero() { return PAcc{{0.f, 0.f}, {0.f, 0.f}}; }
+__device__ __forceinline__ void pacc_add(PAcc &a, PF v) {
+    const PF s = padd(a.s, v);
+    const PF bb = psub(s, a.s);
+    const PF e = padd(psub(a.s, psub(s, bb)), psub(v, bb));
+    a.s = s;
+    a.c = padd(a.c, e);
+}
+__device__ __forceinline__ void pacc_add_prod(PAcc &a, PF x, PF y) {
+    const PF p = pmul(x, y);
+    const PF e = pfma(x, y, pneg(p));
+    pacc_add(a, p);
+    a.c = padd(a.c, e);
+}
+__device__ __forceinline__ Acc2 pacc_total(const PAcc &a) { return acc_merge_tx(Acc2{a.s.a, a.c.a}, Acc2{a.s.b, a.c.b}); }
+// the lanes of v that mask names (the others zero)
+__device__ __forceinline__ PF pmask(PF v, int mask) { return PF{(mask & 1) ? v.a : 0.f, (mask & 2) ? v.b : 0.f}; }
+__device__ __forceinline__ PD pmask(PD v, int mask) { return PD{(mask & 1) ? v.a : 0.0, (mask & 2) ? v.b : 0.0}; }
+
 __global__ void __launch_bounds__(TX_T, 3) k_gain_cols(GainTx a)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
-    float2 *b0 = tx_smem, *b1 = tx_smem + TX_TILE;
+    CF2 *b0 = tx_smem, *b1 = tx_smem + TX_PAIRS;
     int cur = -1;
-    int i0, i1;
-    cta_share(a.nitems, i0, i1);
-    for (int it = i0; it < i1; ++it) {
+    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
         const int2 w = a.items[a.item0 + it];
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
         const float *sq = a.s + X.o;
-        col_forward(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](float2 *) {},
+        col_forward<false, 4>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](CF2 *) {},
                     [&](int j, bool ctr, uint32_t) { return ld4(sq, 4 * static_cast<int64_t>(j), ctr); },
-                    [&](const float4 &v, int ea, int eb, int j, int jm, float2 *U, uint32_t fb) {
-                        const float x0 = (fb & 1) ? 0.f : v.x, x1 = (fb & 2) ? 0.f : v.y;
-                        const float x2 = (fb & 4) ? 0.f : v.z, x3 = (fb & 8) ? 0.f : v.w;
-                        if (j == jm) { U[ea] = make_float2(x0, x1); return; }
-                        U[ea] = make_float2(x0, x2);
-                        U[eb] = make_float2(x3, x1);
+                    [&](const float4 &x, int, bool, uint32_t fb, float2, float2, float (&v)[4]) {
+                        v[0] = (fb & 1) ? 0.f : x.x;
+                        v[1] = (fb & 2) ? 0.f : x.y;
+                        v[2] = (fb & 4) ? 0.f : x.z;
+                        v[3] = (fb & 8) ? 0.f : x.w;
                     });
     }
 }
 
 __global__ void __launch_bounds__(TX_T, 3) k_gain_rows(GainTx a)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     __shared__ double s_red[TX_T / 32], s_out[1];
-    float2 *b0 = tx_smem, *b1 = tx_smem + TX_TILE;
+    CF2 *b0 = tx_smem, *b1 = tx_smem + TX_PAIRS;
     int cur = -1;
-    int i0, i1;
-    cta_share(a.nitems, i0, i1);
-    for (int it = i0; it < i1; ++it) {
+    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
         const int2 w = a.items[a.item0 + it];
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, a.psd, nullptr, cur, a.qsc);
         const float fscale = X.fscale, alpha = X.alpha, s2 = X.s2;
         const int n = X.L.n, m = X.L.m;
-        Acc2 sa[1] = {{0.f, 0.f}};
-        row_pass<float2, true>(X, b0, b1, a.Y, a.tw + X.L.twb, [](float2 *) {}, [&](int, int k, float2 S) {
-            const int ka = k, kb = (k == 0) ? m : n - k;
-            const float wa = ka == 0 ? 0.f : sfu_rcp(s2 * (1.0f + tx_fpow(ka, fscale, alpha)));
-            const float wb = sfu_rcp(s2 * (1.0f + tx_fpow(kb, fscale, alpha)));
-            const float2 Wv = make_float2(S.x * wa, S.y * wb);
-            acc_add_prod(sa[0], S.x, Wv.x);
-            acc_add_prod(sa[0], S.y, Wv.y);
-            return Wv;
+        PAcc sum = pacc_zero();
+        const auto weight = [&](int k) { return sfu_rcp(s2 * (1.0f + tx_fpow(k, fscale, alpha))); };
+        row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, [](CF2 *) {}, [&](int k0, int k1, int mask, CF2 S, CF2) {
+            const PF wa = pset(k0 ? weight(k0) : 0.f, k1 ? weight(k1) : 0.f);
+            const PF wb = pset(weight(k0 ? n - k0 : m), weight(k1 ? n - k1 : m));
+            const CF2 W{pmul(S.x, wa), pmul(S.y, wb)};
+            if (mask != 3) { S.x = pmask(S.x, mask); S.y = pmask(S.y, mask); }
+            pacc_add_prod(sum, S.x, W.x);
+            pacc_add_prod(sum, S.y, W.y);
+            return W;
         });
+        const Acc2 sa[1] = {pacc_total(sum)};
         block_sums<1>(sa, s_red, s_out);
         if (threadIdx.x == 0) a.part[4 * static_cast<int64_t>(a.item0 + it)] = s_out[0];
     }
@@ -651,34 +730,24 @@ __global__ void __launch_bounds__(TX_T, 3) k_gain_rows(GainTx a)
 
 __global__ void __launch_bounds__(TX_T, 3) k_gain_colsinv(GainTx a)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     __shared__ double s_red[TX_T / 32], s_out[1];
-    float2 *b0 = tx_smem, *b1 = tx_smem + TX_TILE;
+    CF2 *b0 = tx_smem, *b1 = tx_smem + TX_PAIRS;
     int cur = -1;
-    int i0, i1;
-    cta_share(a.nitems, i0, i1);
-    for (int it = i0; it < i1; ++it) {
+    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
         const int2 w = a.items[a.item0 + it];
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
         const float *dq = a.d + X.o;
-        Acc2 sb[1] = {{0.f, 0.f}};
-        col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
+        PAcc sum = pacc_zero();
+        col_inverse<2>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
             return ld4(dq, 4 * static_cast<int64_t>(j), ctr);
-        }, [&](const float4 &dv, int ea, int eb, int j, int jm, const float2 *U, uint32_t fb) {
-            const bool ctr = j == jm;
-            const float2 za = U[ea];
-            if (ctr) {
-                acc_add_prod(sb[0], (fb & 1) ? 0.f : dv.x, za.x);
-                acc_add_prod(sb[0], (fb & 2) ? 0.f : dv.y, za.y);
-                return;
-            }
-            const float2 zb = U[eb];
-            acc_add_prod(sb[0], (fb & 1) ? 0.f : dv.x, za.x);
-            acc_add_prod(sb[0], (fb & 2) ? 0.f : dv.y, zb.y);
-            acc_add_prod(sb[0], (fb & 4) ? 0.f : dv.z, za.y);
-            acc_add_prod(sb[0], (fb & 8) ? 0.f : dv.w, zb.x);
+        }, [&](const float4 &dv, int, bool, const float (&v)[4], uint32_t fb) {
+            // at the centre the last two samples are zero
+            pacc_add_prod(sum, pset((fb & 1) ? 0.f : dv.x, (fb & 2) ? 0.f : dv.y), pset(v[0], v[1]));
+            pacc_add_prod(sum, pset((fb & 4) ? 0.f : dv.z, (fb & 8) ? 0.f : dv.w), pset(v[2], v[3]));
         });
+        const Acc2 sb[1] = {pacc_total(sum)};
         block_sums<1>(sb, s_red, s_out);
         if (threadIdx.x == 0) a.part[4 * static_cast<int64_t>(a.item0 + it) + 1] = s_out[0];
     }
@@ -743,6 +812,7 @@ __device__ __forceinline__ void ld4s(const void *x, int64_t t, bool centre, S (&
 }
 
 template <class V> struct Chi2Tx {
+    typedef typename PairOf<V>::Z Z;
     const float *d;
     const void *s;                // float or double [N] as V
     const double *gain;
@@ -751,35 +821,51 @@ template <class V> struct Chi2Tx {
     const int64_t *off;
     const TxLen *txl;
     const int32_t *q_tx;
-    const V *tw;
+    const Z *tw;
     const int2 *items;
     int item0, nitems;
     int ndet;
     double fsamp;
     int64_t obase;
-    V *Y;
+    Z *Y;
     double *part;                 // [item][4]
     void *v_out;                  // float or double [N] (global sample index), or null
+    bool v_al;                    // v_out aligned to two values
+};
+
+// Sums over a CTA's modes or samples, one per lane: FP32 double-words (2^-44
+// relative; FP64 adds issue at 1/64 of the FP32 rate) or FP64
+template <class C> struct LaneSum;
+template <> struct LaneSum<PF> {
+    PAcc a = pacc_zero();
+    __device__ __forceinline__ void add(PF v) { pacc_add(a, v); }
+    __device__ __forceinline__ void add_prod(PF x, PF y) { pacc_add_prod(a, x, y); }
+    __device__ __forceinline__ double total() const { return acc_value(pacc_total(a)); }
+};
+template <> struct LaneSum<PD> {
+    double a = 0.0;
+    __device__ __forceinline__ void add(PD v) { a += v.a + v.b; }
+    __device__ __forceinline__ void add_prod(PD x, PD y) { a += x.a * y.a + x.b * y.b; }
+    __device__ __forceinline__ double total() const { return a; }
 };
 
 template <class V>
 __global__ void __launch_bounds__(TX_T) k_chi2_cols(Chi2Tx<V> a)
 {
     typedef typename VecT<V>::S S;
-    extern __shared__ __align__(16) double2 tx_smem64[];
+    typedef typename PairOf<V>::Z Z;
+    extern __shared__ __align__(16) CD2 tx_smem64[];
     __shared__ TxCtx X;
-    V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_TILE;
+    V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_PAIRS;
     int cur = -1;
-    int i0, i1;
-    cta_share(a.nitems, i0, i1);
-    for (int it = i0; it < i1; ++it) {
+    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
         const int2 w = a.items[a.item0 + it];
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
-        const double gq = a.gain[X.q];
+        const S g = static_cast<S>(a.gain[X.q]);
         const float *dq = a.d + X.o;
         const int64_t o = X.o;
         struct U4 { float4 dv; S sx[4]; };
-        col_forward(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](V *) {},
+        col_forward<false, 2>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](V *) {},
                     [&](int j, bool ctr, uint32_t) {
                         const int64_t t = 4 * static_cast<int64_t>(j);
                         U4 D;
@@ -787,37 +873,29 @@ __global__ void __launch_bounds__(TX_T) k_chi2_cols(Chi2Tx<V> a)
                         ld4s<S>(a.s, o + t, ctr, D.sx);
                         return D;
                     },
-                    [&](const U4 &D, int ea, int eb, int j, int jm, V *U, uint32_t fb) {
-                        const bool ctr = j == jm;
-                        const float4 dv = D.dv;
-                        const struct { S x, y, z, w; } sv = {D.sx[0], D.sx[1], D.sx[2], D.sx[3]};
-                        const S g = static_cast<S>(gq);
-                        const S r0 = (fb & 1) ? S(0) : static_cast<S>(dv.x) - g * static_cast<S>(sv.x);
-                        const S r1 = (fb & 2) ? S(0) : static_cast<S>(dv.y) - g * static_cast<S>(sv.y);
-                        const S r2 = (fb & 4) ? S(0) : static_cast<S>(dv.z) - g * static_cast<S>(sv.z);
-                        const S r3 = (fb & 8) ? S(0) : static_cast<S>(dv.w) - g * static_cast<S>(sv.w);
-                        if (ctr) { U[ea] = vmake<V>(r0, r1); return; }
-                        U[ea] = vmake<V>(r0, r2);
-                        U[eb] = vmake<V>(r3, r1);
+                    [&](const U4 &D, int, bool, uint32_t fb, Z, Z, S (&v)[4]) {
+                        v[0] = (fb & 1) ? S(0) : static_cast<S>(D.dv.x) - g * D.sx[0];
+                        v[1] = (fb & 2) ? S(0) : static_cast<S>(D.dv.y) - g * D.sx[1];
+                        v[2] = (fb & 4) ? S(0) : static_cast<S>(D.dv.z) - g * D.sx[2];
+                        v[3] = (fb & 8) ? S(0) : static_cast<S>(D.dv.w) - g * D.sx[3];
                     });
     }
 }
 
-// FP64 per-mode quantities of the chi^2 row pass: the weights and the
-// gradient factors are formed in the pass's precision from the FP64 PSD.
+// The weights and gradient factors of the modes in the pass's precision, the
+// sums as LaneSum.
 template <class V>
 __global__ void __launch_bounds__(TX_T) k_chi2_rows(Chi2Tx<V> a)
 {
     typedef typename VecT<V>::S S;
-    extern __shared__ __align__(16) double2 tx_smem64[];
+    typedef typename VecT<V>::C C;
+    extern __shared__ __align__(16) CD2 tx_smem64[];
     __shared__ TxCtx X;
     __shared__ double s_red[4 * (TX_T / 32)], s_out[4];
-    __shared__ double s_par[4];       // sigma0^2, ln(fsamp/(2 n f_knee)), alpha, f_knee
-    V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_TILE;
+    __shared__ double s_par[4];       // sigma0, ln(fsamp/(2 n f_knee)), alpha, f_knee
+    V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_PAIRS;
     int cur = -1;
-    int i0, i1;
-    cta_share(a.nitems, i0, i1);
-    for (int it = i0; it < i1; ++it) {
+    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
         const int2 w = a.items[a.item0 + it];
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, a.psd, nullptr, cur);
         if (threadIdx.x == 0) {
@@ -831,30 +909,39 @@ __global__ void __launch_bounds__(TX_T) k_chi2_rows(Chi2Tx<V> a)
         const S sig0 = static_cast<S>(s_par[0]), lfs = static_cast<S>(s_par[1]), al = static_cast<S>(s_par[2]);
         const S fk = static_cast<S>(s_par[3]);
         const S s2 = sig0 * sig0;
+        const S d1 = S(2) / sig0, d2 = -s2 * al / fk;
         const int n = X.L.n, m = X.L.m;
-        // sums: L, dL/dsigma0, dL/dfknee, dL/dalpha (FP64 per thread, as the
-        // FP64 path needs; the FP32 path adds FP32 terms into FP64)
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
-        auto mode_terms = [&](int k, S r) -> S {
+        LaneSum<C> sum[4];            // 2 L, dL/dsigma0, dL/dfknee, dL/dalpha
+        // the modes k0, k1 of coefficients r: r / P, their terms added
+        const auto mode_terms = [&](int k0, int k1, int mask, C r) -> C {
             // ln(f/fk) = ln k + ln(fsamp/(2 n fk)); P = s2 (1 + e^{alpha ln(f/fk)})
-            const S lr = log(static_cast<S>(k)) + lfs;
-            const S pw = exp(al * lr);
-            const S P = s2 * (S(1) + pw);
-            const S iP = S(1) / P;
-            const S r2P = r * r * iP;
-            acc[0] += 0.5 * (static_cast<double>(r2P) + static_cast<double>(log(P)));
-            const S h = S(0.5) * (iP - r2P * iP);             // 1/2 (1/P - r^2/P^2)
-            acc[1] += static_cast<double>(h * S(2) * P / sig0);
-            acc[2] += static_cast<double>(h * (-s2 * al * pw / fk));
-            acc[3] += static_cast<double>(h * s2 * pw * lr);
-            return r * iP;
+            const C lr = pset(log(static_cast<S>(max(k0, 1))) + lfs, log(static_cast<S>(max(k1, 1))) + lfs);
+            const C pw = pset(exp(al * lr.a), exp(al * lr.b));
+            const C P = pmul(pdup<C>(s2), padd(pw, pdup<C>(S(1))));
+            const C iP = pset(S(1) / P.a, S(1) / P.b);
+            const C rP = pmul(r, iP), r2P = pmul(r, rP);
+            const C hh = pmul(pdup<C>(S(0.5)), psub(iP, pmul(r2P, iP)));     // 1/2 (1/P - r^2/P^2)
+            const C sp = pmul(pdup<C>(s2), pmul(pw, lr));
+            C t0 = r2P, tl = pset(log(P.a), log(P.b)), t1 = pmul(hh, pmul(P, pdup<C>(d1)));
+            C t2 = pmul(hh, pmul(pw, pdup<C>(d2))), t3 = pmul(hh, sp);
+            if (mask != 3) {
+                t0 = pmask(t0, mask); tl = pmask(tl, mask); t1 = pmask(t1, mask);
+                t2 = pmask(t2, mask); t3 = pmask(t3, mask);
+            }
+            sum[0].add(t0);
+            sum[0].add(tl);
+            sum[1].add(t1);
+            sum[2].add(t2);
+            sum[3].add(t3);
+            return rP;
         };
-        row_pass<V, true>(X, b0, b1, a.Y, a.tw + X.L.twb, [](V *) {}, [&](int, int k, V Rv) {
-            const int ka = k, kb = (k == 0) ? m : n - k;
-            const S wa = ka == 0 ? S(0) : mode_terms(ka, Rv.x);
-            const S wb = mode_terms(kb, Rv.y);
-            return vmake<V>(ka == 0 ? S(0) : wa, wb);
+        row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, [](V *) {}, [&](int k0, int k1, int mask, V Rv, V) {
+            const int on = (k0 ? 1 : 0) | (k1 ? 2 : 0);         // the offset mode does not enter
+            const C x = mode_terms(k0, k1, mask & on, Rv.x);
+            const C y = mode_terms(k0 ? n - k0 : m, k1 ? n - k1 : m, mask, Rv.y);
+            return vmake<V>(on == 3 ? x : pmask(x, on), y);
         });
+        const double acc[4] = {0.5 * sum[0].total(), sum[1].total(), sum[2].total(), sum[3].total()};
         block_sums_d<4>(acc, s_red, s_out);
         if (threadIdx.x < 4) a.part[4 * static_cast<int64_t>(a.item0 + it) + threadIdx.x] = s_out[threadIdx.x];
     }
@@ -864,38 +951,41 @@ template <class V>
 __global__ void __launch_bounds__(TX_T) k_chi2_colsinv(Chi2Tx<V> a)
 {
     typedef typename VecT<V>::S S;
-    extern __shared__ __align__(16) double2 tx_smem64[];
+    typedef typename VecT<V>::C C;
+    extern __shared__ __align__(16) CD2 tx_smem64[];
     __shared__ TxCtx X;
     __shared__ double s_red[TX_T / 32], s_out[1];
-    V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_TILE;
+    V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_PAIRS;
     int cur = -1;
-    int i0, i1;
-    cta_share(a.nitems, i0, i1);
-    for (int it = i0; it < i1; ++it) {
+    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
         const int2 w = a.items[a.item0 + it];
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
         const int64_t o = X.o;
-        double acc[1] = {0.0};
+        LaneSum<C> sum;
         struct U4 { S sx[4]; };
-        col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
+        col_inverse<2>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
             U4 D;
             ld4s<S>(a.s, o + 4 * static_cast<int64_t>(j), ctr, D.sx);
             return D;
-        }, [&](const U4 &D, int ea, int eb, int j, int jm, const V *U, uint32_t fb) {
-            const bool ctr = j == jm;
-            const int64_t t = 4 * static_cast<int64_t>(j);
-            const S *sx = D.sx;
-            const V za = U[ea];
-            const V zb = ctr ? za : U[eb];
-            S v[4] = {(fb & 1) ? S(0) : za.x, (fb & 2) ? S(0) : (ctr ? za.y : zb.y),
-                      (fb & 4) ? S(0) : za.y, (fb & 8) ? S(0) : zb.x};
-            const int cnt = ctr ? 2 : 4;
-            for (int u = 0; u < cnt; ++u) acc[0] -= static_cast<double>(sx[u] * v[u]);
+        }, [&](const U4 &D, int j, bool ctr, const S (&u)[4], uint32_t fb) {
+            const S v[4] = {(fb & 1) ? S(0) : u[0], (fb & 2) ? S(0) : u[1], (fb & 4) ? S(0) : u[2],
+                            (fb & 8) ? S(0) : u[3]};
+            // at the centre the last two samples are zero
+            sum.add_prod(pset(D.sx[0], D.sx[1]), pset(v[0], v[1]));
+            sum.add_prod(pset(D.sx[2], D.sx[3]), pset(v[2], v[3]));
             if (a.v_out) {
-                S *vo = static_cast<S *>(a.v_out) + o + t;
-                for (int u = 0; u < cnt; ++u) vo[u] = v[u];
+                typedef typename PairOf<V>::Z Z;
+                Z *vo = reinterpret_cast<Z *>(static_cast<S *>(a.v_out) + o + 4 * static_cast<int64_t>(j));
+                if (a.v_al) {
+                    vo[0] = Z{v[0], v[1]};
+                    if (!ctr) vo[1] = Z{v[2], v[3]};
+                } else {
+                    S *vs = reinterpret_cast<S *>(vo);
+                    for (int s = 0; s < (ctr ? 2 : 4); ++s) vs[s] = v[s];
+                }
             }
         });
+        const double acc[1] = {-sum.total()};
         block_sums_d<1>(acc, s_red, s_out);
         if (threadIdx.x == 0) a.part[4 * static_cast<int64_t>(a.item0 + it) + 1] = s_out[0];
     }
@@ -1216,43 +1306,45 @@ __device__ void nc_detscan_index(const NcorrTx &a, NcShared &S, int q)
 // Phase 3, column pass of the right-hand side: M (r/sigma0^2 + w1/sigma0),
 // r = d - g s; w1 of z_j is normal pair j of the NC_W1 stream (pair j mod 4
 // of Philox block j/4).
-__device__ void nc_rhs_cols(const NcorrTx &a, const TxCtx &X, float2 *b0, float2 *b1, uint64_t gi)
+__device__ void nc_rhs_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1, uint64_t gi)
 {
     const bool draw = a.mode == TOD_MODE_DRAW;
     const float *dq = a.d + X.o, *sq = a.s + X.o;
     const float g = X.g, inv_s2 = X.inv_s2, inv_s = X.inv_s;
     const uint64_t q = static_cast<uint64_t>(X.q);
-    const ColGeo G(X.L, X.blk);
     struct U8 { float4 dv, sv; };
-    col_forward(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags,
-                [&](float2 *U) {
-                    // the tile's normals: one Philox block per thread, its four
-                    // pairs to the tile elements whose index j falls in it
-                    const ColGeo G(X.L, X.blk);
+    col_forward<true, 2>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags,
+                [&](CF2 *U) {
+                    // the tile's normals: one Philox block per thread and
+                    // round, its four pairs to the elements whose index j
+                    // falls in it.  Lane a of row j1 holds columns p0 ..
+                    // p0 + np - 1, lane b their mirrors: np consecutive j each.
+                    const ColThread C(X.L, X.blk);
+                    const int TP = C.TP, np = C.np, m1 = C.m1, m2 = C.m2, p0 = X.blk * TP;
                     if (!draw) {
-                        for (int e = threadIdx.x; e < G.m1 * G.W; e += TX_T) U[e] = make_float2(0.f, 0.f);
+                        for (int e = threadIdx.x; e < m1 * TP; e += TX_T) sst(U + e, vzero<CF2>());
                         return;
                     }
-                    const int nbk = (G.np + 3) / 4 + 1;          // blocks touching a side's j range of a row
-                    const int total = G.m1 * 2 * nbk;
+                    // a side's j range of a row touches at most (np + 6) / 4
+                    // blocks; 2^lb >= that, so that no division is needed
+                    int lb = 0;
+                    while ((4 << lb) < np + 3) ++lb;
+                    const int total = m1 << (lb + 1);
                     for (int w = threadIdx.x; w < total; w += TX_T) {
-                        const int j1 = w / (2 * nbk), rest = w - j1 * 2 * nbk;
-                        const int side = rest / nbk, bi = rest - side * nbk;
-                        // j range of this row and side: [ja, jb)
-                        int ja, jb;
-                        if (side == 0) { ja = j1 * G.m2 + G.p0; jb = ja + G.np; }
-                        else { jb = j1 * G.m2 + G.m2 - G.p0; ja = jb - G.np; }
+                        const int j1 = w >> (lb + 1), side = (w >> lb) & 1, bi = w & ((1 << lb) - 1);
+                        const int ja = j1 * m2 + (side ? m2 - p0 - np : p0), jb = ja + np;
                         const int bk = (ja >> 2) + bi;
                         if (4 * bk >= jb) continue;
                         const u64x4 rw = philox4x64(static_cast<uint64_t>(bk), q, 1, gi, a.rng.seed, a.rng.band);
+                        float *row = reinterpret_cast<float *>(U + j1 * TP);
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             const int j = 4 * bk + u;
                             if (j < ja || j >= jb) continue;
-                            const int c = j - j1 * G.m2;
-                            const int lc = side == 0 ? c - G.p0 : G.TP + (G.m2 - 1 - c - G.p0);
-                            if (G.col(lc) < 0) continue;      // the middle column's duplicate
-                            U[j1 * G.W + lc] = philox_normal_pair(rw, u);
+                            const int i = side ? jb - 1 - j : j - ja;
+                            const float2 z = philox_normal_pair(rw, u);
+                            row[4 * i + side] = z.x;
+                            row[4 * i + 2 + side] = z.y;
                         }
                     }
                 },
@@ -1260,36 +1352,33 @@ __device__ void nc_rhs_cols(const NcorrTx &a, const TxCtx &X, float2 *b0, float2
                     const int64_t t = 4 * static_cast<int64_t>(j);
                     return U8{ld4(dq, t, ctr), ld4(sq, t, ctr)};
                 },
-                [&](const U8 &D, int ea, int eb, int j, int jm, float2 *U, uint32_t fb) {
-                    const bool ctr = j == jm;
+                [&](const U8 &D, int, bool ctr, uint32_t fb, float2 wa, float2 wb, float (&v)[4]) {
                     const float4 dv = D.dv, sv = D.sv;
-                    const float2 wa = U[ea];
-                    if (ctr) {
-                        U[ea] = make_float2((fb & 1) ? 0.f : fmaf(dv.x - g * sv.x, inv_s2, wa.x * inv_s),
-                                            (fb & 2) ? 0.f : fmaf(dv.y - g * sv.y, inv_s2, wa.y * inv_s));
-                        return;
-                    }
-                    const float2 wb = U[eb];
-                    // samples 4j, 4j+2 -> z_j = (v_{2j}, v_{2j+1}); 4j+3, 4j+1 -> z_{m-1-j}
-                    U[ea] = make_float2((fb & 1) ? 0.f : fmaf(dv.x - g * sv.x, inv_s2, wa.x * inv_s),
-                                        (fb & 4) ? 0.f : fmaf(dv.z - g * sv.z, inv_s2, wa.y * inv_s));
-                    U[eb] = make_float2((fb & 8) ? 0.f : fmaf(dv.w - g * sv.w, inv_s2, wb.x * inv_s),
-                                        (fb & 2) ? 0.f : fmaf(dv.y - g * sv.y, inv_s2, wb.y * inv_s));
+                    // samples 4j, 4j+2 -> z_j; 4j+3, 4j+1 -> z_{m-1-j}; at the centre 4j, 4j+1 -> z_j
+                    v[0] = (fb & 1) ? 0.f : fmaf(dv.x - g * sv.x, inv_s2, wa.x * inv_s);
+                    v[1] = (fb & 2) ? 0.f : fmaf(dv.y - g * sv.y, inv_s2, (ctr ? wa.y : wb.y) * inv_s);
+                    v[2] = (fb & 4) ? 0.f : fmaf(dv.z - g * sv.z, inv_s2, wa.y * inv_s);
+                    v[3] = (fb & 8) ? 0.f : fmaf(dv.w - g * sv.w, inv_s2, wb.x * inv_s);
                 });
 }
 
-// Filter weights of the packed slot pair: beta = 1/(phi + 1/sigma0^2) =
-// sigma0^2/(1 + r), gamma = sigma0^2 r/(1 + r) with r = sigma0^2 phi =
-// (f/f_knee)^-alpha (r = 0 at mode 0).  With every sample flagged beta is
-// 1/phi = sigma0^2 / r (0 at mode 0).
+// Filter weights of a mode: beta = 1/(phi + 1/sigma0^2) = sigma0^2/(1 + r),
+// gamma = sigma0^2 r/(1 + r) with r = sigma0^2 phi = (f/f_knee)^-alpha (r = 0
+// at mode 0).  With every sample flagged beta is 1/phi = sigma0^2 / r (0 at
+// mode 0).
 __device__ __forceinline__ float nc_r(int k, const TxCtx &X) {
     return k == 0 ? 0.f : tx_fpow(k, X.fscale, -X.alpha);
+}
+__device__ __forceinline__ float nc_beta(int k, float s2, const TxCtx &X) { return s2 * sfu_rcp(1.0f + nc_r(k, X)); }
+__device__ __forceinline__ float nc_gamma(int k, float s2, const TxCtx &X) {
+    const float r = nc_r(k, X);
+    return s2 * r * sfu_rcp(1.0f + r);
 }
 
 // Phase 3, row pass of the right-hand side: + sqrt(phi) w2 (mode pair k of
 // the NC_W2 stream), times beta; the spectrum beta (C b + prior term) is
 // written when asked for.
-__device__ void nc_rhs_rows(const NcorrTx &a, const TxCtx &X, float2 *b0, float2 *b1, uint64_t gi)
+__device__ void nc_rhs_rows(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1, uint64_t gi)
 {
     const bool draw = a.mode == TOD_MODE_DRAW;
     const bool allf = X.mode == CG_ALLFLAG;
@@ -1297,96 +1386,95 @@ __device__ void nc_rhs_rows(const NcorrTx &a, const TxCtx &X, float2 *b0, float2
     const float s2 = X.s2, inv_s2 = X.inv_s2;
     const int n = X.L.n, m = X.L.m;
     float *spec = a.spec_out ? a.spec_out + X.o : nullptr;
-    float2 *nu = nullptr;
-    row_pass<float2, true>(X, b0, b1, a.Y, a.tw + X.L.twb,
-        [&](float2 *Fr) {
-            nu = Fr;
-            const RowGeo G(X.L, X.blk);
-            const int npl = G.nr, m1 = G.m1, m2 = G.m2, p0 = G.r0;
+    row_pass<true>(X, b0, b1, a.Y, a.tw + X.L.twb,
+        [&](CF2 *Fr) {
+            const int m1 = X.L.m1, m2 = X.L.m2, m2p = X.L.m2p, TR = X.L.TR;
+            const int p0 = X.blk * TR, npl = min(TR, X.L.P1 - p0);
             if (!draw) {
-                for (int e = threadIdx.x; e < 2 * G.TR * G.m2p; e += TX_T) Fr[e] = make_float2(0.f, 0.f);
+                for (int e = threadIdx.x; e < TR * m2p; e += TX_T) sst(Fr + e, vzero<CF2>());
                 return;
             }
-            // for a fixed k2 the even slots hold k = p0 + pl + m1 k2 and the
-            // odd ones k = m1 - p0 - pl + m1 k2: one Philox block per thread
-            // for up to four consecutive modes of a parity
-            const int nbk = (npl + 3) / 4 + 1;
-            const int items = 2 * nbk * m2;
-            for (int w = threadIdx.x; w < items; w += TX_T) {
-                const int rest = fdiv(w, X.L.f_m2), k2 = w - rest * m2;
-                const int par = rest / nbk, bi = rest - par * nbk;
-                const int kbase = (par == 0 ? p0 : m1 - p0 - (npl - 1)) + m1 * k2;
-                const int bk = (kbase >> 2) + bi;
-                if (npl <= 0 || 4 * bk >= kbase + npl) continue;
-                const u64x4 rw = philox4x64(static_cast<uint64_t>(bk), q, 2, gi, a.rng.seed, a.rng.band);
+            // for a fixed k2 lane a holds k = p0 + pl + m1 k2 and lane b
+            // k = m1 - p0 - pl + m1 k2 (row m1/2, or none, for pair 0): runs
+            // of consecutive modes, one Philox block for up to four of them
+            const int lo = p0 ? p0 : 1;                        // first pair whose lane b runs with the others
+            const float zero = 0.f;
+            for (int w = threadIdx.x; w < 2 * m2; w += TX_T) {
+                const int side = w >= m2, k2 = w - (side ? m2 : 0);
+                const int ka = (side ? m1 - p0 - (npl - 1) : p0) + m1 * k2;
+                const int kb = ka + (side ? p0 + npl - lo : npl);       // modes [ka, kb)
+                float *e0 = reinterpret_cast<float *>(Fr + k2) + side;
+                for (int bk = ka >> 2; 4 * bk < kb; ++bk) {
+                    const u64x4 rw = philox4x64(static_cast<uint64_t>(bk), q, 2, gi, a.rng.seed, a.rng.band);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int k = 4 * bk + u;
-                    if (k < kbase || k >= kbase + npl) continue;
-                    const int pl = par == 0 ? k - kbase : (npl - 1) - (k - kbase);
-                    const int p = p0 + pl;
-                    const int e = (2 * pl + par) * G.m2p + k2;
-                    if (par == 1 && (p == 0 || m1 - p == p)) { Fr[e] = make_float2(0.f, 0.f); continue; }
-                    const int ka = k, kb = (k == 0) ? m : n - k;
-                    const float ra = nc_r(ka, X), rb = nc_r(kb, X);
-                    const float2 w2 = philox_normal_pair(rw, u);
-                    Fr[e] = make_float2(sqrtf(ra * inv_s2) * w2.x, sqrtf(rb * inv_s2) * w2.y);
+                    for (int u = 0; u < 4; ++u) {
+                        const int k = 4 * bk + u;
+                        if (k < ka || k >= kb) continue;
+                        const int pl = side ? npl - 1 - (k - ka) : k - ka;
+                        const float2 z = philox_normal_pair(rw, u);
+                        e0[4 * pl * m2p] = z.x;
+                        e0[4 * pl * m2p + 2] = z.y;
+                    }
+                }
+                if (side && p0 == 0) {
+                    float2 z = make_float2(zero, zero);
+                    if (!(m1 & 1)) {
+                        const int k = (m1 >> 1) + m1 * k2;
+                        z = stream_normal_pair(a.rng.seed, a.rng.band, q, 2, gi, 2 * static_cast<int64_t>(k));
+                    }
+                    e0[0] = z.x;
+                    e0[2] = z.y;
                 }
             }
         },
-        [&](int e, int k, float2 Yv) {
-            const int ka = k, kb = (k == 0) ? m : n - k;
-            const float ra = nc_r(ka, X), rb = nc_r(kb, X);
-            float ba, bb;
-            if (allf) { ba = ka == 0 ? 0.f : s2 * sfu_rcp(ra); bb = s2 * sfu_rcp(rb); }
-            else { ba = s2 * sfu_rcp(1.0f + ra); bb = s2 * sfu_rcp(1.0f + rb); }
-            const float2 cb = make_float2(Yv.x + nu[e].x, Yv.y + nu[e].y);
-            const float2 xs = make_float2(cb.x * ba, cb.y * bb);
-            if (spec) { spec[ka] = xs.x; spec[kb] = xs.y; }
+        [&](int k0, int k1, int mask, CF2 Y, CF2 nu) {
+            const int l0 = k0 ? n - k0 : m, l1 = k1 ? n - k1 : m;
+            const float r0 = nc_r(k0, X), r1 = nc_r(k1, X), u0 = nc_r(l0, X), u1 = nc_r(l1, X);
+            PF bx, by;
+            if (allf) {
+                bx = pset(k0 ? s2 * sfu_rcp(r0) : 0.f, k1 ? s2 * sfu_rcp(r1) : 0.f);
+                by = pset(s2 * sfu_rcp(u0), s2 * sfu_rcp(u1));
+            } else {
+                bx = pset(s2 * sfu_rcp(1.0f + r0), s2 * sfu_rcp(1.0f + r1));
+                by = pset(s2 * sfu_rcp(1.0f + u0), s2 * sfu_rcp(1.0f + u1));
+            }
+            const PF px = pset(sqrtf(r0 * inv_s2), sqrtf(r1 * inv_s2)), py = pset(sqrtf(u0 * inv_s2), sqrtf(u1 * inv_s2));
+            const CF2 xs{pmul(pfma(px, nu.x, Y.x), bx), pmul(pfma(py, nu.y, Y.y), by)};
+            if (spec) {
+                if (mask & 1) { spec[k0] = xs.x.a; spec[l0] = xs.y.a; }
+                if (mask & 2) { spec[k1] = xs.x.b; spec[l1] = xs.y.b; }
+            }
             return xs;
         });
 }
 
 // Phase 3, inverse column pass: x0 out; its flagged samples are the CG
 // right-hand side E^T x0.
-__device__ void nc_x0_cols(const NcorrTx &a, const TxCtx &X, float2 *b0, float2 *b1)
+__device__ void nc_x0_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1)
 {
     const bool cg = X.mode == CG_ACTIVE;
     float *xq = a.x_out + X.o;
     const int64_t o = X.o, obase = a.off[a.q0], w_lo = obase >> 5;
     float *r = a.cgv + a.cgcap;
-    const ColGeo G(X.L, X.blk);
-    col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, cg ? a.flags : nullptr, [&](int, bool, uint32_t) { return 0; },
-                [&](int, int ea, int eb, int j, int jm, const float2 *U, uint32_t fbits) {
-        const bool ctr = j == jm;
+    col_inverse<4>(X, b0, b1, a.Y, a.tw + X.L.twb, cg ? a.flags : nullptr, [&](int, bool, uint32_t) { return 0; },
+                [&](int, int j, bool ctr, const float (&v)[4], uint32_t fb) {
         const int64_t t = 4 * static_cast<int64_t>(j);
-        const float2 za = U[ea];
-        float v[4];
-        if (ctr) { v[0] = za.x; v[1] = za.y; }
-        else {
-            const float2 zb = U[eb];
-            v[0] = za.x; v[1] = zb.y; v[2] = za.y; v[3] = zb.x;
-        }
         reinterpret_cast<float2 *>(xq + t)[0] = make_float2(v[0], v[1]);
         if (!ctr) reinterpret_cast<float2 *>(xq + t + 2)[0] = make_float2(v[2], v[3]);
-        if (cg) {
-            uint32_t fb = fbits;
-            while (fb) {
-                const int u = __ffs(fb) - 1;
-                fb &= fb - 1;
-                r[flag_rank(a.flags, a.wpre, w_lo, obase, o + t + u)] = v[u];
-            }
+        while (fb) {                  // cg only: no flags are read otherwise
+            const int u = __ffs(fb) - 1;
+            fb &= fb - 1;
+            r[flag_rank(a.flags, a.wpre, w_lo, obase, o + t + u)] = u == 0 ? v[0] : u == 1 ? v[1] : u == 2 ? v[2] : v[3];
         }
     });
 }
 
 // CG column pass: z = E vec (the flagged samples' entries of vec, zero
 // elsewhere), forward columns.
-__device__ void nc_scatter_cols(const NcorrTx &a, const TxCtx &X, float2 *b0, float2 *b1, const float *vec)
+__device__ void nc_scatter_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1, const float *vec)
 {
     const int64_t o = X.o, obase = a.off[a.q0], w_lo = obase >> 5;
-    const ColGeo G(X.L, X.blk);
-    col_forward(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](float2 *) {},
+    col_forward<false, 4>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](CF2 *) {},
                 [&](int j, bool, uint32_t fb) {
                     // the unit's flagged entries of vec (a rank lookup only where flagged)
                     const int64_t t = 4 * static_cast<int64_t>(j);
@@ -1399,32 +1487,26 @@ __device__ void nc_scatter_cols(const NcorrTx &a, const TxCtx &X, float2 *b0, fl
                     }
                     return v;
                 },
-                [&](const float4 &D, int ea, int eb, int j, int jm, float2 *U, uint32_t) {
-                    const float v[4] = {D.x, D.y, D.z, D.w};
-                    if (j == jm) { U[ea] = make_float2(v[0], v[1]); return; }
-                    U[ea] = make_float2(v[0], v[2]);
-                    U[eb] = make_float2(v[3], v[1]);
+                [&](const float4 &D, int, bool, uint32_t, float2, float2, float (&v)[4]) {
+                    v[0] = D.x; v[1] = D.y; v[2] = D.z; v[3] = D.w;
                 });
 }
 
 // CG row pass: times gamma (apply S), or times beta (the final B^{-1} E y,
 // whose spectrum is added to the one written at the right-hand side).
 template <bool BETA>
-__device__ void nc_filter_rows(const NcorrTx &a, const TxCtx &X, float2 *b0, float2 *b1)
+__device__ void nc_filter_rows(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1)
 {
     const float s2 = X.s2;
     const int n = X.L.n, m = X.L.m;
     float *spec = (BETA && a.spec_out) ? a.spec_out + X.o : nullptr;
-    row_pass<float2, true>(X, b0, b1, a.Y, a.tw + X.L.twb, [](float2 *) {}, [&](int, int k, float2 Yv) {
-        const int ka = k, kb = (k == 0) ? m : n - k;
-        const float ra = nc_r(ka, X), rb = nc_r(kb, X);
-        float2 r;
-        const float ia = sfu_rcp(1.0f + ra), ib = sfu_rcp(1.0f + rb);
-        if (BETA) {
-            r = make_float2(Yv.x * (s2 * ia), Yv.y * (s2 * ib));
-            if (spec) { spec[ka] += r.x; spec[kb] += r.y; }
-        } else {
-            r = make_float2(Yv.x * (s2 * ra * ia), Yv.y * (s2 * rb * ib));
+    const auto weight = [&](int k) { return BETA ? nc_beta(k, s2, X) : nc_gamma(k, s2, X); };
+    row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, [](CF2 *) {}, [&](int k0, int k1, int mask, CF2 Y, CF2) {
+        const int l0 = k0 ? n - k0 : m, l1 = k1 ? n - k1 : m;
+        const CF2 r{pmul(Y.x, pset(weight(k0), weight(k1))), pmul(Y.y, pset(weight(l0), weight(l1)))};
+        if (spec) {
+            if (mask & 1) { spec[k0] += r.x.a; spec[l0] += r.y.a; }
+            if (mask & 2) { spec[k1] += r.x.b; spec[l1] += r.y.b; }
         }
         return r;
     });
@@ -1432,11 +1514,11 @@ __device__ void nc_filter_rows(const NcorrTx &a, const TxCtx &X, float2 *b0, flo
 
 // CG inverse column pass: q = E^T (...) (gather), or x += (...) (final).
 template <bool ADD>
-__device__ void nc_gather_cols(const NcorrTx &a, const TxCtx &X, float2 *b0, float2 *b1, float *qv)
+__device__ void nc_gather_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1, float *qv)
 {
     const int64_t o = X.o, obase = a.off[a.q0], w_lo = obase >> 5;
     float *xq = a.x_out + X.o;
-    col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, ADD ? nullptr : a.flags, [&](int j, bool ctr, uint32_t) {
+    col_inverse<2>(X, b0, b1, a.Y, a.tw + X.L.twb, ADD ? nullptr : a.flags, [&](int j, bool ctr, uint32_t) {
         // ADD: the unit's x0 (written earlier in this launch: coherent loads,
         // not the read-only path); the gather needs only the flag bits
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1447,28 +1529,18 @@ __device__ void nc_gather_cols(const NcorrTx &a, const TxCtx &X, float2 *b0, flo
             x = make_float4(a01.x, a01.y, a23.x, a23.y);
         }
         return x;
-    }, [&](const float4 &x0, int ea, int eb, int j, int jm, const float2 *U, uint32_t fbits) {
-        if (!ADD && fbits == 0) return;          // no flagged sample in the unit
-        const bool ctr = j == jm;
+    }, [&](const float4 &x0, int j, bool ctr, const float (&v)[4], uint32_t fb) {
         const int64_t t = 4 * static_cast<int64_t>(j);
-        const float2 za = U[ea];
-        float v[4];
-        if (ctr) { v[0] = za.x; v[1] = za.y; }
-        else {
-            const float2 zb = U[eb];
-            v[0] = za.x; v[1] = zb.y; v[2] = za.y; v[3] = zb.x;
-        }
         if (ADD) {
             float2 *p = reinterpret_cast<float2 *>(xq + t);
             p[0] = make_float2(x0.x + v[0], x0.y + v[1]);
             if (!ctr) p[1] = make_float2(x0.z + v[2], x0.w + v[3]);
-        } else {
-            uint32_t fb = fbits;
-            while (fb) {
-                const int u = __ffs(fb) - 1;
-                fb &= fb - 1;
-                qv[flag_rank(a.flags, a.wpre, w_lo, obase, o + t + u)] = v[u];
-            }
+            return;
+        }
+        while (fb) {
+            const int u = __ffs(fb) - 1;
+            fb &= fb - 1;
+            qv[flag_rank(a.flags, a.wpre, w_lo, obase, o + t + u)] = u == 0 ? v[0] : u == 1 ? v[1] : u == 2 ? v[2] : v[3];
         }
     });
 }
@@ -2034,17 +2106,18 @@ __device__ void nc_cg_update(const NcorrTx &a, NcShared &S, int q, float *gb, in
 // cooperative tail kernel finishes any detscan still iterating (grid
 // barriers between its passes; it returns at once when none is).
 // ---------------------------------------------------------------------------
-// Every work item of the launch range, a contiguous share per CTA (tiles of
-// one length together).
+// Every work item of the launch range, grid-stride: neighbouring tiles run at
+// the same time on neighbouring CTAs, so the runs of 64 to 256 bytes that a
+// column tile reads and writes of every row come as whole rows while their
+// DRAM pages are open (a contiguous share per CTA, one tile after the other:
+// k_gain_cols on 82M samples 422 us, k_gain_colsinv 622; so 358, 509).
 template <class Fn>
 __device__ __forceinline__ void nc_items(const NcorrTx &a, TxCtx &X, bool rows, int &cur, Fn fn)
 {
     const int2 *items = rows ? a.rowitems : a.colitems;
     const int j0 = rows ? a.row_off[a.q0] : a.col_off[a.q0];
     const int j1 = rows ? a.row_off[a.q1] : a.col_off[a.q1];
-    int i0, i1;
-    cta_share(j1 - j0, i0, i1);
-    for (int it = j0 + i0; it < j0 + i1; ++it) {
+    for (int it = j0 + blockIdx.x; it < j1; it += gridDim.x) {
         const int2 w = items[it];
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.off[a.q0], a.ndet, a.fsamp, a.psd, a.gain, cur, a.qsc);
         if (threadIdx.x == 0) { X.mode = a.cgs[w.x].mode; X.koff = a.cgs[w.x].koff; }
@@ -2121,23 +2194,21 @@ __device__ void nc_list_by_last(const NcorrTx &a)
     nc_build_list(a, CG_ACTIVE);
 }
 
-// The listed detscans' column (or row) items, a contiguous share per CTA:
-// consecutive items of a CTA are mostly tiles of one detscan.
+// The listed detscans' column (or row) items, grid-stride.
 template <class Fn>
 __device__ __forceinline__ void nc_list_items(const NcorrTx &a, TxCtx &X, bool rows, int &cur, Fn fn)
 {
     const int n = *reinterpret_cast<volatile const int32_t *>(a.list);
     if (n <= 0) return;
     const int32_t *lq = nl_q(a), *lo = rows ? nl_row(a) : nl_col(a);
-    int i0, i1;
-    cta_share(lo[n], i0, i1);
+    const int i0 = blockIdx.x, i1 = lo[n];
     if (i0 >= i1) return;
     int pos = 0, hi = n - 1;                      // last detscan whose items start at or before i0
     while (pos < hi) {
         const int mid = (pos + hi + 1) >> 1;
         if (lo[mid] <= i0) pos = mid; else hi = mid - 1;
     }
-    for (int ii = i0; ii < i1; ++ii) {
+    for (int ii = i0; ii < i1; ii += gridDim.x) {
         while (lo[pos + 1] <= ii) ++pos;
         const int q = lq[pos];
         tx_begin(X, a.txl, a.q_tx, a.off, q, ii - lo[pos], a.off[a.q0], a.ndet, a.fsamp, a.psd, a.gain, cur, a.qsc);
@@ -2173,30 +2244,30 @@ __global__ void __launch_bounds__(TX_T) k_nc_coarse(NcorrTx a)
 }
 __global__ void __launch_bounds__(TX_T, 3) k_nc_rhs_cols(NcorrTx a)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     const uint64_t gi = a.rng.gibbs_iter_dev ? *a.rng.gibbs_iter_dev : a.rng.gibbs_iter;
     int cur = -1;
-    nc_items(a, X, false, cur, [&] { nc_rhs_cols(a, X, tx_smem, tx_smem + TX_TILE, gi); });
+    nc_items(a, X, false, cur, [&] { nc_rhs_cols(a, X, tx_smem, tx_smem + TX_PAIRS, gi); });
 }
 __global__ void __launch_bounds__(TX_T, 3) k_nc_rhs_rows(NcorrTx a)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     const uint64_t gi = a.rng.gibbs_iter_dev ? *a.rng.gibbs_iter_dev : a.rng.gibbs_iter;
     int cur = -1;
-    nc_items(a, X, true, cur, [&] { nc_rhs_rows(a, X, tx_smem, tx_smem + TX_TILE, gi); });
+    nc_items(a, X, true, cur, [&] { nc_rhs_rows(a, X, tx_smem, tx_smem + TX_PAIRS, gi); });
 }
 __global__ void __launch_bounds__(TX_T, 3) k_nc_x0_cols(NcorrTx a)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     int cur = -1;
-    nc_items(a, X, false, cur, [&] { nc_x0_cols(a, X, tx_smem, tx_smem + TX_TILE); });
+    nc_items(a, X, false, cur, [&] { nc_x0_cols(a, X, tx_smem, tx_smem + TX_PAIRS); });
 }
 __global__ void __launch_bounds__(TX_T, 3) k_nc_cg_init(NcorrTx a)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ NcShared S;
     for (int q = a.q0 + blockIdx.x; q < a.q1; q += gridDim.x) {
         __syncthreads();
@@ -2209,7 +2280,7 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_cg_init(NcorrTx a)
 template <bool FINAL>
 __global__ void __launch_bounds__(TX_T, 3) k_nc_scatter(NcorrTx a, int par)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     if (!FINAL) {
         if (blockIdx.x == 0 && threadIdx.x == 0) a.count[par ^ 1] = 0;
@@ -2217,27 +2288,27 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_scatter(NcorrTx a, int par)
     }
     const CgVec V = cg_vecs(a);
     int cur = -1;
-    nc_list_items(a, X, false, cur, [&] { nc_scatter_cols(a, X, tx_smem, tx_smem + TX_TILE, FINAL ? V.y : V.p); });
+    nc_list_items(a, X, false, cur, [&] { nc_scatter_cols(a, X, tx_smem, tx_smem + TX_PAIRS, FINAL ? V.y : V.p); });
 }
 template <bool FINAL>
 __global__ void __launch_bounds__(TX_T, 3) k_nc_filter(NcorrTx a, int par)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     if (!FINAL && *reinterpret_cast<volatile const int32_t *>(a.count + par) == 0) return;
     int cur = -1;
-    nc_list_items(a, X, true, cur, [&] { nc_filter_rows<FINAL>(a, X, tx_smem, tx_smem + TX_TILE); });
+    nc_list_items(a, X, true, cur, [&] { nc_filter_rows<FINAL>(a, X, tx_smem, tx_smem + TX_PAIRS); });
 }
 template <bool FINAL>
 __global__ void __launch_bounds__(TX_T, 3) k_nc_gather(NcorrTx a, int par)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
     if (!FINAL && *reinterpret_cast<volatile const int32_t *>(a.count + par) == 0) return;
     const CgVec V = cg_vecs(a);
     int cur = -1;
     nc_list_items(a, X, false, cur,
-                  [&] { nc_gather_cols<FINAL>(a, X, tx_smem, tx_smem + TX_TILE, FINAL ? nullptr : V.q); });
+                  [&] { nc_gather_cols<FINAL>(a, X, tx_smem, tx_smem + TX_PAIRS, FINAL ? nullptr : V.q); });
 }
 // the listed (iterating) detscans' CG update
 __device__ __forceinline__ void nc_update_listed(const NcorrTx &a, NcShared &S, float *gb, int32_t *count_next)
@@ -2250,7 +2321,7 @@ __device__ __forceinline__ void nc_update_listed(const NcorrTx &a, NcShared &S, 
 }
 __global__ void __launch_bounds__(TX_T, 3) k_nc_update(NcorrTx a, int par)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ NcShared S;
     if (*reinterpret_cast<volatile const int32_t *>(a.count + par) == 0) return;
     nc_update_listed(a, S, reinterpret_cast<float *>(tx_smem), a.count + (par ^ 1));
@@ -2263,18 +2334,18 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_update(NcorrTx a, int par)
 // iteration counts, and the status of detscans left at x0 for want of CG room.
 __global__ void __launch_bounds__(TX_T, 3) k_nc_tail(NcorrTx a, int par)
 {
-    extern __shared__ __align__(16) float2 tx_smem[];
+    extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ NcShared S;
     cgrp::grid_group grid = cgrp::this_grid();
     const CgVec V = cg_vecs(a);
     int cur = -1;
     while (*reinterpret_cast<volatile const int32_t *>(a.count + par) != 0) {
         if (blockIdx.x == 0 && threadIdx.x == 0) a.count[par ^ 1] = 0;
-        nc_list_items(a, S.X, false, cur, [&] { nc_scatter_cols(a, S.X, tx_smem, tx_smem + TX_TILE, V.p); });
+        nc_list_items(a, S.X, false, cur, [&] { nc_scatter_cols(a, S.X, tx_smem, tx_smem + TX_PAIRS, V.p); });
         grid.sync();
-        nc_list_items(a, S.X, true, cur, [&] { nc_filter_rows<false>(a, S.X, tx_smem, tx_smem + TX_TILE); });
+        nc_list_items(a, S.X, true, cur, [&] { nc_filter_rows<false>(a, S.X, tx_smem, tx_smem + TX_PAIRS); });
         grid.sync();
-        nc_list_items(a, S.X, false, cur, [&] { nc_gather_cols<false>(a, S.X, tx_smem, tx_smem + TX_TILE, V.q); });
+        nc_list_items(a, S.X, false, cur, [&] { nc_gather_cols<false>(a, S.X, tx_smem, tx_smem + TX_PAIRS, V.q); });
         grid.sync();
         nc_update_listed(a, S, reinterpret_cast<float *>(tx_smem), a.count + (par ^ 1));
         grid.sync();
@@ -2293,9 +2364,9 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_tail(NcorrTx a, int par)
 // ===========================================================================
 // launchers
 // ===========================================================================
-static size_t tx_smem_bytes(bool fp64) { return (fp64 ? sizeof(double2) : sizeof(float2)) * 2 * TX_TILE; }
+static size_t tx_smem_bytes(bool fp64) { return (fp64 ? sizeof(CD2) : sizeof(CF2)) * 2 * TX_PAIRS; }
 constexpr size_t kGbBytes = (5 * TX_GBCAP + CZ_FLOATS) * sizeof(float);   // preconditioner staging
-static_assert(kGbBytes <= sizeof(float2) * 2 * TX_TILE, "the preconditioner staging fits the tile buffers");
+static_assert(kGbBytes <= sizeof(CF2) * 2 * TX_PAIRS, "the preconditioner staging fits the tile buffers");
 // CG iterations as separate launches.  The two-level preconditioner takes 2.1
 // on average and 4 to 5 at most on the 30 to 70 GHz bands; the rest runs in
 // the cooperative tail, whose grid barriers cost what a launch does.  Launches
@@ -2316,11 +2387,11 @@ cudaError_t setup_tx_kernels(Plan &p)
     const size_t sgb = std::max(s32, kGbBytes);
     if ((e = smem_attr(k_gain_cols, s32)) || (e = smem_attr(k_gain_rows, s32)) || (e = smem_attr(k_gain_colsinv, s32)))
         return e;
-    if ((e = smem_attr(k_chi2_cols<float2>, s32)) || (e = smem_attr(k_chi2_rows<float2>, s32)) ||
-        (e = smem_attr(k_chi2_colsinv<float2>, s32)))
+    if ((e = smem_attr(k_chi2_cols<CF2>, s32)) || (e = smem_attr(k_chi2_rows<CF2>, s32)) ||
+        (e = smem_attr(k_chi2_colsinv<CF2>, s32)))
         return e;
-    if ((e = smem_attr(k_chi2_cols<double2>, s64)) || (e = smem_attr(k_chi2_rows<double2>, s64)) ||
-        (e = smem_attr(k_chi2_colsinv<double2>, s64)))
+    if ((e = smem_attr(k_chi2_cols<CD2>, s64)) || (e = smem_attr(k_chi2_rows<CD2>, s64)) ||
+        (e = smem_attr(k_chi2_colsinv<CD2>, s64)))
         return e;
     if ((e = smem_attr(k_nc_rhs_cols, s32)) || (e = smem_attr(k_nc_rhs_rows, s32)) ||
         (e = smem_attr(k_nc_x0_cols, s32)) || (e = smem_attr(k_nc_cg_init, sgb)) ||
@@ -2387,12 +2458,14 @@ static cudaError_t chi2_range(const Plan &p, const float *d, const void *s, cons
 {
     Chi2Tx<V> a = {};
     a.d = d; a.s = s; a.gain = gain; a.flags = flags; a.psd = psd; a.off = p.off; a.txl = p.txl; a.q_tx = p.q_tx;
-    a.tw = reinterpret_cast<const V *>(sizeof(V) == sizeof(float2) ? static_cast<const void *>(p.txtw)
-                                                                     : static_cast<const void *>(p.txtw64));
+    typedef typename PairOf<V>::Z Z;
+    constexpr bool f32 = sizeof(Z) == sizeof(float2);
+    a.tw = reinterpret_cast<const Z *>(f32 ? static_cast<const void *>(p.txtw) : static_cast<const void *>(p.txtw64));
     a.ndet = p.ndet; a.fsamp = p.fsamp; a.obase = p.h_off[q0];
-    a.Y = reinterpret_cast<V *>(p.ybuf);
+    a.Y = reinterpret_cast<Z *>(p.ybuf);
     a.v_out = v_out;
-    const size_t sm = tx_smem_bytes(sizeof(V) != sizeof(float2));
+    a.v_al = (reinterpret_cast<uintptr_t>(v_out) & (sizeof(Z) - 1)) == 0;
+    const size_t sm = tx_smem_bytes(!f32);
     const int c0 = p.h_col_off[q0], c1 = p.h_col_off[q1], r0 = p.h_row_off[q0], r1 = p.h_row_off[q1];
     double *cpart = p.part;
     double *rpart = p.part + 4 * static_cast<int64_t>(p.h_col_off[p.nq]);
@@ -2425,7 +2498,7 @@ cudaError_t launch_tx_chi2(const Plan &p, bool fp64, const float *d, const void 
 {
     cudaError_t e = cudaSuccess;
     if (!fp64) {
-        e = chi2_range<float2>(p, d, s, gain, flags, psd, chi2_q, dgain, dpsd_q, v_out, st, 0, p.nq);
+        e = chi2_range<CF2>(p, d, s, gain, flags, psd, chi2_q, dgain, dpsd_q, v_out, st, 0, p.nq);
     } else {
         // the intermediate holds ybuf_floats / 4 double2: waves of detscans of
         // at most ybuf_floats / 2 samples (a whole detscan always fits)
@@ -2433,7 +2506,7 @@ cudaError_t launch_tx_chi2(const Plan &p, bool fp64, const float *d, const void 
         while (q < p.nq && e == cudaSuccess) {
             int q1 = q + 1;
             while (q1 < p.nq && p.h_off[q1 + 1] - p.h_off[q] <= p.ybuf_floats / 2) ++q1;
-            e = chi2_range<double2>(p, d, s, gain, flags, psd, chi2_q, dgain, dpsd_q, v_out, st, q, q1);
+            e = chi2_range<CD2>(p, d, s, gain, flags, psd, chi2_q, dgain, dpsd_q, v_out, st, q, q1);
             q = q1;
         }
     }
