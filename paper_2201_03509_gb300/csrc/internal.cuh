@@ -60,7 +60,6 @@ constexpr int TX_PAIRS = TX_TILE / 2;  // as pairs of complex values (fft_reg.cu
 constexpr int TX_RMAX = 10;           // largest Stockham radix of the pair butterflies
 constexpr int TX_MAXR = 20;           // radix stages per sub-transform
 constexpr int TX_GBMAX = 256;         // preconditioner gap blocks per detscan
-constexpr int TX_GBCAP = 2048;        // padded preconditioner elements staged per round
 // Coarse correction of the preconditioner (two-level, balancing form): two
 // vectors per gap block (its indicator and its centred ramp); S Z kept for
 // the TX_CZW neighbouring blocks on either side of each block.

@@ -1112,9 +1112,7 @@ struct NcShared {
     double out[4];
     int3 scan[TX_T / 32 + 1];
     int gbeg[TX_GBMAX], gend[TX_GBMAX];
-    int blen[TX_GBMAX], brank[TX_GBMAX], boff[TX_GBMAX], bq[TX_GBMAX];
-    int rnd[TX_GBMAX + 1];
-    int nrnd, nb;
+    int next, grab[TX_T / 64];         // gap blocks handed out to the warp pairs
     int64_t i64[2];
     double d64[4];
     int flag;
@@ -1546,10 +1544,34 @@ __device__ void nc_gather_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b
 }
 
 // z = M^{-1} r over the detscan's gap blocks: T_L^{-1} = (L(x) L(x)^T -
-// L(w) L(w)^T) / x_0 (Gohberg-Semencul; x = T_L^{-1} e_1 from the Durbin
-// tables, w = (0, x_{L-1}, .., x_1)), blocks staged in rounds of at most
-// TX_GBCAP padded floats.  Returns r.z (CTA total, every thread).  gb: five
-// TX_GBCAP float arrays.
+// L(w) L(w)^T) / x_0 (Gohberg-Semencul; x = T_L^{-1} e_1 from the Toeplitz
+// tables, w = (0, x_{L-1}, .., x_1)).  Returns r.z (CTA total, every thread)
+// with RZ.  z may be r (a block reads its r before it writes its z).
+//
+// A block is taken by a group of two warps, the next free one by each group
+// (the blocks are independent and of very different lengths); a warp forms
+// 128 outputs at a time, four per lane:
+//   u[i] = sum_k (x, w)[k] r[i + k],  z[i] = (1/x_0) sum_s x[s] u1[i-s] - w[s] u2[i-s],
+// with x, w and u1, u2 the lanes of packed FMAs.  A step of four k takes 16
+// packed FMAs, two broadcast loads of (x, w) and one (u: two) 16-byte load of
+// the sliding window, so the FMA pipe is the bound; with the whole CTA on one
+// round of blocks after the other, every operand loaded per output, it was
+// shared memory, and the barriers between the rounds (cg_init of 240
+// detscans of 30 GHz: 151 -> 110 us; of 360 of 70 GHz 268 -> 214, of which
+// these products are 119).
+// gb: GB_FLOATS of shared memory.
+constexpr int GB_GROUPS = TX_T / 64;
+constexpr int GB_TILE = 128;                             // outputs of a warp tile
+constexpr int GB_PAD = GB_TILE + 8;                      // zeros beyond r, and before u
+constexpr int GB_XW = 2 * TOEP_LMAX, GB_U = 2 * (GB_PAD + TOEP_LMAX), GB_R = TOEP_LMAX + GB_PAD;
+constexpr int GB_GROUP_FLOATS = GB_XW + GB_U + GB_R;
+constexpr int GB_FLOATS = GB_GROUPS * GB_GROUP_FLOATS;
+static_assert(GB_XW % 4 == 0 && GB_U % 4 == 0 && GB_R % 4 == 0 && GB_PAD % 4 == 0, "16-byte accesses");
+
+__device__ __forceinline__ void group_sync(int group) {
+    asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
+}
+template <bool RZ>
 __device__ double nc_precond_m1(const NcorrTx &a, NcShared &S, int q, const float *r, float *z, float *gb)
 {
     const int nb = a.gnb[q];
@@ -1562,141 +1584,92 @@ __device__ double nc_precond_m1(const NcorrTx &a, NcShared &S, int q, const floa
             z[i] = v;
             acc_add_prod(rz[0], v, v);
         }
+        if (!RZ) return 0.0;
         block_sums<1>(rz, S.red, S.out);
         return S.out[0];
     }
-    const int det = q % a.ndet;
-    const float *xt_det = a.xtab + static_cast<int64_t>(det) * (TOEP_LMAX * (TOEP_LMAX + 1) / 2);
-    if (threadIdx.x == 0) {
-        int nrnd = 0, len = 0, rq = 0;
-        for (int b = 0; b < nb; ++b) {
-            const int2 bl = a.gblk[static_cast<int64_t>(q) * TX_GBMAX + b];
-            const int reg = ((bl.y + 3) & ~3) + 16;
-            if (b == 0 || len + reg > TX_GBCAP) { S.rnd[nrnd++] = b; len = 0; rq = 0; }
-            S.brank[b] = bl.x; S.blen[b] = bl.y; S.boff[b] = len; S.bq[b] = rq;
-            len += reg;
-            rq += (bl.y + 3) >> 2;
+    const float *xt_det = a.xtab + static_cast<int64_t>(q % a.ndet) * (TOEP_LMAX * (TOEP_LMAX + 1) / 2);
+    const int2 *gbl = a.gblk + static_cast<int64_t>(q) * TX_GBMAX;
+    const int group = threadIdx.x >> 6, gt = threadIdx.x & 63, wg = gt >> 5, lane = threadIdx.x & 31;
+    float *g0 = gb + group * GB_GROUP_FLOATS;
+    PF *xw = reinterpret_cast<PF *>(g0), *u0 = reinterpret_cast<PF *>(g0 + GB_XW), *u = u0 + GB_PAD;
+    float *rb = g0 + GB_XW + GB_U;
+    for (int i = gt; i < GB_PAD; i += 64) u0[i] = PF{0.f, 0.f};
+    if (threadIdx.x == 0) S.next = GB_GROUPS;
+    __syncthreads();
+    for (int b = group; b < nb;) {
+        const int2 bl = gbl[b];
+        const int L = bl.y, L4 = (L + 3) & ~3;
+        const float *xt = xt_det + L * (L - 1) / 2;
+        if (gt == 0) S.grab[group] = atomicAdd(&S.next, 1);
+        for (int i = gt; i < L; i += 64) {
+            const float xv = xt[i];
+            xw[i].a = xv;
+            xw[i ? L - i : 0].b = i ? xv : 0.f;
+            rb[i] = r[bl.x + i];
         }
-        S.rnd[nrnd] = nb;
-        S.nrnd = nrnd;
+        for (int i = L + gt; i < L4 + GB_PAD; i += 64) {
+            if (i < L4) xw[i] = PF{0.f, 0.f};
+            rb[i] = 0.f;                                  // L4 + GB_PAD <= GB_R
+        }
+        group_sync(group);
+        const float inv = 1.0f / xw[0].a;
+        const int nt = (L + GB_TILE - 1) / GB_TILE;
+        // tiles to warps, balancing the triangular sums (u: long first tiles; z: long last ones)
+        for (int t = 0; t < nt; ++t) {
+            if (((t == 1 || t == 2) ? 1 : 0) != wg) continue;
+            const int i0 = t * GB_TILE + 4 * lane;
+            PF acc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+            float4 rc = *reinterpret_cast<const float4 *>(rb + i0);
+#pragma unroll 2
+            for (int k = 0; k < L - t * GB_TILE; k += 4) {
+                const float4 rn = *reinterpret_cast<const float4 *>(rb + i0 + k + 4);
+                const float4 p = *reinterpret_cast<const float4 *>(xw + k), q4 = *reinterpret_cast<const float4 *>(xw + k + 2);
+                const PF w4[4] = {{p.x, p.y}, {p.z, p.w}, {q4.x, q4.y}, {q4.z, q4.w}};
+                const float rw[7] = {rc.x, rc.y, rc.z, rc.w, rn.x, rn.y, rn.z};
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[j] = pfma(w4[kk], pdup<PF>(rw[kk + j]), acc[j]);
+                rc = rn;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) u[i0 + j] = acc[j];
+        }
+        group_sync(group);
+        for (int t = 0; t < nt; ++t) {
+            if ((nt == 3 ? (t == 2 ? 1 : 0) : (t == 1 || t == 2) ? 1 : 0) != wg) continue;
+            const int i0 = t * GB_TILE + 4 * lane;
+            PF acc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+            float4 ua = *reinterpret_cast<const float4 *>(u + i0), ub = *reinterpret_cast<const float4 *>(u + i0 + 2);
+            const int smax = min((t + 1) * GB_TILE, L4);
+#pragma unroll 2
+            for (int s = 0; s < smax; s += 4) {
+                const float4 va = *reinterpret_cast<const float4 *>(u + i0 - s - 4);
+                const float4 vb = *reinterpret_cast<const float4 *>(u + i0 - s - 2);
+                const float4 p = *reinterpret_cast<const float4 *>(xw + s), q4 = *reinterpret_cast<const float4 *>(xw + s + 2);
+                const PF w4[4] = {{p.x, p.y}, {p.z, p.w}, {q4.x, q4.y}, {q4.z, q4.w}};
+                // u[i0 - s - 3 .. i0 - s + 3]
+                const PF uw[7] = {{va.z, va.w}, {vb.x, vb.y}, {vb.z, vb.w}, {ua.x, ua.y}, {ua.z, ua.w},
+                                  {ub.x, ub.y}, {ub.z, ub.w}};
+#pragma unroll
+                for (int ss = 0; ss < 4; ++ss)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[j] = pfma(w4[ss], uw[3 + j - ss], acc[j]);
+                ua = va;
+                ub = vb;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (i0 + j < L) z[bl.x + i0 + j] = (acc[j].a - acc[j].b) * inv;
+        }
+        b = S.grab[group];
+        group_sync(group);
     }
     __syncthreads();
-    float *gb_r = gb, *gb_x = gb + TX_GBCAP, *gb_w = gb + 2 * TX_GBCAP;
-    float *gb_u1 = gb + 3 * TX_GBCAP, *gb_u2 = gb + 4 * TX_GBCAP;
-    for (int rd = 0; rd < S.nrnd; ++rd) {
-        const int b0 = S.rnd[rd], b1 = S.rnd[rd + 1];
-        const int Ll = S.blen[b1 - 1];
-        const int tot = S.boff[b1 - 1] + ((Ll + 3) & ~3) + 16;
-        const int totq = S.bq[b1 - 1] + ((Ll + 3) >> 2);
-        for (int f = threadIdx.x; f < tot; f += TX_T) {
-            int b = b0;
-            while (b + 1 < b1 && S.boff[b + 1] <= f) ++b;
-            const int L = S.blen[b], li = f - S.boff[b] - 8;
-            float rv = 0.f, xv = 0.f, wv = 0.f;
-            if (li >= 0 && li < L) {
-                const float *xt = xt_det + static_cast<int64_t>(L) * (L - 1) / 2;
-                rv = r[S.brank[b] + li];
-                xv = xt[li];
-                wv = li == 0 ? 0.f : xt[L - li];
-            }
-            gb_r[f] = rv; gb_x[f] = xv; gb_w[f] = wv; gb_u1[f] = 0.f; gb_u2[f] = 0.f;
-        }
-        __syncthreads();
-        // u1 = L(x)^T r, u2 = L(w)^T r: four outputs per group of QT threads
-        const int QT = (totq * 4 <= TX_T) ? 4 : (totq * 2 <= TX_T) ? 2 : 1;
-        const int qsh = QT == 4 ? 2 : QT == 2 ? 1 : 0;
-        const int totw = totq << qsh;
-        for (int t0 = 0; t0 < totw; t0 += TX_T) {
-            const int t = t0 + threadIdx.x;
-            const bool act = t < totw;
-            const int qi = t >> qsh, part = t & (QT - 1);
-            float4 a1 = make_float4(0.f, 0.f, 0.f, 0.f), a2 = a1;
-            int base = 0, i0 = 0;
-            if (act) {
-                int b = b0;
-                while (b + 1 < b1 && S.bq[b + 1] <= qi) ++b;
-                const int L = S.blen[b];
-                i0 = 4 * (qi - S.bq[b]);
-                base = S.boff[b] + 8;
-                const float *xb = gb_x + base, *wb = gb_w + base, *rb = gb_r + base + i0;
-                for (int k = 4 * part; k < L - i0; k += 4 * QT) {
-                    const float4 xk = *reinterpret_cast<const float4 *>(xb + k);
-                    const float4 wk = *reinterpret_cast<const float4 *>(wb + k);
-                    const float4 rc = *reinterpret_cast<const float4 *>(rb + k);
-                    const float4 rn = *reinterpret_cast<const float4 *>(rb + k + 4);
-                    a1.x = fmaf(xk.x, rc.x, fmaf(xk.y, rc.y, fmaf(xk.z, rc.z, fmaf(xk.w, rc.w, a1.x))));
-                    a1.y = fmaf(xk.x, rc.y, fmaf(xk.y, rc.z, fmaf(xk.z, rc.w, fmaf(xk.w, rn.x, a1.y))));
-                    a1.z = fmaf(xk.x, rc.z, fmaf(xk.y, rc.w, fmaf(xk.z, rn.x, fmaf(xk.w, rn.y, a1.z))));
-                    a1.w = fmaf(xk.x, rc.w, fmaf(xk.y, rn.x, fmaf(xk.z, rn.y, fmaf(xk.w, rn.z, a1.w))));
-                    a2.x = fmaf(wk.x, rc.x, fmaf(wk.y, rc.y, fmaf(wk.z, rc.z, fmaf(wk.w, rc.w, a2.x))));
-                    a2.y = fmaf(wk.x, rc.y, fmaf(wk.y, rc.z, fmaf(wk.z, rc.w, fmaf(wk.w, rn.x, a2.y))));
-                    a2.z = fmaf(wk.x, rc.z, fmaf(wk.y, rc.w, fmaf(wk.z, rn.x, fmaf(wk.w, rn.y, a2.z))));
-                    a2.w = fmaf(wk.x, rc.w, fmaf(wk.y, rn.x, fmaf(wk.z, rn.y, fmaf(wk.w, rn.z, a2.w))));
-                }
-            }
-            for (int ofs = 1; ofs < QT; ofs <<= 1) {
-                a1.x += __shfl_xor_sync(0xffffffffu, a1.x, ofs); a1.y += __shfl_xor_sync(0xffffffffu, a1.y, ofs);
-                a1.z += __shfl_xor_sync(0xffffffffu, a1.z, ofs); a1.w += __shfl_xor_sync(0xffffffffu, a1.w, ofs);
-                a2.x += __shfl_xor_sync(0xffffffffu, a2.x, ofs); a2.y += __shfl_xor_sync(0xffffffffu, a2.y, ofs);
-                a2.z += __shfl_xor_sync(0xffffffffu, a2.z, ofs); a2.w += __shfl_xor_sync(0xffffffffu, a2.w, ofs);
-            }
-            if (act && part == 0) {
-                *reinterpret_cast<float4 *>(gb_u1 + base + i0) = a1;
-                *reinterpret_cast<float4 *>(gb_u2 + base + i0) = a2;
-            }
-        }
-        __syncthreads();
-        // z = (L(x) u1 - L(w) u2) / x_0
-        for (int t0 = 0; t0 < totw; t0 += TX_T) {
-            const int t = t0 + threadIdx.x;
-            const bool act = t < totw;
-            const int qi = t >> qsh, part = t & (QT - 1);
-            float4 z1 = make_float4(0.f, 0.f, 0.f, 0.f), z2 = z1;
-            int b = b0, i0 = 0, L = 0, base = 0;
-            if (act) {
-                while (b + 1 < b1 && S.bq[b + 1] <= qi) ++b;
-                L = S.blen[b];
-                i0 = 4 * (qi - S.bq[b]);
-                base = S.boff[b] + 8;
-                const float *xb = gb_x + base, *wb = gb_w + base;
-                const float *u1b = gb_u1 + base + i0, *u2b = gb_u2 + base + i0;
-                for (int s0 = 4 * part; s0 <= i0; s0 += 4 * QT) {
-                    const float4 xs = *reinterpret_cast<const float4 *>(xb + s0);
-                    const float4 ws = *reinterpret_cast<const float4 *>(wb + s0);
-                    const float4 ua = *reinterpret_cast<const float4 *>(u1b - s0);
-                    const float4 va = *reinterpret_cast<const float4 *>(u2b - s0);
-                    const float4 ub = *reinterpret_cast<const float4 *>(u1b - s0 - 4);
-                    const float4 vb = *reinterpret_cast<const float4 *>(u2b - s0 - 4);
-                    z1.x = fmaf(xs.x, ua.x, fmaf(xs.y, ub.w, fmaf(xs.z, ub.z, fmaf(xs.w, ub.y, z1.x))));
-                    z1.y = fmaf(xs.x, ua.y, fmaf(xs.y, ua.x, fmaf(xs.z, ub.w, fmaf(xs.w, ub.z, z1.y))));
-                    z1.z = fmaf(xs.x, ua.z, fmaf(xs.y, ua.y, fmaf(xs.z, ua.x, fmaf(xs.w, ub.w, z1.z))));
-                    z1.w = fmaf(xs.x, ua.w, fmaf(xs.y, ua.z, fmaf(xs.z, ua.y, fmaf(xs.w, ua.x, z1.w))));
-                    z2.x = fmaf(ws.x, va.x, fmaf(ws.y, vb.w, fmaf(ws.z, vb.z, fmaf(ws.w, vb.y, z2.x))));
-                    z2.y = fmaf(ws.x, va.y, fmaf(ws.y, va.x, fmaf(ws.z, vb.w, fmaf(ws.w, vb.z, z2.y))));
-                    z2.z = fmaf(ws.x, va.z, fmaf(ws.y, va.y, fmaf(ws.z, va.x, fmaf(ws.w, vb.w, z2.z))));
-                    z2.w = fmaf(ws.x, va.w, fmaf(ws.y, va.z, fmaf(ws.z, va.y, fmaf(ws.w, va.x, z2.w))));
-                }
-            }
-            for (int ofs = 1; ofs < QT; ofs <<= 1) {
-                z1.x += __shfl_xor_sync(0xffffffffu, z1.x, ofs); z1.y += __shfl_xor_sync(0xffffffffu, z1.y, ofs);
-                z1.z += __shfl_xor_sync(0xffffffffu, z1.z, ofs); z1.w += __shfl_xor_sync(0xffffffffu, z1.w, ofs);
-                z2.x += __shfl_xor_sync(0xffffffffu, z2.x, ofs); z2.y += __shfl_xor_sync(0xffffffffu, z2.y, ofs);
-                z2.z += __shfl_xor_sync(0xffffffffu, z2.z, ofs); z2.w += __shfl_xor_sync(0xffffffffu, z2.w, ofs);
-            }
-            if (act && part == 0) {
-                const float inv = 1.0f / gb_x[base];
-                const float zz[4] = {z1.x - z2.x, z1.y - z2.y, z1.z - z2.z, z1.w - z2.w};
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj)
-                    if (i0 + jj < L) {
-                        const float zj = zz[jj] * inv;
-                        z[S.brank[b] + i0 + jj] = zj;
-                        acc_add_prod(rz[0], gb_r[base + i0 + jj], zj);
-                    }
-            }
-        }
-        __syncthreads();
-    }
+    if (!RZ) return 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < K; i += TX_T) acc_add_prod(rz[0], r[i], z[i]);
     block_sums<1>(rz, S.red, S.out);
     return S.out[0];
 }
@@ -1914,16 +1887,15 @@ __device__ __forceinline__ void cz_solve(const float *L, int nc, const float *u,
 
 // z = M r (two-level when the detscan has a coarse correction, else the
 // block inverses alone).  Returns r.z (CTA total, every thread).  gb: the
-// five TX_GBCAP arrays of the block inverses, then CZ_FLOATS for the
-// coarse vectors.
+// block inverses' GB_FLOATS, then CZ_FLOATS for the coarse vectors.
 __device__ double nc_precond(const NcorrTx &a, NcShared &S, int q, const float *r, float *z, float *gb)
 {
     const CgState cs = a.cgs[q];
     const int nb = cs.ncz;
-    if (nb <= 0) return nc_precond_m1(a, S, q, r, z, gb);
+    if (nb <= 0) return nc_precond_m1<true>(a, S, q, r, z, gb);
     const int nc = 2 * nb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float *cL = gb + 5 * TX_GBCAP;                      // [(nc + TX_CZB) rows][CZ_LROW]
+    float *cL = gb + GB_FLOATS;                      // [(nc + TX_CZB) rows][CZ_LROW]
     float *ct = cL + (2 * TX_CBMAX + TX_CZB) * CZ_LROW;  // t = E^{-1} Z^T r
     float *cu = ct + 2 * TX_CBMAX;                      // Z^T r, then (S Z)^T z1
     float *cs2 = cu + 2 * TX_CBMAX;                     // t - E^{-1} (S Z)^T z1
@@ -1936,6 +1908,7 @@ __device__ double nc_precond(const NcorrTx &a, NcShared &S, int q, const float *
     for (int b = warp; b < nb; b += TX_T / 32) {
         const int2 bl = gbl[b];
         float s0 = 0.f, s1 = 0.f;
+#pragma unroll 4
         for (int l = lane; l < bl.y; l += 32) {
             const float v = r[bl.x + l];
             s0 += v;
@@ -1953,6 +1926,7 @@ __device__ double nc_precond(const NcorrTx &a, NcShared &S, int q, const float *
     // w = r - (S Z) t, into z
     for (int b = warp; b < nb; b += TX_T / 32) {
         const int2 bl = gbl[b];
+#pragma unroll 4
         for (int l = lane; l < bl.y; l += 32) {
             const int i = bl.x + l;
             const float2 *row = reinterpret_cast<const float2 *>(sz + static_cast<int64_t>(i) * TX_CZJ);
@@ -1971,7 +1945,7 @@ __device__ double nc_precond(const NcorrTx &a, NcShared &S, int q, const float *
     }
     __syncthreads();
     // z1 = M1 w, in place
-    nc_precond_m1(a, S, q, z, z, gb);
+    nc_precond_m1<false>(a, S, q, z, z, gb);
     __syncthreads();
     // (S Z)^T z1: per block the sums over its rows of each stored column
     for (int b = warp; b < nb; b += TX_T / 32) {
@@ -1979,6 +1953,7 @@ __device__ double nc_precond(const NcorrTx &a, NcShared &S, int q, const float *
         float e[TX_CZJ];
 #pragma unroll
         for (int k = 0; k < TX_CZJ; ++k) e[k] = 0.f;
+#pragma unroll 4
         for (int l = lane; l < bl.y; l += 32) {
             const int i = bl.x + l;
             const float2 *row = reinterpret_cast<const float2 *>(sz + static_cast<int64_t>(i) * TX_CZJ);
@@ -2016,6 +1991,7 @@ __device__ double nc_precond(const NcorrTx &a, NcShared &S, int q, const float *
     for (int b = warp; b < nb; b += TX_T / 32) {
         const int2 bl = gbl[b];
         const float c0 = cs2[2 * b], c1 = cs2[2 * b + 1];
+#pragma unroll 4
         for (int l = lane; l < bl.y; l += 32) {
             const int i = bl.x + l;
             const float zi = z[i] + fmaf(c1, cz_ramp(l, bl.y), c0);
@@ -2037,6 +2013,7 @@ __device__ void nc_cg_init(const NcorrTx &a, NcShared &S, int q, float *gb)
     const int64_t k0 = cs.koff;
     const int K = cs.K;
     Acc2 rr[1] = {{0.f, 0.f}};
+#pragma unroll 4
     for (int i = threadIdx.x; i < K; i += TX_T) {
         const float v = V.r[k0 + i];
         V.y[k0 + i] = 0.f;
@@ -2045,6 +2022,7 @@ __device__ void nc_cg_init(const NcorrTx &a, NcShared &S, int q, float *gb)
     block_sums<1>(rr, S.red, S.out);
     const double rr0 = S.out[0];
     const double rz = nc_precond(a, S, q, V.r + k0, V.z + k0, gb);
+#pragma unroll 4
     for (int i = threadIdx.x; i < K; i += TX_T) V.p[k0 + i] = V.z[k0 + i];
     if (threadIdx.x == 0) {
         cs.rz = rz;
@@ -2065,10 +2043,12 @@ __device__ void nc_cg_update(const NcorrTx &a, NcShared &S, int q, float *gb, in
     const int64_t k0 = cs.koff;
     const int K = cs.K;
     Acc2 pq[1] = {{0.f, 0.f}};
+#pragma unroll 4
     for (int i = threadIdx.x; i < K; i += TX_T) acc_add_prod(pq[0], V.p[k0 + i], V.q[k0 + i]);
     block_sums<1>(pq, S.red, S.out);
     const float alp = static_cast<float>(cs.rz / S.out[0]);
     Acc2 rr[1] = {{0.f, 0.f}};
+#pragma unroll 4
     for (int i = threadIdx.x; i < K; i += TX_T) {
         V.y[k0 + i] = fmaf(alp, V.p[k0 + i], V.y[k0 + i]);
         const float rn = fmaf(-alp, V.q[k0 + i], V.r[k0 + i]);
@@ -2088,7 +2068,8 @@ __device__ void nc_cg_update(const NcorrTx &a, NcShared &S, int q, float *gb, in
     if (cont) {
         const double rzn = nc_precond(a, S, q, V.r + k0, V.z + k0, gb);
         const float beta = static_cast<float>(rzn / cs.rz);
-        for (int i = threadIdx.x; i < K; i += TX_T) V.p[k0 + i] = fmaf(beta, V.p[k0 + i], V.z[k0 + i]);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < K; i += TX_T) V.p[k0 + i] = fmaf(beta, V.p[k0 + i], V.z[k0 + i]);
         cs.rz = rzn;
     }
     __syncthreads();
@@ -2365,7 +2346,7 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_tail(NcorrTx a, int par)
 // launchers
 // ===========================================================================
 static size_t tx_smem_bytes(bool fp64) { return (fp64 ? sizeof(CD2) : sizeof(CF2)) * 2 * TX_PAIRS; }
-constexpr size_t kGbBytes = (5 * TX_GBCAP + CZ_FLOATS) * sizeof(float);   // preconditioner staging
+constexpr size_t kGbBytes = (GB_FLOATS + CZ_FLOATS) * sizeof(float);   // preconditioner staging
 static_assert(kGbBytes <= sizeof(CF2) * 2 * TX_PAIRS, "the preconditioner staging fits the tile buffers");
 // CG iterations as separate launches.  The two-level preconditioner takes 2.1
 // on average and 4 to 5 at most on the 30 to 70 GHz bands; the rest runs in
