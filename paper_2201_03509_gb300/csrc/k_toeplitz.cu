@@ -296,70 +296,133 @@ k_cz_tables(const float *__restrict__ hk, int href, const float4 *__restrict__ c
 // 1 + r . y^(k) is Q_k[0], and
 //   P_{k+1}[m] = P_k[m+1] + alpha Q_k[m+1],  Q_{k+1}[m] = Q_k[m] + alpha P_k[m],
 //   y^(k+1) = (y^(k) + alpha reversed y^(k), alpha):
-// element-wise, one barrier per order.  Half of the CTA owns the (P, Q)
-// elements, the other half y and the output rows.  Arithmetic in FP32
+// element-wise, one barrier per order.  A thread of the first half of the CTA
+// owns four consecutive (P, Q) elements (an order needs one neighbour's value
+// through shared memory), one of the second half two pairs (i, k - 1 - i) of
+// y; both updates are two multiply-adds with one alpha, the lanes of packed
 // double-words (about 2^-45 relative: the input lags carry the 2^-24 of an
-// FP32 transform), because this part issues FP64 at 1/64 of the FP32 rate
-// and one dependent FP64 division costs more than a whole order does here.
-// Measured, 1 to 12 detectors: 2540 us with the dot products, 223 us so.
-constexpr int DT = 2 * TOEP_LMAX;
-static_assert(TOEP_LMAX == 512, "one thread per element in each half of the CTA");
+// FP32 transform; FP64 issues at 1/64 of the FP32 rate on this part and one
+// dependent FP64 division costs more than a whole order does here).  The
+// first thread forms the next order's alpha while the others still update.
+// Measured, 1 to 12 detectors: 2540 us with the dot products, 223 us with
+// scalar double-words and a thread per element and per y, 176 us packed,
+// 162 us with four elements a thread (an order is bound by its
+// chain of dependent operations and the barrier).
+constexpr int DTE = 4, DTY = 2;                    // elements, y pairs per thread
+constexpr int DTH = TOEP_LMAX / DTE;               // threads of each half
+constexpr int DT = 2 * DTH;
+static_assert(DTH * DTY * 2 == TOEP_LMAX, "the second half covers every pair of y");
+
+// double-words in the two lanes: x + a b with a one double-word for both
+struct DW2 { PF h, l; };
+__device__ __forceinline__ DW2 dw2_fma(DW2 x, DW a, DW2 b) {
+    const PF ah = pdup<PF>(a.h), al = pdup<PF>(a.l);
+    const PF p = pmul(ah, b.h);
+    PF e = pfma(ah, b.h, pneg(p));
+    e = pfma(ah, b.l, e);
+    e = pfma(al, b.h, e);
+    const PF s = padd(x.h, p);
+    const PF bb = psub(s, x.h);
+    PF r = padd(psub(x.h, psub(s, bb)), psub(p, bb));
+    r = padd(r, padd(x.l, e));
+    DW2 o;
+    o.h = padd(s, r);
+    o.l = psub(r, psub(o.h, s));
+    return o;
+}
+
+// (alpha of the next order, 1 / (its pivot h(0)), the pivot) from P[0], Q[0].
+// The reciprocal approximation gets one Newton step; alpha a correction.
+__device__ __forceinline__ float4 schur_pivot(DW P, DW Q, float it0) {
+    float inv;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(Q.h));
+    inv = __fmaf_rn(__fmaf_rn(-Q.h, inv, 1.0f), inv, inv);
+    const float q = __fmul_rn(-P.h, inv);
+    // the remainder -P - q Q
+    float r = __fmaf_rn(-q, Q.h, -P.h);
+    r = __fadd_rn(r, __fmaf_rn(-q, Q.l, -P.l));
+    const DW al = dw_renorm(q, __fmul_rn(r, inv));
+    return make_float4(al.h, al.l, it0 * inv, Q.h);
+}
 
 __global__ void __launch_bounds__(DT)
 k_toep_durbin(const float *__restrict__ hk, int href, float *__restrict__ xtab, int32_t *__restrict__ lvalid)
 {
     const int det = blockIdx.x;
-    const int t = threadIdx.x & (TOEP_LMAX - 1);        // element index
-    const bool pq = threadIdx.x < TOEP_LMAX;            // the (P, Q) half; else the y half
-    __shared__ float4 s_pq[2][TOEP_LMAX + 1];           // (P, Q) double-words of the even and odd orders
+    const bool pq = threadIdx.x < DTH;
+    const int g = pq ? threadIdx.x : threadIdx.x - DTH;
+    __shared__ float4 s_pq[2][DTH + 1];                 // first (P, Q) of each thread: heads, tails; by parity
     __shared__ DW s_y[2][TOEP_LMAX];
+    __shared__ float4 s_pv[2];                          // the order's pivot values (schur_pivot)
     const float *h = hk + static_cast<int64_t>(det) * href;
     float *xt = xtab + static_cast<int64_t>(det) * (TOEP_LMAX * (TOEP_LMAX + 1) / 2);
     const float t0 = h[0];
     if (!(t0 > 0.0f)) { if (threadIdx.x == 0) lvalid[det] = 0; return; }
-    DW P{0.f, 0.f}, Q{0.f, 0.f};
+    const float it0 = 1.0f / t0;
+    DW2 V[DTE];                                         // lanes P, Q
     if (pq) {
         // order 0: P[m] = r(1 + m), Q[m] = r(m), r = h / h(0)
         const DW d0{t0, 0.f};
-        if (t + 1 < TOEP_LMAX) P = dw_div(DW{h[t + 1], 0.f}, d0);
-        Q = dw_div(DW{h[t], 0.f}, d0);
-        s_pq[0][t] = make_float4(P.h, P.l, Q.h, Q.l);
-        if (t == 0) {
-            s_pq[0][TOEP_LMAX] = s_pq[1][TOEP_LMAX] = make_float4(0.f, 0.f, 0.f, 0.f);
-            xt[0] = 1.0f / t0;
+#pragma unroll
+        for (int i = 0; i < DTE; ++i) {
+            const int e = DTE * g + i;
+            const DW P = dw_div(DW{e + 1 < TOEP_LMAX ? h[e + 1] : 0.f, 0.f}, d0), Q = dw_div(DW{h[e], 0.f}, d0);
+            V[i] = DW2{{P.h, Q.h}, {P.l, Q.l}};
+        }
+        s_pq[0][g] = make_float4(V[0].h.a, V[0].h.b, V[0].l.a, V[0].l.b);
+        if (g == 0) {
+            s_pq[0][DTH] = s_pq[1][DTH] = make_float4(0.f, 0.f, 0.f, 0.f);
+            s_pv[0] = schur_pivot(DW{V[0].h.a, V[0].l.a}, DW{V[0].h.b, V[0].l.b}, it0);
+            xt[0] = it0;
         }
     }
     __syncthreads();
     int valid = 1;
+    float *xk = xt;                                     // the row of order k (length k)
     for (int k = 0; k < TOEP_LMAX; ++k) {
         const int cur = k & 1;
-        const float4 z = s_pq[cur][0];                  // P_k[0], Q_k[0]: the pivot is Q_k[0]
-        const DW beta{z.z, z.w};
-        if (!(beta.h > 0.0f) || !isfinite(beta.h)) break;
-        if (k > 0) {
-            // order k + 1: x = (1, y^(k)) / (pivot h(0))
-            valid = k + 1;
-            if (!pq) {
-                const float sc = 1.0f / (beta.h * t0);
-                float *xk = xt + (k + 1) * k / 2;
-                if (t < k) { const DW v = s_y[cur][t]; xk[t + 1] = (v.h + v.l) * sc; }
-                else if (t == k) xk[0] = sc;
-            }
-            if (k + 1 >= TOEP_LMAX) break;
-        }
-        const DW alpha = dw_div(DW{-z.x, -z.y}, beta);
+        const float4 pv = s_pv[cur];
+        if (!(pv.w > 0.0f) || pv.w > 3.0e38f) break;    // pivot not positive, or not finite
+        xk += k;                                        // the row of order k + 1
+        if (k > 0) valid = k + 1;
+        const bool last = k + 1 >= TOEP_LMAX;
+        const DW alpha{pv.x, pv.y};
         if (pq) {
-            if (t < TOEP_LMAX - k) {
-                const float4 nx = s_pq[cur][t + 1];
-                const DW Qn = dw_fma(Q, alpha, P);
-                P = dw_fma(DW{nx.x, nx.y}, alpha, DW{nx.z, nx.w});
-                Q = Qn;
-                s_pq[cur ^ 1][t] = make_float4(P.h, P.l, Q.h, Q.l);
+            if (last) break;
+            if (DTE * g < TOEP_LMAX - k) {
+                const float4 n4 = s_pq[cur][g + 1];
+                const DW2 nx{{n4.x, n4.y}, {n4.z, n4.w}};
+#pragma unroll
+                for (int i = 0; i < DTE; ++i) {
+                    // (P[e+1], Q[e]) + alpha (Q[e+1], P[e])
+                    const DW2 up = i + 1 < DTE ? V[i + 1] : nx;
+                    V[i] = dw2_fma(DW2{{up.h.a, V[i].h.b}, {up.l.a, V[i].l.b}}, alpha,
+                                   DW2{{up.h.b, V[i].h.a}, {up.l.b, V[i].l.a}});
+                    if (i == 0) {
+                        s_pq[cur ^ 1][g] = make_float4(V[0].h.a, V[0].h.b, V[0].l.a, V[0].l.b);
+                        if (g == 0) s_pv[cur ^ 1] = schur_pivot(DW{V[0].h.a, V[0].l.a}, DW{V[0].h.b, V[0].l.b}, it0);
+                    }
+                }
             }
         } else {
-            if (t < k) s_y[cur ^ 1][t] = dw_fma(s_y[cur][t], alpha, s_y[cur][k - 1 - t]);
-            else if (t == k) s_y[cur ^ 1][t] = alpha;
+            // order k + 1: x = (1, y^(k)) / (pivot h(0)); then y^(k+1)
+#pragma unroll
+            for (int i = 0; i < DTY; ++i) {
+                const int t = g + i * DTH, j = k - 1 - t;       // an element and its partner
+                if (t > j) break;
+                const DW a = s_y[cur][t], b = s_y[cur][j];
+                const DW2 n = dw2_fma(DW2{{a.h, b.h}, {a.l, b.l}}, alpha, DW2{{b.h, a.h}, {b.l, a.l}});
+                s_y[cur ^ 1][t] = DW{n.h.a, n.l.a};
+                if (j != t) s_y[cur ^ 1][j] = DW{n.h.b, n.l.b};
+                xk[t + 1] = (a.h + a.l) * pv.z;
+                if (j != t) xk[j + 1] = (b.h + b.l) * pv.z;
+            }
+            if (g == 0) {
+                if (k > 0) xk[0] = pv.z;
+                s_y[cur ^ 1][k] = alpha;
+            }
         }
+        if (last) break;
         __syncthreads();
     }
     if (threadIdx.x == 0) lvalid[det] = valid;

@@ -753,20 +753,33 @@ __global__ void __launch_bounds__(TX_T, 3) k_gain_colsinv(GainTx a)
     }
 }
 
-// Per detscan: a and b summed over its row and column items in item order,
-// then the draw g ~ N(b/a, 1/a); a <= 0 (no usable sample) or a non-finite
-// sum gives g = 0 and TOD_ERR_ARG.  One thread per detscan.
+// The sum over items [i0, i1) of value k of their partials, one warp (lanes
+// stride, then a tree: a fixed order); every lane gets it.  A thread adding
+// the items one after the other waits out an FP64 add (about 40 ns here)
+// for each.
+__device__ __forceinline__ double item_sum(const double *__restrict__ part, int i0, int i1, int k)
+{
+    double t = 0.0;
+    for (int i = i0 + static_cast<int>(threadIdx.x & 31); i < i1; i += 32) t += part[4 * static_cast<int64_t>(i) + k];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+// Per detscan (one warp): a and b summed over its row and column items, then
+// the draw g ~ N(b/a, 1/a); a <= 0 (no usable sample) or a non-finite sum
+// gives g = 0 and TOD_ERR_ARG.
 __global__ void __launch_bounds__(256) k_gain_fin(const double *__restrict__ rpart, const double *__restrict__ cpart,
                                                   const int32_t *__restrict__ row_off,
-                                                  const int32_t *__restrict__ col_off, int q0, int q1,
-                                                  int rbase, int cbase, tod_rng rng, int mode, double *g_out,
-                                                  double *mu_out, double *sig_out, int32_t *status)
+                                                  const int32_t *__restrict__ col_off, int q0, int q1, tod_rng rng,
+                                                  int mode, double *g_out, double *mu_out, double *sig_out,
+                                                  int32_t *status)
 {
-    const int q = q0 + blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = q0 + static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (q >= q1) return;
-    double A = 0.0, B = 0.0;
-    for (int i = row_off[q]; i < row_off[q + 1]; ++i) A += rpart[4 * static_cast<int64_t>(i - rbase)];
-    for (int i = col_off[q]; i < col_off[q + 1]; ++i) B += cpart[4 * static_cast<int64_t>(i - cbase) + 1];
+    const double A = item_sum(rpart, row_off[q], row_off[q + 1], 0);
+    const double B = item_sum(cpart, col_off[q], col_off[q + 1], 1);
+    if (threadIdx.x & 31) return;
     if (!(A > 0.0) || !isfinite(A) || !isfinite(B)) {
         set_status(status, q, TOD_ERR_ARG);
         g_out[q] = 0.0;
@@ -991,40 +1004,44 @@ __global__ void __launch_bounds__(TX_T) k_chi2_colsinv(Chi2Tx<V> a)
     }
 }
 
-// Per detscan: chi^2 and its PSD-parameter terms from the row items, the
-// gain derivative from the column items (item order).
+// Per detscan (one warp): chi^2 and its PSD-parameter terms from the row
+// items, the gain derivative from the column items.
 __global__ void __launch_bounds__(256) k_chi2_fin(const double *__restrict__ rpart, const double *__restrict__ cpart,
                                                   const int32_t *__restrict__ row_off,
-                                                  const int32_t *__restrict__ col_off, int q0, int q1, int rbase,
-                                                  int cbase, double *chi2_q, double *dgain, double *dpsd_q)
+                                                  const int32_t *__restrict__ col_off, int q0, int q1,
+                                                  double *chi2_q, double *dgain, double *dpsd_q)
 {
-    const int q = q0 + blockIdx.x * blockDim.x + threadIdx.x;
+    const int q = q0 + static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (q >= q1) return;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = row_off[q]; i < row_off[q + 1]; ++i)
-        for (int k = 0; k < 4; ++k) s[k] += rpart[4 * static_cast<int64_t>(i - rbase) + k];
-    double g = 0.0;
-    for (int i = col_off[q]; i < col_off[q + 1]; ++i) g += cpart[4 * static_cast<int64_t>(i - cbase) + 1];
+    double s[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = item_sum(rpart, row_off[q], row_off[q + 1], k);
+    const double g = item_sum(cpart, col_off[q], col_off[q + 1], 1);
+    if (threadIdx.x & 31) return;
     chi2_q[q] = s[0];
     dgain[q] = g;
     for (int k = 0; k < 3; ++k) dpsd_q[3 * static_cast<int64_t>(q) + k] = s[k + 1];
 }
 
-// Band totals in detscan order (one thread): chi^2 and the PSD gradient of
-// every detector.
-__global__ void k_chi2_total(const double *__restrict__ chi2_q, const double *__restrict__ dpsd_q, int nq, int ndet,
-                             double *total, double *dpsd_det)
+// Band totals, one CTA each in a fixed order (strided lanes, then a tree):
+// chi^2 (CTA 0) and the PSD gradient of every detector (CTA 1 + det).  One
+// thread adding 800 detscans, and 200 for each of 12 derivatives, took 225 us.
+__global__ void __launch_bounds__(256) k_chi2_total(const double *__restrict__ chi2_q,
+                                                    const double *__restrict__ dpsd_q, int nq, int ndet,
+                                                    double *total, double *dpsd_det)
 {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    double t = 0.0;
-    for (int q = 0; q < nq; ++q) t += chi2_q[q];
-    total[0] = t;
-    for (int det = 0; det < ndet; ++det)
-        for (int k = 0; k < 3; ++k) {
-            double s = 0.0;
-            for (int q = det; q < nq; q += ndet) s += dpsd_q[3 * static_cast<int64_t>(q) + k];
-            dpsd_det[3 * det + k] = s;
-        }
+    __shared__ double s_red[3 * (TX_T / 32)], s_out[3];
+    double t[3] = {0.0, 0.0, 0.0};
+    if (blockIdx.x == 0) {
+        for (int q = threadIdx.x; q < nq; q += TX_T) t[0] += chi2_q[q];
+    } else {
+        for (int q = static_cast<int>(blockIdx.x) - 1 + ndet * static_cast<int>(threadIdx.x); q < nq; q += ndet * TX_T)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) t[k] += dpsd_q[3 * static_cast<int64_t>(q) + k];
+    }
+    block_sums_d<3>(t, s_red, s_out);
+    if (blockIdx.x == 0) { if (threadIdx.x == 0) total[0] = s_out[0]; }
+    else if (threadIdx.x < 3) dpsd_det[3 * (blockIdx.x - 1) + threadIdx.x] = s_out[threadIdx.x];
 }
 
 // ===========================================================================
@@ -2426,8 +2443,8 @@ cudaError_t launch_tx_gain(const Plan &p, const float *d, const float *s, const 
     }
     {
         KTIME(TOD_KT_GAIN_FIN);
-        k_gain_fin<<<(q1 - q0 + 255) / 256, 256, 0, st>>>(rpart, cpart, p.row_off, p.col_off, q0, q1, 0, 0, rng, mode,
-                                                          g, mu, sig, p.status);
+        k_gain_fin<<<(q1 - q0 + 7) / 8, 256, 0, st>>>(rpart, cpart, p.row_off, p.col_off, q0, q1, rng, mode, g, mu, sig,
+                                                      p.status);
     }
     return cudaGetLastError();
 }
@@ -2467,8 +2484,7 @@ static cudaError_t chi2_range(const Plan &p, const float *d, const void *s, cons
     }
     {
         KTIME(TOD_KT_CHI2_FIN);
-        k_chi2_fin<<<(q1 - q0 + 255) / 256, 256, 0, st>>>(rpart, cpart, p.row_off, p.col_off, q0, q1, 0, 0, chi2_q, dgain,
-                                                           dpsd_q);
+        k_chi2_fin<<<(q1 - q0 + 7) / 8, 256, 0, st>>>(rpart, cpart, p.row_off, p.col_off, q0, q1, chi2_q, dgain, dpsd_q);
     }
     return cudaGetLastError();
 }
@@ -2494,7 +2510,7 @@ cudaError_t launch_tx_chi2(const Plan &p, bool fp64, const float *d, const void 
     if (e != cudaSuccess) return e;
     {
         KTIME(TOD_KT_CHI2_FIN);
-        k_chi2_total<<<1, 1, 0, st>>>(chi2_q, dpsd_q, p.nq, p.ndet, total, dpsd_det);
+        k_chi2_total<<<1 + p.ndet, TX_T, 0, st>>>(chi2_q, dpsd_q, p.nq, p.ndet, total, dpsd_det);
     }
     return cudaGetLastError();
 }
