@@ -470,7 +470,8 @@ bool valid_streams(const tod_huff_streams &h, int64_t nq, int64_t nscan, const s
 cudaError_t build_huff(Plan &p, HuffDev &d, const tod_huff_streams &h)
 {
     cudaError_t e;
-    std::vector<uint32_t> words(h.nwords + 4, 0u);
+    d.nchunks = (h.nwords + 7) / 4;
+    std::vector<uint32_t> words(4 * d.nchunks, 0u);
     std::memcpy(words.data(), h.words, sizeof(uint32_t) * h.nwords);
     if ((e = dev_upload(p, d.words, words.data(), words.size()))) return e;
     if ((e = dev_upload(p, d.word_off, h.word_off, p.nq + 1))) return e;

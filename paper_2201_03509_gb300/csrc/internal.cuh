@@ -10,8 +10,8 @@ namespace tg {
 
 constexpr int DEC_LUTB = 13;          // first-level decode table: 2^13 packed 32-bit entries
 constexpr int32_t DEC_WIDE = -(1 << 26);   // table value: symbol too wide for the entry, read canonically
-constexpr int DEC_T = 512;            // decode threads per CTA (one checkpoint block each)
-constexpr int DEC_ROUND = 16;         // symbols staged per thread before a coalesced write
+constexpr int DEC_T = 256;            // decode threads per CTA (one checkpoint block each)
+constexpr int DEC_ROUND = 16;         // symbols staged per thread before a write of whole sectors
 // what a decoded value becomes: itself (pointing), the FP32 TOD, a flag bit
 enum : int { DEC_VALUE = 0, DEC_TOD = 1, DEC_FLAG = 2 };
 constexpr int ELEM_TILE = 4096;       // samples per tile of the element-wise kernels
@@ -20,7 +20,8 @@ constexpr int BIN_TILE = 2048;        // sorted samples staged per binning tile
 
 // Compressed stream kind, device copy + decode tables.
 struct HuffDev {
-    uint32_t *words = nullptr;       // + 2 zero pad words
+    uint32_t *words = nullptr;       // + zero pad words to a whole 16-byte chunk and one more
+    int64_t nchunks = 0;
     int64_t *word_off = nullptr;     // [nq+1]
     int64_t *nbits = nullptr;        // [nq]
     int64_t *blk_off = nullptr;      // [nq+1]

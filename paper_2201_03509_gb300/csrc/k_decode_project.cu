@@ -6,19 +6,32 @@
 // up to DEC_T consecutive blocks of one scan and stages that scan's code
 // (a 2^DEC_LUTB-entry first-level table, per-length limits for the long
 // codes) in shared memory; the rare long codes read their symbol through
-// the cache.  Each thread's decode is one long dependency chain, so the
-// CTA is large (the table is staged once for more threads) and three fit
-// on an SM.  Values are undone
-// from their differences on the fly and staged DEC_ROUND at a time per
-// thread in shared memory, then written with coalesced stores.
+// the cache.  Values are undone from their differences on the fly, staged
+// DEC_ROUND at a time per thread in shared memory, and written by their own
+// warp in pairs (no CTA barrier after the table is staged).
+//
+// A block is one long dependency chain, and what it waits for decides the
+// speed.  Threads run out of bits at different symbols, so a load of the next
+// word where it is needed stalls the warp at nearly every symbol for a trip
+// to L2.  Each thread's words come through a ring of four 16-byte chunks in
+// shared memory instead, filled by asynchronous copies two groups of symbols
+// ahead (a group of DEC_GROUP symbols takes less than one chunk, 24 bits each
+// at most, so one copy per group keeps the ring full); and a symbol takes no
+// branch but those to a refill and to the long codes, whose symbols are staged
+// in shared memory too when a scan has at most DEC_CANON of them (30 % of the
+// 70 GHz pixel symbols are longer than the table).  27M samples of pointing:
+// 474 -> 268 us; of TOD 305 -> 232, of flags 149 -> 73 us; 65k samples 111 -> 63 us
+// a stream; 102M samples of 70 GHz pointing 1972 -> 784 us.  A symbol's chain of
+// dependent operations is the bound.  (Asking L2 for a block's lines at its
+// start cost 15 %, a ring of eight chunks gained nothing.)
 //
 // The same decoder serves the TOD and quality-flag streams (Sect. 4.1:
 // the ADC integers and flag words are differenced and coded like the
 // pointing; Listing `tod`: tod and flag held as compressed bytes).  What a
 // decoded value becomes is the kernel's KIND: the value itself (pointing),
-// the FP32 TOD d = fl32(scale_q * count) (one FP64 product, one rounding),
-// or the flag bit (word & select) != 0, packed into the sample bitmask with
-// one warp vote and at most two atomic ORs per DEC_ROUND samples.
+// the FP32 TOD d = fl32(scale_q * count) (the FP64 product, rounded once),
+// or the flag bit (word & select) != 0, collected per DEC_ROUND samples and
+// ORed into the sample bitmask with at most two atomics.
 #include <type_traits>
 
 #include "common.cuh"
@@ -26,11 +39,34 @@
 
 namespace tg {
 
-static_assert(DEC_ROUND == 16, "the flag packing takes two runs of 16 samples per warp");
+constexpr int DEC_GROUP = 4;                  // symbols between two refills of the ring
+constexpr int DEC_CANON = 8192;               // most symbols of a code staged in shared memory
+constexpr int DEC_RING = 16;                  // words of a thread's ring (four chunks)
+constexpr int DEC_RSTRIDE = DEC_RING + 4;     // its stride, 16-byte aligned
+static_assert(DEC_ROUND % DEC_GROUP == 0 && DEC_GROUP * TOD_HUFF_MAXLEN < 128, "a group takes less than a chunk");
+static_assert(DEC_ROUND == 16 && TOD_CKPT_BLOCK % DEC_ROUND == 0, "flags are packed 16 at a time");
+static_assert((1 << DEC_LUTB) % (4 * DEC_T) == 0, "the table is staged 16 bytes a thread");
+
+// fl32 of the FP64 product c * scale (scale = s1 + s2 + ..., FP32 parts) in
+// FP32: the product as head + tail to about 2^-46, rounded; where that lies
+// too near a rounding boundary to be sure (or out of the easy range), the
+// FP64 product itself (FP64 issues at 1/64 of the FP32 rate here).
+__device__ __forceinline__ float tod_value(int32_t c, float s1, float s2, double scale) {
+    const float fc = static_cast<float>(c);
+    const float ph = __fmul_rn(fc, s1);
+    const float l = __fadd_rn(__fmaf_rn(fc, s1, -ph), __fmul_rn(fc, s2));
+    const float r = __fadd_rn(ph, l);
+    const float e = fabsf(__fsub_rn(l, __fsub_rn(r, ph)));       // distance to the rounded value
+    const uint32_t rb = __float_as_uint(r);
+    const float half = __uint_as_float(rb & 0x7f800000u) * 5.9604644775390625e-08f;    // half an ulp of r
+    const bool sure = c == 0 || (e < 0.9999f * half && (rb & 0x7fffffu) != 0u && abs(c) < (1 << 24) &&
+                                 fabsf(r) > 1e-25f && fabsf(r) < 1e25f);
+    return sure ? r : __double2float_rn(static_cast<double>(c) * scale);
+}
 
 template <typename OutT, int KIND>
 __global__ void __launch_bounds__(DEC_T)
-k_decode(const uint32_t *__restrict__ words, const int64_t *__restrict__ word_off,
+k_decode(const uint32_t *__restrict__ words, int64_t nchunks, const int64_t *__restrict__ word_off,
          const int64_t *__restrict__ nbits, const int64_t *__restrict__ blk_off,
          const uint32_t *__restrict__ ckpt_bit, const int32_t *__restrict__ ckpt_val,
          const int32_t *__restrict__ blk_q, const int32_t *__restrict__ lut,
@@ -38,66 +74,110 @@ k_decode(const uint32_t *__restrict__ words, const int64_t *__restrict__ word_of
          const int32_t *__restrict__ canon_off, const int32_t *__restrict__ canon_vals,
          const int32_t *__restrict__ cta_scan, const int64_t *__restrict__ cta_blk0,
          const int32_t *__restrict__ cta_nblk, const int64_t *__restrict__ off,
-         const double *__restrict__ scale, uint32_t select, OutT *__restrict__ out, int32_t *status)
+         const double *__restrict__ scale, uint32_t select, bool staged, OutT *__restrict__ out, bool pairs,
+         int32_t *status)
 {
-    using StageT = typename std::conditional<KIND == DEC_FLAG, uint8_t, OutT>::type;
-    extern __shared__ int32_t s_lut[];                     // [1 << DEC_LUTB]
+    struct alignas(2 * sizeof(OutT)) Pair { OutT a, b; };
+    constexpr int TS = DEC_ROUND / 2 + 1;                  // pairs per thread of the tile, odd
+    extern __shared__ __align__(16) int32_t s_lut[];       // [1 << DEC_LUTB], then the rings
+    uint32_t *s_ring = reinterpret_cast<uint32_t *>(s_lut + (1 << DEC_LUTB));
     __shared__ unsigned long long s_lim[26];
     __shared__ int32_t s_base[26];
-    __shared__ StageT s_tile[DEC_T][DEC_ROUND + 1];
+    __shared__ Pair s_tile[KIND == DEC_FLAG ? 1 : DEC_T * TS];
     __shared__ int64_t s_out0[DEC_T];
     __shared__ int32_t s_cnt[DEC_T];
 
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, w32 = tid & ~31;
     const int scan = cta_scan[blockIdx.x];
     const int64_t b0 = cta_blk0[blockIdx.x];
     const int nb = cta_nblk[blockIdx.x];
 
-    for (int i = tid; i < (1 << DEC_LUTB); i += DEC_T) s_lut[i] = lut[(int64_t)scan * (1 << DEC_LUTB) + i];
+    {
+        const int4 *src = reinterpret_cast<const int4 *>(lut + (static_cast<int64_t>(scan) << DEC_LUTB));
+        int4 *dst = reinterpret_cast<int4 *>(s_lut);
+#pragma unroll
+        for (int i = 0; i < (1 << DEC_LUTB) / (4 * DEC_T); ++i) dst[tid + i * DEC_T] = src[tid + i * DEC_T];
+    }
     if (tid < 26) { s_lim[tid] = lim_g[scan * 26 + tid]; s_base[tid] = base_g[scan * 26 + tid]; }
-    // symbols of long codes (longer than DEC_LUTB bits: rare) through the cache
+    // symbols of long codes (longer than DEC_LUTB bits)
     const int c0 = canon_off[scan], nc = canon_off[scan + 1] - c0;
+    int32_t *s_canon = reinterpret_cast<int32_t *>(s_ring + DEC_T * DEC_RSTRIDE);
+    if (staged)
+        for (int i = tid; i < nc; i += DEC_T) s_canon[i] = __ldg(canon_vals + c0 + i);
+    const int32_t *canon = staged ? s_canon : canon_vals + c0;
 
     // this thread's block
-    const bool active = tid < nb;
     int q = 0, cnt = 0;
-    int64_t pos = 0, end = 0, wptr = 0;
+    int64_t end = 0, out0 = 0;
     int32_t x = 0;
     double sc = 0.0;                    // DEC_TOD: the detscan's ADC quantum
-    unsigned long long buf = 0;
-    int have = 0;                       // valid bits in buf (left-aligned)
+    float s1 = 0.f, s2 = 0.f;
+    uint32_t hi = 0, lo = 0;            // the next bits, left-aligned
+    int have = 64;                      // valid bits in hi:lo
+    int64_t chunk0 = 0;                 // first chunk of the ring's numbering
+    int wi = 0, fetched = 0;            // next word, next chunk to copy, relative to chunk0
     bool ok = true;
-    if (active) {
+    uint32_t *ring = s_ring + tid * DEC_RSTRIDE;
+    const auto fetch = [&]() {          // the next chunk, once its place is free
+        if (fetched < (wi >> 2) + DEC_RING / 4 && chunk0 + fetched < nchunks) {
+            const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(ring + 4 * (fetched & (DEC_RING / 4 - 1))));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(words + 4 * (chunk0 + fetched)) : "memory");
+            ++fetched;
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    if (tid < nb) {
         const int64_t b = b0 + tid;
         q = blk_q[b];
         const int64_t j = b - blk_off[q];
         const int64_t n = off[q + 1] - off[q];
         cnt = static_cast<int>((n - j * TOD_CKPT_BLOCK < TOD_CKPT_BLOCK ? n - j * TOD_CKPT_BLOCK : TOD_CKPT_BLOCK));
-        s_out0[tid] = off[q] + j * TOD_CKPT_BLOCK;
-        s_cnt[tid] = cnt;
-        const int64_t w0 = word_off[q];
-        pos = w0 * 32 + ckpt_bit[b];
-        end = w0 * 32 + nbits[q];
+        out0 = off[q] + j * TOD_CKPT_BLOCK;
+        const int64_t w0 = word_off[q] * 32;
+        const int64_t pos = w0 + ckpt_bit[b];
+        end = w0 + nbits[q];
         x = ckpt_val[b];
-        if constexpr (KIND == DEC_TOD) sc = scale[q];
-        wptr = pos >> 5;
+        if constexpr (KIND == DEC_TOD) {
+            sc = scale[q];
+            s1 = static_cast<float>(sc);
+            s2 = static_cast<float>(sc - static_cast<double>(s1));
+        }
+        chunk0 = pos >> 7;
+        wi = static_cast<int>((pos >> 5) & 3);
+#pragma unroll
+        for (int i = 0; i < DEC_RING / 4; ++i) fetch();
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
         const int sh = static_cast<int>(pos & 31);
-        buf = ((static_cast<unsigned long long>(words[wptr]) << 32) | words[wptr + 1]) << sh;
+        const uint32_t a = ring[wi], c = ring[wi + 1];
+        hi = __funnelshift_l(c, a, sh);
+        lo = c << sh;
         have = 64 - sh;
-        wptr += 2;
-    } else {
-        s_cnt[tid] = 0;
-        s_out0[tid] = 0;
+        wi += 2;
     }
+    s_cnt[tid] = cnt;
+    s_out0[tid] = out0;
+    uint32_t nw = ring[wi & (DEC_RING - 1)];               // the word after hi:lo
     __syncthreads();
+    // the limits of the first lengths past the table
+    constexpr int NL = 4;
+    unsigned long long lim[NL];
+#pragma unroll
+    for (int l = 0; l < NL; ++l) lim[l] = s_lim[DEC_LUTB + 1 + l];
 
     for (int round = 0; round < TOD_CKPT_BLOCK / DEC_ROUND; ++round) {
-#pragma unroll 4
-        for (int i = 0; i < DEC_ROUND; ++i) {
-            const int idx = round * DEC_ROUND + i;
-            if (active && ok && idx < cnt) {
-                const uint32_t peek = static_cast<uint32_t>(buf >> 32);
-                const int32_t e = s_lut[peek >> (32 - DEC_LUTB)];
+        uint32_t bits = 0;
+#pragma unroll
+        for (int g = 0; g < DEC_ROUND / DEC_GROUP; ++g) {
+            if (cnt > 0) fetch();
+            else asm volatile("cp.async.commit_group;\n" ::: "memory");
+            // every chunk but the last two copies' has arrived: the current
+            // chunk and the next, more than a group can take
+            asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+            OutT val[DEC_GROUP];
+#pragma unroll
+            for (int i = 0; i < DEC_GROUP; ++i) {
+                const int idx = round * DEC_ROUND + g * DEC_GROUP + i;
+                const int32_t e = s_lut[hi >> (32 - DEC_LUTB)];
                 int len = e & 31;
                 int32_t v = e >> 5;
                 if (len == 0 || v == DEC_WIDE) {
@@ -107,64 +187,83 @@ k_decode(const uint32_t *__restrict__ words, const int64_t *__restrict__ word_of
                     int L = len;
                     if (len == 0) {
                         L = DEC_LUTB + 1;
-                        while (L <= TOD_HUFF_MAXLEN && static_cast<unsigned long long>(peek) >= s_lim[L]) ++L;
+#pragma unroll
+                        for (int l = 0; l < NL; ++l) L += hi >= lim[l];
+                        if (L == DEC_LUTB + 1 + NL)
+                            while (L <= TOD_HUFF_MAXLEN && static_cast<unsigned long long>(hi) >= s_lim[L]) ++L;
                     }
-                    if (L > TOD_HUFF_MAXLEN) { ok = false; len = 1; v = 0; }
-                    else {
-                        const int ci = s_base[L] + static_cast<int>(peek >> (32 - L));
-                        if (ci < 0 || ci >= nc) { ok = false; v = 0; }
-                        else v = __ldg(canon_vals + c0 + ci);
+                    const int ci = L > TOD_HUFF_MAXLEN ? -1 : s_base[L] + static_cast<int>(hi >> (32 - L));
+                    if (ci < 0 || ci >= nc) {
+                        if (idx < cnt) ok = false;
+                        v = 0;
+                        len = L > TOD_HUFF_MAXLEN ? 1 : L;
+                    } else {
+                        v = canon[ci];
                         len = L;
                     }
                 }
+                if (idx >= cnt) { len = 0; v = 0; }         // past a short block: nothing more is taken
                 x += v;
-                buf <<= len;
+                hi = __funnelshift_l(lo, hi, len);
+                lo <<= len;
                 have -= len;
-                pos += len;
-                if (pos > end) ok = false;       // never read past the stream (+pad)
-                if (ok && have < 32) {
-                    buf |= static_cast<unsigned long long>(words[wptr]) << (32 - have);
-                    ++wptr;
-                    have += 32;
-                }
-                if constexpr (KIND == DEC_TOD)
-                    s_tile[tid][i] = __double2float_rn(static_cast<double>(x) * sc);
-                else if constexpr (KIND == DEC_FLAG)
-                    s_tile[tid][i] = (static_cast<uint32_t>(x) & select) != 0u;
-                else
-                    s_tile[tid][i] = static_cast<OutT>(x);
+                // 8 <= have: codes have at most 24 bits
+                const bool need = have < 32;
+                hi |= need ? nw >> (have & 31) : 0u;
+                lo = need ? nw << (32 - have & 31) : lo;
+                have += need ? 32 : 0;
+                if (need) { ++wi; nw = ring[wi & (DEC_RING - 1)]; }
+                if constexpr (KIND == DEC_TOD) val[i] = tod_value(x, s1, s2, sc);
+                else if constexpr (KIND == DEC_FLAG) {
+                    if (idx < cnt && (static_cast<uint32_t>(x) & select) != 0u) bits |= 1u << (g * DEC_GROUP + i);
+                } else val[i] = static_cast<OutT>(x);
+            }
+            if constexpr (KIND != DEC_FLAG) {
+#pragma unroll
+                for (int i = 0; i < DEC_GROUP; i += 2)
+                    s_tile[tid * TS + (g * DEC_GROUP + i) / 2] = Pair{val[i], val[i + 1]};
             }
         }
-        __syncthreads();
-        // coalesced write-out: consecutive threads take consecutive values of a block
-        for (int e = tid; e < DEC_T * DEC_ROUND; e += DEC_T) {
-            const int bl = e / DEC_ROUND, i = e % DEC_ROUND;
-            const int idx = round * DEC_ROUND + i;
-            if constexpr (KIND == DEC_FLAG) {
-                // lanes 0-15 and 16-31 each hold DEC_ROUND consecutive samples
-                // of one block; their flagged bits are ORed into the bitmask
-                // (bit t & 31 of word t >> 5; the words start zeroed)
-                const uint32_t vote =
-                    __ballot_sync(0xffffffffu, idx < s_cnt[bl] && s_tile[bl][i] != 0);
-                const uint32_t mine = (vote >> (tid & 31 & ~(DEC_ROUND - 1))) & 0xffffu;
-                if (i == 0 && mine) {
-                    const int64_t g0 = s_out0[bl] + round * DEC_ROUND;
-                    const unsigned long long v = static_cast<unsigned long long>(mine) << (g0 & 31);
-                    atomicOr(out + (g0 >> 5), static_cast<uint32_t>(v));
-                    if (v >> 32) atomicOr(out + (g0 >> 5) + 1, static_cast<uint32_t>(v >> 32));
-                }
-            } else {
-                if (idx < s_cnt[bl]) out[s_out0[bl] + idx] = s_tile[bl][i];
+        if constexpr (KIND == DEC_FLAG) {
+            // DEC_ROUND consecutive samples' flags into the bitmask (bit
+            // t & 31 of word t >> 5; the words start zeroed)
+            if (bits) {
+                const int64_t g0 = out0 + round * DEC_ROUND;
+                const unsigned long long v = static_cast<unsigned long long>(bits) << (g0 & 31);
+                atomicOr(out + (g0 >> 5), static_cast<uint32_t>(v));
+                if (v >> 32) atomicOr(out + (g0 >> 5) + 1, static_cast<uint32_t>(v >> 32));
             }
+        } else {
+            // the warp's values: eight lanes a block, two values each
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < DEC_ROUND / 2; ++k) {
+                const int bl = w32 + 4 * k + (lane >> 3), pi = lane & 7;
+                const int idx = round * DEC_ROUND + 2 * pi;
+                const Pair v = s_tile[bl * TS + pi];
+                OutT *o = out + s_out0[bl] + idx;
+                const int left = s_cnt[bl] - idx;
+                if (pairs && left >= 2) *reinterpret_cast<Pair *>(o) = v;
+                else {
+                    if (left >= 1) o[0] = v.a;
+                    if (left >= 2) o[1] = v.b;
+                }
+            }
+            __syncwarp();
         }
-        __syncthreads();
     }
-    if (active && (!ok || pos > end)) set_status(status, q, TOD_ERR_CORRUPT_STREAM);
+    // the bits taken: the next word's place less what is still in hi:lo
+    if (cnt > 0 && (!ok || (chunk0 * 4 + wi) * 32 - have > end)) set_status(status, q, TOD_ERR_CORRUPT_STREAM);
+}
+
+// shared memory of a launch: the table, the rings, and the symbols when staged
+static size_t dec_smem(int canon) {
+    return sizeof(int32_t) * ((1 << DEC_LUTB) + DEC_T * DEC_RSTRIDE + (canon <= DEC_CANON ? (canon + 3 & ~3) : 0));
 }
 
 cudaError_t setup_decode_kernel()
 {
-    const int smem = static_cast<int>(sizeof(int32_t) * (1 << DEC_LUTB));
+    const int smem = static_cast<int>(dec_smem(DEC_CANON));
     cudaError_t e = cudaFuncSetAttribute(k_decode<int32_t, DEC_VALUE>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
@@ -187,12 +286,14 @@ cudaError_t decode_into(const Plan &p, const HuffDev &h, const double *scale, ui
                         cudaStream_t st)
 {
     if (h.ncta == 0) return cudaSuccess;
-    const size_t smem = sizeof(int32_t) * (1 << DEC_LUTB);
+    // pairs of values: every detscan starts at an even sample
+    const bool pairs = (reinterpret_cast<uintptr_t>(out) & (2 * sizeof(OutT) - 1)) == 0;
     {
         KTIME(kind_id<KIND>());
-        k_decode<OutT, KIND><<<h.ncta, DEC_T, smem, st>>>(
-            h.words, h.word_off, h.nbits, h.blk_off, h.ckpt_bit, h.ckpt_val, h.blk_q, h.lut, h.lim, h.base,
-            h.canon_off, h.canon_vals, h.cta_scan, h.cta_blk0, h.cta_nblk, p.off, scale, select, out, p.status);
+        k_decode<OutT, KIND><<<h.ncta, DEC_T, dec_smem(h.max_canon), st>>>(
+            h.words, h.nchunks, h.word_off, h.nbits, h.blk_off, h.ckpt_bit, h.ckpt_val, h.blk_q, h.lut, h.lim, h.base,
+            h.canon_off, h.canon_vals, h.cta_scan, h.cta_blk0, h.cta_nblk, p.off, scale, select,
+            h.max_canon <= DEC_CANON, out, pairs, p.status);
     }
     return cudaGetLastError();
 }
