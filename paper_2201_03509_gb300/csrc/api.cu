@@ -784,6 +784,7 @@ tod_status tod_plan_create(tod_plan **out, const tod_band_desc *band)
         if ((e = dev_upload(*p, p->psd_sumlnf, sumlnf.data(), sumlnf.size()))) return fail(e);
         if ((e = dev_upload(*p, p->psd_part, static_cast<double *>(nullptr), static_cast<size_t>(p->ntile))))
             return fail(e);
+        if ((e = dev_upload(*p, p->psd_w, static_cast<double *>(nullptr), static_cast<size_t>(p->nq)))) return fail(e);
         if ((e = dev_upload(*p, p->psd_state, static_cast<double *>(nullptr), static_cast<size_t>(p->ndet) * 8)))
             return fail(e);
     }

@@ -143,6 +143,7 @@ struct Plan {
     double *lnfs = nullptr;          // [nq] ln(fsamp / (2 n_q))
     double *psd_nmodes = nullptr;    // [ndet] modes k >= 1 of the detector's detscans
     double *psd_sumlnf = nullptr;    // [ndet] sum of ln f_k over them
+    double *psd_w = nullptr;         // [nq] e^{-alpha c_q} of the evaluation
     double *psd_part = nullptr;      // [ntile] partial sums of one evaluation
     double *psd_state = nullptr;     // [ndet][8] chain state
     // binning
