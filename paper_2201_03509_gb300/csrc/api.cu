@@ -236,6 +236,9 @@ void free_plan(Plan *p)
     cudaSetDevice(p->device);
     for (void *a : p->allocs) cudaFree(a);
     for (cudaEvent_t ev : p->kt.pool) cudaEventDestroy(ev);
+    if (p->prep_fork) cudaEventDestroy(p->prep_fork);
+    if (p->prep_done) cudaEventDestroy(p->prep_done);
+    if (p->prep_stream) cudaStreamDestroy(p->prep_stream);
     cudaSetDevice(cur);
     delete p;
 }
@@ -524,17 +527,17 @@ cudaError_t build_huff(Plan &p, HuffDev &d, const tod_huff_streams &h)
 // detscan.
 cudaError_t ncorr_draw(const Plan &p, const float *d, const float *s, const double *gain, const uint32_t *flags,
                        const double *psd, tod_rng rng, int mode, float tol, int maxit, float *x, int32_t *iters,
-                       cudaStream_t st)
+                       cudaStream_t st, cudaEvent_t prepared = nullptr)
 {
     const TxNcorrScratch sc = {p.ybuf, p.wpre, p.cgv, p.cgcap};
     if (p.schedule != TOD_SCHED_PER_SCAN)
         return launch_tx_ncorr(p, d, s, gain, flags, psd, rng, mode, tol, maxit, x, iters, st, 0, p.nq, sc,
-                               p.pass_grid);
+                               p.pass_grid, prepared);
     cudaError_t e = cudaSuccess;
     for (int q = 0; q < p.nq && e == cudaSuccess; ++q) {
         const int items = std::max(p.h_col_off[q + 1] - p.h_col_off[q], p.h_row_off[q + 1] - p.h_row_off[q]);
         e = launch_tx_ncorr(p, d, s, gain, flags, psd, rng, mode, tol, maxit, x, iters, st, q, q + 1, sc,
-                            std::min(p.pass_grid, std::max(1, items)));
+                            std::min(p.pass_grid, std::max(1, items)), prepared);
     }
     return e;
 }
@@ -875,6 +878,12 @@ tod_status tod_plan_create(tod_plan **out, const tod_band_desc *band)
         if ((e = dev_upload(*p, p->col_off, p->h_col_off.data(), p->h_col_off.size()))) return fail(e);
         if ((e = dev_upload(*p, p->row_off, p->h_row_off.data(), p->h_row_off.size()))) return fail(e);
         if ((e = setup_tx_kernels(*p))) return fail(e);
+        // the preparation's side stream: ahead of the draw's passes where both want an SM
+        int least = 0, greatest = 0;
+        if ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest))) return fail(e);
+        if ((e = cudaStreamCreateWithPriority(&p->prep_stream, cudaStreamNonBlocking, greatest))) return fail(e);
+        if ((e = cudaEventCreateWithFlags(&p->prep_fork, cudaEventDisableTiming))) return fail(e);
+        if ((e = cudaEventCreateWithFlags(&p->prep_done, cudaEventDisableTiming))) return fail(e);
         // scratch: the complex intermediate (room for one whole detscan in FP64
         // too), per-item partial sums, the flag prefix, CG state and vectors
         p->ybuf_floats = std::max<int64_t>(p->N, 2 * static_cast<int64_t>(maxlen));
@@ -1289,8 +1298,10 @@ tod_status tod_sample_ncorr(tod_plan *pl, const float *d, const float *s, const 
     DeviceGuard dg(p->device);
     const float tol = cg_tol > 0 ? static_cast<float>(cg_tol) : 1e-6f;
     const int maxit = cg_maxiter > 0 ? cg_maxiter : 500;
-    cudaError_t e = p->use_prec ? launch_toeplitz_prep(*p, psd, stream) : cudaSuccess;
-    if (e == cudaSuccess) e = ncorr_draw(*p, d, s, gain, flags, psd, rng, mode, tol, maxit, ncorr_out, cg_iters_out, stream);
+    cudaError_t e = p->use_prec ? fork_toeplitz_prep(*p, psd, stream) : cudaSuccess;
+    if (e == cudaSuccess)
+        e = ncorr_draw(*p, d, s, gain, flags, psd, rng, mode, tol, maxit, ncorr_out, cg_iters_out, stream,
+                       p->use_prec ? p->prep_done : nullptr);
     return to_status(e);
 }
 

@@ -186,6 +186,10 @@ struct Plan {
     int32_t *nclist = nullptr;       // [3 nq + 3] detscans of a CG pass with their item counts
     double *chi2_dpsd = nullptr;     // [nq][3] per-detscan PSD terms of the chi^2 gradient
     float4 *qsc = nullptr;           // [nq][2] per-detscan FP32 noise scalars of the current call
+    // the n_corr draw's preconditioner preparation runs on prep_stream beside
+    // the draw's first passes (forked from and joined to the caller's stream)
+    cudaStream_t prep_stream = nullptr;
+    cudaEvent_t prep_fork = nullptr, prep_done = nullptr;
     int32_t coop_grid = 0;           // co-resident CTAs of the cooperative n_corr kernel
     int32_t pass_grid = 0;           // persistent grid of the other pass kernels
     int32_t tile_pairs = 0;          // requested column pairs per tile (0 = choose)
@@ -249,16 +253,19 @@ cudaError_t setup_tx_kernels(Plan &p);
 cudaError_t launch_tx_gain(const Plan &p, const float *d, const float *s, const uint32_t *flags, const double *psd,
                            tod_rng rng, int mode, double *g, double *mu, double *sig, cudaStream_t st, int q0, int q1);
 // the draw over detscans [q0, q1): pass kernels with at most `grid` CTAs
-// (at most p.pass_grid), the cooperative tail with at most p.coop_grid
+// (at most p.pass_grid), the cooperative tail with at most p.coop_grid; the
+// preconditioner tables are first read after `prepared` (null: they are ready)
 cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const double *gain,
                             const uint32_t *flags, const double *psd, tod_rng rng, int mode, float tol, int maxit,
                             float *x, int32_t *iters, cudaStream_t st, int q0, int q1, const TxNcorrScratch &sc,
-                            int grid);
+                            int grid, cudaEvent_t prepared = nullptr);
 cudaError_t launch_tx_chi2(const Plan &p, bool fp64, const float *d, const void *s, const double *gain,
                            const uint32_t *flags, const double *psd, double *chi2_q, double *dgain, double *dpsd_q,
                            double *total, double *dpsd_det, void *v_out, cudaStream_t st);
 cudaError_t setup_bin_kernel(Plan &p);
 cudaError_t launch_toeplitz_prep(const Plan &p, const double *psd, cudaStream_t st);
+// the same on the plan's side stream, forked from st: prep_done marks its end
+cudaError_t fork_toeplitz_prep(const Plan &p, const double *psd, cudaStream_t st);
 cudaError_t launch_noise_psd(const Plan &p, const float *spec, const double *psd_in, tod_rng rng, int nsteps,
                              double step_lnfk, double step_al, double *psd_out, int32_t *acc_out,
                              double *loglike_out, cudaStream_t st);

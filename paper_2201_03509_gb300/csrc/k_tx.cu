@@ -1299,7 +1299,8 @@ __device__ void nc_detscan_index(const NcorrTx &a, NcShared &S, int q)
         a.cgs[q] = cs;
         // preconditioner blocks (rank within the detscan, length)
         int nb = 0;
-        const int lmax = (a.xtab && a.lvalid) ? min(TOEP_LMAX, a.lvalid[det]) : 0;
+        // (blocks of TOEP_LMAX: the tables may not be there yet, see nc_resplit)
+        const int lmax = a.xtab ? TOEP_LMAX : 0;
         if (cs.mode == CG_ACTIVE && ngap <= TX_GBMAX && lmax >= 1) {
             int rank = 0;
             for (int g = 0; g < ngap && nb >= 0; ++g)
@@ -1307,7 +1308,7 @@ __device__ void nc_detscan_index(const NcorrTx &a, NcShared &S, int q)
                     const int len = min(lmax, S.gend[g] - b0);
                     if (nb >= TX_GBMAX) { nb = -1; break; }
                     a.gblk[static_cast<int64_t>(q) * TX_GBMAX + nb] = make_int2(rank, len);
-                    if (a.gbpos) a.gbpos[static_cast<int64_t>(q) * TX_GBMAX + nb] = b0;
+                    a.gbpos[static_cast<int64_t>(q) * TX_GBMAX + nb] = b0;
                     ++nb;
                     rank += len;
                 }
@@ -1764,6 +1765,38 @@ __device__ __forceinline__ float2 cz_entry(const float4 *__restrict__ t, int p, 
         ramp = (v.h + v.l) * (1.0f / (0.5f * static_cast<float>(L - 1)));
     }
     return make_float2(I.h + I.l, ramp);
+}
+
+// Cuts detscan q's gaps anew when the tables stop short of TOEP_LMAX (a pivot
+// of the recursion was not positive): blocks of at most lvalid samples, or no
+// preconditioner when there are too many of them or no table at all.
+__device__ void nc_resplit(const NcorrTx &a, int q)
+{
+    if (!a.xtab) return;
+    const int lmax = a.lvalid[q % a.ndet], nb = a.gnb[q];
+    if (lmax >= TOEP_LMAX || nb < 0) return;
+    __shared__ int3 s_old[TX_GBMAX];              // rank, length, first sample
+    int2 *gbl = a.gblk + static_cast<int64_t>(q) * TX_GBMAX;
+    int32_t *pos = a.gbpos + static_cast<int64_t>(q) * TX_GBMAX;
+    for (int b = threadIdx.x; b < nb; b += TX_T) s_old[b] = make_int3(gbl[b].x, gbl[b].y, pos[b]);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int n = lmax >= 1 ? 0 : -1;
+        for (int b = 0; b < nb && n >= 0;) {
+            // a gap: blocks that follow one another without a sample between
+            int e = b + 1, len = s_old[b].y;
+            while (e < nb && s_old[e].z == s_old[b].z + len) len += s_old[e++].y;
+            for (int i = 0; i < len; i += lmax) {
+                if (n >= TX_GBMAX) { n = -1; break; }
+                gbl[n] = make_int2(s_old[b].x + i, min(lmax, len - i));
+                pos[n] = s_old[b].z + i;
+                ++n;
+            }
+            b = e;
+        }
+        a.gnb[q] = n;
+    }
+    __syncthreads();
 }
 
 // Builds the coarse correction of detscan q (after the index phase): S Z
@@ -2238,7 +2271,10 @@ __global__ void __launch_bounds__(TX_T) k_nc_index(NcorrTx a)
 }
 __global__ void __launch_bounds__(TX_T) k_nc_coarse(NcorrTx a)
 {
-    for (int q = a.q0 + blockIdx.x; q < a.q1; q += gridDim.x) nc_coarse_setup(a, q);
+    for (int q = a.q0 + blockIdx.x; q < a.q1; q += gridDim.x) {
+        nc_resplit(a, q);
+        nc_coarse_setup(a, q);
+    }
 }
 __global__ void __launch_bounds__(TX_T, 3) k_nc_rhs_cols(NcorrTx a)
 {
@@ -2518,7 +2554,7 @@ cudaError_t launch_tx_chi2(const Plan &p, bool fp64, const float *d, const void 
 cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const double *gain,
                             const uint32_t *flags, const double *psd, tod_rng rng, int mode, float tol, int maxit,
                             float *x, int32_t *iters, cudaStream_t st, int q0, int q1, const TxNcorrScratch &sc,
-                            int grid)
+                            int grid, cudaEvent_t prepared)
 {
     if (q1 <= q0) return cudaSuccess;
     NcorrTx a = {};
@@ -2550,10 +2586,6 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
         KTIME(TOD_KT_NC_INDEX);
         k_nc_index<<<gq, TX_T, 0, st>>>(a);
     }
-    {
-        KTIME(TOD_KT_NC_COARSE);
-        k_nc_coarse<<<gq, TX_T, 0, st>>>(a);
-    }
     // x0 = B^{-1} b
     {
         KTIME(TOD_KT_NC_RHS_COLS);
@@ -2568,6 +2600,14 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
         k_nc_x0_cols<<<gc, TX_T, s32, st>>>(a);
     }
     // CG on the Schur complement
+    if (prepared) {
+        const cudaError_t ew = cudaStreamWaitEvent(st, prepared, 0);
+        if (ew != cudaSuccess) return ew;
+    }
+    {
+        KTIME(TOD_KT_NC_COARSE);
+        k_nc_coarse<<<gq, TX_T, 0, st>>>(a);
+    }
     {
         KTIME(TOD_KT_NC_CG_INIT);
         k_nc_cg_init<<<gq, TX_T, sgb, st>>>(a);

@@ -74,3 +74,38 @@ def test_kernel_of_every_detector(length):
                              cg_tol=1e-7)
         wl.plan.status()
         assert 1 <= int(its.min()) and int(its.max()) <= 8, (levels, its.tolist())
+
+
+def test_draw_on_other_streams_and_under_capture():
+    """The draw's preparation runs beside its first passes on a stream of the
+    plan: the same bits on the default stream, on another stream with the
+    spectra freed in stream order right after the call, and replayed from a
+    captured graph."""
+    torch = pytest.importorskip("torch")
+    import paper_2201_03509_gb300 as tg
+    from gpu_workload import Workload
+    cfg = synth.scaled(synth.CONFIGS["tiny"], ndet=3, nscan=4, len_lo=9000, len_hi=20000, fsamp=78.8, flag_frac=0.03)
+    wl = Workload(cfg)
+    gain = torch.ones(wl.nq, dtype=torch.float64, device=wl.dev)
+    out = [torch.zeros(wl.N, dtype=torch.float32, device=wl.dev) for _ in range(3)]
+
+    def draw(psd, x):
+        wl.plan.sample_ncorr(wl.t_d, wl.t_s, gain, wl.t_flags, psd, tg.Rng(SEED, BAND, IT), tg.MODE_DRAW, x)
+
+    draw(wl.t_psd, out[0])
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        psd = wl.t_psd.clone()
+        draw(psd, out[1])
+        del psd
+        torch.full((3, 3), float("nan"), dtype=torch.float64, device=wl.dev)      # may take the freed memory
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        draw(wl.t_psd, out[2])
+    g.replay()
+    torch.cuda.synchronize()
+    wl.plan.status()
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
