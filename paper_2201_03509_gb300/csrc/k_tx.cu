@@ -925,8 +925,10 @@ __global__ void __launch_bounds__(TX_T) k_chi2_rows(Chi2Tx<V> a)
         const S d1 = S(2) / sig0, d2 = -s2 * al / fk;
         const int n = X.L.n, m = X.L.m;
         LaneSum<C> sum[4];            // 2 L, dL/dsigma0, dL/dfknee, dL/dalpha
-        // the modes k0, k1 of coefficients r: r / P, their terms added
-        const auto mode_terms = [&](int k0, int k1, int mask, C r) -> C {
+        // the modes k0, k1 of coefficients r: r / P, their terms added; in
+        // FP64 all but ln P (P in the mask's lanes, 1 elsewhere, left in Pm)
+        constexpr bool kF64 = sizeof(S) == sizeof(double);
+        const auto mode_terms = [&](int k0, int k1, int mask, C r, C &Pm) -> C {
             // ln(f/fk) = ln k + ln(fsamp/(2 n fk)); P = s2 (1 + e^{alpha ln(f/fk)})
             const C lr = pset(log(static_cast<S>(max(k0, 1))) + lfs, log(static_cast<S>(max(k1, 1))) + lfs);
             const C pw = pset(exp(al * lr.a), exp(al * lr.b));
@@ -935,14 +937,17 @@ __global__ void __launch_bounds__(TX_T) k_chi2_rows(Chi2Tx<V> a)
             const C rP = pmul(r, iP), r2P = pmul(r, rP);
             const C hh = pmul(pdup<C>(S(0.5)), psub(iP, pmul(r2P, iP)));     // 1/2 (1/P - r^2/P^2)
             const C sp = pmul(pdup<C>(s2), pmul(pw, lr));
-            C t0 = r2P, tl = pset(log(P.a), log(P.b)), t1 = pmul(hh, pmul(P, pdup<C>(d1)));
+            C t0 = r2P, tl, t1 = pmul(hh, pmul(P, pdup<C>(d1)));
             C t2 = pmul(hh, pmul(pw, pdup<C>(d2))), t3 = pmul(hh, sp);
+            if constexpr (kF64) Pm = mask == 3 ? P : pset((mask & 1) ? P.a : S(1), (mask & 2) ? P.b : S(1));
+            else tl = pset(log(P.a), log(P.b));
             if (mask != 3) {
-                t0 = pmask(t0, mask); tl = pmask(tl, mask); t1 = pmask(t1, mask);
+                t0 = pmask(t0, mask); t1 = pmask(t1, mask);
                 t2 = pmask(t2, mask); t3 = pmask(t3, mask);
+                if constexpr (!kF64) tl = pmask(tl, mask);
             }
             sum[0].add(t0);
-            sum[0].add(tl);
+            if constexpr (!kF64) sum[0].add(tl);
             sum[1].add(t1);
             sum[2].add(t2);
             sum[3].add(t3);
@@ -950,8 +955,22 @@ __global__ void __launch_bounds__(TX_T) k_chi2_rows(Chi2Tx<V> a)
         };
         row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, [](V *) {}, [&](int k0, int k1, int mask, V Rv, V) {
             const int on = (k0 ? 1 : 0) | (k1 ? 2 : 0);         // the offset mode does not enter
-            const C x = mode_terms(k0, k1, mask & on, Rv.x);
-            const C y = mode_terms(k0 ? n - k0 : m, k1 ? n - k1 : m, mask, Rv.y);
+            C P0, P1;
+            const C x = mode_terms(k0, k1, mask & on, Rv.x, P0);
+            const C y = mode_terms(k0 ? n - k0 : m, k1 ? n - k1 : m, mask, Rv.y, P1);
+            if constexpr (kF64) {
+                // one logarithm for the four modes (an FP64 one takes about 30
+                // operations, at 1/64 of the FP32 rate: 25 scans of 4 x 65536,
+                // rows 2168 -> 1815 us) of the product, which leaves the range
+                // only past 1e72 a mode: then one each
+                const S pr = (P0.a * P0.b) * (P1.a * P1.b);
+                if (pr > S(1e-290) && pr < S(1e290)) {
+                    sum[0].add(pset(log(pr), S(0)));
+                } else {
+                    sum[0].add(pset(log(P0.a), log(P0.b)));
+                    sum[0].add(pset(log(P1.a), log(P1.b)));
+                }
+            }
             return vmake<V>(on == 3 ? x : pmask(x, on), y);
         });
         const double acc[4] = {0.5 * sum[0].total(), sum[1].total(), sum[2].total(), sum[3].total()};
