@@ -191,7 +191,8 @@ struct Plan {
     cudaStream_t prep_stream = nullptr;
     cudaEvent_t prep_fork = nullptr, prep_done = nullptr;
     int32_t coop_grid = 0;           // co-resident CTAs of the cooperative n_corr kernel
-    int32_t pass_grid = 0;           // persistent grid of the other pass kernels
+    int32_t pass_grid = 0;           // persistent grid of the row passes and the CG kernels
+    int32_t sm_count = 0;
     int32_t tile_pairs = 0;          // requested column pairs per tile (0 = choose)
     int64_t device_bytes = 0;
     std::vector<void *> allocs;

@@ -210,6 +210,12 @@ __device__ __forceinline__ int y_plane(int m1, int p) { return (m1 & 1) ? 2 * (p
 // elements j1 and m1-1-j1.
 // ---------------------------------------------------------------------------
 constexpr int TX_ROWS = 4;
+// CTAs per SM of the column passes and the chi^2 passes: at three (80
+// registers) the four rows of loads that a thread keeps in flight spill; two
+// at 128 registers are faster but for the scatter, which loads only flags
+// (82M samples: k_gain_cols 359 -> 343 us, k_nc_gather_final 476 -> 418; chi^2 rows of 52M
+// 1093 -> 840 us, there with a grid that is resident at once).
+constexpr int TX_CTAS_COL = 2;
 struct ColThread {
     int m, m1, m2, TP, np, i, c, c2, r0, rstep, m1h;
     __device__ __forceinline__ ColThread(const TxLen &L, int blk) {
@@ -342,10 +348,9 @@ __device__ __forceinline__ void col_forward(const TxCtx &X, V *b0, V *b1, typena
 
 // Inverse column pass: the tile's Y values (every load of a thread in
 // flight), the conjugate twiddle, inverse FFT of the columns; then for every
-// unit D = ld(j, centre, fb) (UNR rows issued at a time) and
-// out(D, j, centre, v, fb) with v its samples (the flag bits are read while
-// the tile loads).
-template <int UNR, class V, class Ld, class Out>
+// unit out(D, j, centre, v, fb) with v its samples, D = ld(j, centre, fb) issued
+// ahead of the transform (the flag bits are read while the tile loads).
+template <class V, class Ld, class Out>
 __device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
                                             const typename PairOf<V>::Z *__restrict__ Y,
                                             const typename PairOf<V>::Z *__restrict__ twb,
@@ -368,14 +373,14 @@ __device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
             if (p >= C.m1h) break;
             if (p == 0 && (m1 & 1)) {
                 const Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
-                A[r][0] = y[C.c];
-                A[r][1] = y[C.c2];
+                A[r][0] = __ldcg(&y[C.c]);
+                A[r][1] = __ldcg(&y[C.c2]);
             } else {
                 const Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
-                A[r][0] = y[C.c];
-                A[r][1] = y[C.c2];
-                A[r][2] = y[m2 + C.c];
-                A[r][3] = y[m2 + C.c2];
+                A[r][0] = __ldcg(&y[C.c]);
+                A[r][1] = __ldcg(&y[C.c2]);
+                A[r][2] = __ldcg(&y[m2 + C.c]);
+                A[r][3] = __ldcg(&y[m2 + C.c2]);
             }
         }
         fnib = unit_flags(C, fl, X.o);
@@ -400,37 +405,37 @@ __device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
             w = vmul(w, wstep);
         }
     }
+    // the units' loads, in flight through the transform
+    decltype(ld(0, false, 0u)) D[TX_ROWS][2];
+    if (C.c >= 0) {
+#pragma unroll
+        for (int r = 0; r < TX_ROWS; ++r) {
+            const int j1 = C.row(r);
+            if (j1 >= C.m1h) continue;
+            const uint32_t fb = fnib >> (8 * r);
+            D[r][0] = ld(j1 * m2 + C.c, C.centre(j1), fb & 15u);
+            if (C.second(j1)) D[r][1] = ld(j1 * m2 + C.c2, false, (fb >> 4) & 15u);
+        }
+    }
     __syncthreads();
     V *R = sp_transform<true, TX_T, true>(b0, b1, m1, X.L.s1, X.L.nr1, X.L.lgW, 0, T.tw1);
     if (C.c < 0) return;
 #pragma unroll
-    for (int r1 = 0; r1 < TX_ROWS; r1 += UNR) {
-        decltype(ld(0, false, 0u)) D[UNR][2];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const int j1 = C.row(r1 + u);
-            if (j1 >= C.m1h) continue;
-            const uint32_t fb = fnib >> (8 * (r1 + u));
-            D[u][0] = ld(j1 * m2 + C.c, C.centre(j1), fb & 15u);
-            if (C.second(j1)) D[u][1] = ld(j1 * m2 + C.c2, false, (fb >> 4) & 15u);
+    for (int r = 0; r < TX_ROWS; ++r) {
+        const int j1 = C.row(r);
+        if (j1 >= C.m1h) continue;
+        const uint32_t fb = fnib >> (8 * r);
+        const V ea = sld(R + j1 * TP + C.i), eb = sld(R + (m1 - 1 - j1) * TP + C.i);
+        if (C.centre(j1)) {
+            const S v[4] = {ea.x.a, ea.y.a, S(0), S(0)};
+            out(D[r][0], j1 * m2 + C.c, true, v, fb & 15u);
+        } else {
+            const S v[4] = {ea.x.a, eb.y.b, ea.y.a, eb.x.b};
+            out(D[r][0], j1 * m2 + C.c, false, v, fb & 15u);
         }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const int j1 = C.row(r1 + u);
-            if (j1 >= C.m1h) continue;
-            const uint32_t fb = fnib >> (8 * (r1 + u));
-            const V ea = sld(R + j1 * TP + C.i), eb = sld(R + (m1 - 1 - j1) * TP + C.i);
-            if (C.centre(j1)) {
-                const S v[4] = {ea.x.a, ea.y.a, S(0), S(0)};
-                out(D[u][0], j1 * m2 + C.c, true, v, fb & 15u);
-            } else {
-                const S v[4] = {ea.x.a, eb.y.b, ea.y.a, eb.x.b};
-                out(D[u][0], j1 * m2 + C.c, false, v, fb & 15u);
-            }
-            if (C.second(j1)) {
-                const S v[4] = {ea.x.b, eb.y.a, ea.y.b, eb.x.a};
-                out(D[u][1], j1 * m2 + C.c2, false, v, (fb >> 4) & 15u);
-            }
+        if (C.second(j1)) {
+            const S v[4] = {ea.x.b, eb.y.a, ea.y.b, eb.x.a};
+            out(D[r][1], j1 * m2 + C.c2, false, v, (fb >> 4) & 15u);
         }
     }
 }
@@ -678,7 +683,7 @@ __device__ __forceinline__ Acc2 pacc_total(const PAcc &a) { return acc_merge_tx(
 __device__ __forceinline__ PF pmask(PF v, int mask) { return PF{(mask & 1) ? v.a : 0.f, (mask & 2) ? v.b : 0.f}; }
 __device__ __forceinline__ PD pmask(PD v, int mask) { return PD{(mask & 1) ? v.a : 0.0, (mask & 2) ? v.b : 0.0}; }
 
-__global__ void __launch_bounds__(TX_T, 3) k_gain_cols(GainTx a)
+__global__ void __launch_bounds__(TX_T, TX_CTAS_COL) k_gain_cols(GainTx a)
 {
     extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
@@ -728,7 +733,7 @@ __global__ void __launch_bounds__(TX_T, 3) k_gain_rows(GainTx a)
     }
 }
 
-__global__ void __launch_bounds__(TX_T, 3) k_gain_colsinv(GainTx a)
+__global__ void __launch_bounds__(TX_T, TX_CTAS_COL) k_gain_colsinv(GainTx a)
 {
     extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
@@ -740,7 +745,7 @@ __global__ void __launch_bounds__(TX_T, 3) k_gain_colsinv(GainTx a)
         tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
         const float *dq = a.d + X.o;
         PAcc sum = pacc_zero();
-        col_inverse<2>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
+        col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
             return ld4(dq, 4 * static_cast<int64_t>(j), ctr);
         }, [&](const float4 &dv, int, bool, const float (&v)[4], uint32_t fb) {
             // at the centre the last two samples are zero
@@ -863,7 +868,7 @@ template <> struct LaneSum<PD> {
 };
 
 template <class V>
-__global__ void __launch_bounds__(TX_T) k_chi2_cols(Chi2Tx<V> a)
+__global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL : 1) k_chi2_cols(Chi2Tx<V> a)
 {
     typedef typename VecT<V>::S S;
     typedef typename PairOf<V>::Z Z;
@@ -898,7 +903,7 @@ __global__ void __launch_bounds__(TX_T) k_chi2_cols(Chi2Tx<V> a)
 // The weights and gradient factors of the modes in the pass's precision, the
 // sums as LaneSum.
 template <class V>
-__global__ void __launch_bounds__(TX_T) k_chi2_rows(Chi2Tx<V> a)
+__global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL : 1) k_chi2_rows(Chi2Tx<V> a)
 {
     typedef typename VecT<V>::S S;
     typedef typename VecT<V>::C C;
@@ -980,7 +985,7 @@ __global__ void __launch_bounds__(TX_T) k_chi2_rows(Chi2Tx<V> a)
 }
 
 template <class V>
-__global__ void __launch_bounds__(TX_T) k_chi2_colsinv(Chi2Tx<V> a)
+__global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL : 1) k_chi2_colsinv(Chi2Tx<V> a)
 {
     typedef typename VecT<V>::S S;
     typedef typename VecT<V>::C C;
@@ -995,7 +1000,7 @@ __global__ void __launch_bounds__(TX_T) k_chi2_colsinv(Chi2Tx<V> a)
         const int64_t o = X.o;
         LaneSum<C> sum;
         struct U4 { S sx[4]; };
-        col_inverse<2>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
+        col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
             U4 D;
             ld4s<S>(a.s, o + 4 * static_cast<int64_t>(j), ctr, D.sx);
             return D;
@@ -1491,7 +1496,7 @@ __device__ void nc_x0_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1)
     float *xq = a.x_out + X.o;
     const int64_t o = X.o, obase = a.off[a.q0], w_lo = obase >> 5;
     float *r = a.cgv + a.cgcap;
-    col_inverse<4>(X, b0, b1, a.Y, a.tw + X.L.twb, cg ? a.flags : nullptr, [&](int, bool, uint32_t) { return 0; },
+    col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, cg ? a.flags : nullptr, [&](int, bool, uint32_t) { return 0; },
                 [&](int, int j, bool ctr, const float (&v)[4], uint32_t fb) {
         const int64_t t = 4 * static_cast<int64_t>(j);
         reinterpret_cast<float2 *>(xq + t)[0] = make_float2(v[0], v[1]);
@@ -1553,7 +1558,7 @@ __device__ void nc_gather_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b
 {
     const int64_t o = X.o, obase = a.off[a.q0], w_lo = obase >> 5;
     float *xq = a.x_out + X.o;
-    col_inverse<2>(X, b0, b1, a.Y, a.tw + X.L.twb, ADD ? nullptr : a.flags, [&](int j, bool ctr, uint32_t) {
+    col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, ADD ? nullptr : a.flags, [&](int j, bool ctr, uint32_t) {
         // ADD: the unit's x0 (written earlier in this launch: coherent loads,
         // not the read-only path); the gather needs only the flag bits
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -2295,7 +2300,7 @@ __global__ void __launch_bounds__(TX_T) k_nc_coarse(NcorrTx a)
         nc_coarse_setup(a, q);
     }
 }
-__global__ void __launch_bounds__(TX_T, 3) k_nc_rhs_cols(NcorrTx a)
+__global__ void __launch_bounds__(TX_T, TX_CTAS_COL) k_nc_rhs_cols(NcorrTx a)
 {
     extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
@@ -2311,7 +2316,7 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_rhs_rows(NcorrTx a)
     int cur = -1;
     nc_items(a, X, true, cur, [&] { nc_rhs_rows(a, X, tx_smem, tx_smem + TX_PAIRS, gi); });
 }
-__global__ void __launch_bounds__(TX_T, 3) k_nc_x0_cols(NcorrTx a)
+__global__ void __launch_bounds__(TX_T, TX_CTAS_COL) k_nc_x0_cols(NcorrTx a)
 {
     extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
@@ -2353,7 +2358,7 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_filter(NcorrTx a, int par)
     nc_list_items(a, X, true, cur, [&] { nc_filter_rows<FINAL>(a, X, tx_smem, tx_smem + TX_PAIRS); });
 }
 template <bool FINAL>
-__global__ void __launch_bounds__(TX_T, 3) k_nc_gather(NcorrTx a, int par)
+__global__ void __launch_bounds__(TX_T, TX_CTAS_COL) k_nc_gather(NcorrTx a, int par)
 {
     extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ TxCtx X;
@@ -2460,10 +2465,13 @@ cudaError_t setup_tx_kernels(Plan &p)
     p.coop_grid = std::max(1, per) * nsm;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_gain_rows, TX_T, s32))) return e;
     p.pass_grid = std::max(1, per) * nsm;
+    p.sm_count = nsm;
     return cudaSuccess;
 }
 
+// persistent grids: the row passes', and that of kernels with `ctas` per SM
 static int grid_for(const Plan &p, int nitems) { return std::max(1, std::min(nitems, p.pass_grid)); }
+static int grid_ctas(const Plan &p, int nitems, int ctas) { return std::max(1, std::min(nitems, p.sm_count * ctas)); }
 
 cudaError_t launch_tx_gain(const Plan &p, const float *d, const float *s, const uint32_t *flags, const double *psd,
                            tod_rng rng, int mode, double *g, double *mu, double *sig, cudaStream_t st, int q0, int q1)
@@ -2484,7 +2492,7 @@ cudaError_t launch_tx_gain(const Plan &p, const float *d, const float *s, const 
     a.items = p.colitems; a.item0 = c0; a.nitems = c1 - c0; a.part = cpart;
     {
         KTIME(TOD_KT_GAIN_COLS);
-        k_gain_cols<<<grid_for(p, a.nitems), TX_T, sm, st>>>(a);
+        k_gain_cols<<<grid_ctas(p, a.nitems, TX_CTAS_COL), TX_T, sm, st>>>(a);
     }
     a.items = p.rowitems; a.item0 = r0; a.nitems = r1 - r0; a.part = rpart;
     {
@@ -2494,7 +2502,7 @@ cudaError_t launch_tx_gain(const Plan &p, const float *d, const float *s, const 
     a.items = p.colitems; a.item0 = c0; a.nitems = c1 - c0; a.part = cpart;
     {
         KTIME(TOD_KT_GAIN_COLSINV);
-        k_gain_colsinv<<<grid_for(p, a.nitems), TX_T, sm, st>>>(a);
+        k_gain_colsinv<<<grid_ctas(p, a.nitems, TX_CTAS_COL), TX_T, sm, st>>>(a);
     }
     {
         KTIME(TOD_KT_GAIN_FIN);
@@ -2525,17 +2533,17 @@ static cudaError_t chi2_range(const Plan &p, const float *d, const void *s, cons
     a.items = p.colitems; a.item0 = c0; a.nitems = c1 - c0; a.part = cpart;
     {
         KTIME(TOD_KT_CHI2_COLS);
-        k_chi2_cols<V><<<grid_for(p, a.nitems), TX_T, sm, st>>>(a);
+        k_chi2_cols<V><<<grid_ctas(p, a.nitems, f32 ? TX_CTAS_COL : 3), TX_T, sm, st>>>(a);
     }
     a.items = p.rowitems; a.item0 = r0; a.nitems = r1 - r0; a.part = rpart;
     {
         KTIME(TOD_KT_CHI2_ROWS);
-        k_chi2_rows<V><<<grid_for(p, a.nitems), TX_T, sm, st>>>(a);
+        k_chi2_rows<V><<<grid_ctas(p, a.nitems, f32 ? TX_CTAS_COL : 3), TX_T, sm, st>>>(a);
     }
     a.items = p.colitems; a.item0 = c0; a.nitems = c1 - c0; a.part = cpart;
     {
         KTIME(TOD_KT_CHI2_COLSINV);
-        k_chi2_colsinv<V><<<grid_for(p, a.nitems), TX_T, sm, st>>>(a);
+        k_chi2_colsinv<V><<<grid_ctas(p, a.nitems, f32 ? TX_CTAS_COL : 3), TX_T, sm, st>>>(a);
     }
     {
         KTIME(TOD_KT_CHI2_FIN);
@@ -2590,6 +2598,7 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
     const int nq = q1 - q0;
     const int ncol = p.h_col_off[q1] - p.h_col_off[q0], nrow = p.h_row_off[q1] - p.h_row_off[q0];
     const int gc = std::min(grid_for(p, ncol), grid), gr = std::min(grid_for(p, nrow), grid);
+    const int gc2 = std::min(gc, grid_ctas(p, ncol, TX_CTAS_COL));
     const int gq = std::min(nq, std::max(1, grid));
     // flag index (count and write use the same grid)
     const int gf = std::max(1, std::min(p.pass_grid, grid));
@@ -2608,7 +2617,7 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
     // x0 = B^{-1} b
     {
         KTIME(TOD_KT_NC_RHS_COLS);
-        k_nc_rhs_cols<<<gc, TX_T, s32, st>>>(a);
+        k_nc_rhs_cols<<<gc2, TX_T, s32, st>>>(a);
     }
     {
         KTIME(TOD_KT_NC_RHS_ROWS);
@@ -2616,7 +2625,7 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
     }
     {
         KTIME(TOD_KT_NC_X0_COLS);
-        k_nc_x0_cols<<<gc, TX_T, s32, st>>>(a);
+        k_nc_x0_cols<<<gc2, TX_T, s32, st>>>(a);
     }
     // CG on the Schur complement
     if (prepared) {
@@ -2643,7 +2652,7 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
         }
         {
             KTIME(TOD_KT_NC_GATHER);
-            k_nc_gather<false><<<gc, TX_T, s32, st>>>(a, par);
+            k_nc_gather<false><<<gc2, TX_T, s32, st>>>(a, par);
         }
         {
             KTIME(TOD_KT_NC_UPDATE);
@@ -2671,7 +2680,7 @@ cudaError_t launch_tx_ncorr(const Plan &p, const float *d, const float *s, const
     }
     {
         KTIME(TOD_KT_NC_GATHER_FINAL);
-        k_nc_gather<true><<<gc, TX_T, s32, st>>>(a, 0);
+        k_nc_gather<true><<<gc2, TX_T, s32, st>>>(a, 0);
     }
     return cudaGetLastError();
 }
