@@ -9,8 +9,8 @@
 // BIN_TILE samples, or one longer run alone).
 //   k_bin:    one CTA per tile gathers the tile's data, residual and
 //             psi/flag words in sorted order into shared memory (the
-//             detscan's samples stay in L2 while its tiles run), then one
-//             thread sums each run.  Products of FP32 values are formed
+//             detscan's samples stay in L2 while its tiles run), then four
+//             lanes sum each run.  Products of FP32 values are formed
 //             exactly and summed as FP32 double-words (FP64 accuracy at FP32
 //             issue rate), the residual d - x taken exactly as a
 //             double-word; each run's sums are scaled by the detscan's
@@ -21,8 +21,8 @@
 //             in FP64, in ascending detscan order.
 #include <algorithm>
 #include "common.cuh"
+#include "fft_reg.cuh"
 #include "internal.cuh"
-
 
 namespace tg {
 
@@ -49,57 +49,92 @@ struct BinArgs {
     const double *y64;
 };
 
-// sum of two double-words (two-sum on the heads, tails added)
-__device__ __forceinline__ Acc2 acc_merge(const Acc2 &a, const Acc2 &b) {
-    Acc2 r = a;
-    acc_add(r, b.s);
-    r.c = __fadd_rn(r.c, b.c);
-    return r;
-}
-
 // the per-run sums: 1 (as hits), c, s, cc, cs, ss, r, cr, sr with r = d - x
-// (taken exactly as a double-word: its head and tail)
-constexpr int NSUM = 8;
+// (taken exactly as a double-word: its head and tail), as the lanes of packed
+// double-words: (c, s), (cc, ss), (cs, r), (cr, sr)
+constexpr int NSUM = 4;
+struct PSum { PF s, c; };
 struct RunSums {
-    Acc2 a[NSUM];
+    PSum a[NSUM];
     int hits;
 };
 __device__ __forceinline__ void sums_zero(RunSums &r) {
 #pragma unroll
-    for (int i = 0; i < NSUM; ++i) r.a[i] = Acc2{0.f, 0.f};
+    for (int i = 0; i < NSUM; ++i) r.a[i] = PSum{{0.f, 0.f}, {0.f, 0.f}};
     r.hits = 0;
+}
+__device__ __forceinline__ void psum_add(PSum &a, PF v) {
+    const PF s = padd(a.s, v);
+    const PF bb = psub(s, a.s);
+    const PF e = padd(psub(a.s, psub(s, bb)), psub(v, bb));
+    a.s = s;
+    a.c = padd(a.c, e);
+}
+// add the exact products x y and the small values t
+__device__ __forceinline__ void psum_add_prod(PSum &a, PF x, PF y, PF t) {
+    const PF p = pmul(x, y);
+    const PF e = pfma(x, y, pneg(p));
+    psum_add(a, p);
+    a.c = padd(a.c, padd(e, t));
+}
+__device__ __forceinline__ void psum_merge(PSum &a, const PSum &b) {
+    psum_add(a, b.s);
+    a.c = padd(a.c, b.c);
 }
 __device__ __forceinline__ void sums_add(RunSums &r, float2 cs, float dv, float xv) {
     ++r.hits;
-    acc_add(r.a[0], cs.x);
-    acc_add(r.a[1], cs.y);
-    acc_add_prod(r.a[2], cs.x, cs.x);
-    acc_add_prod(r.a[3], cs.x, cs.y);
-    acc_add_prod(r.a[4], cs.y, cs.y);
+    const PF v{cs.x, cs.y}, zero{0.f, 0.f};
     // r = d - x exactly: head rh (rounded difference) and tail rl (two-sum)
     const float rh = __fsub_rn(dv, xv);
     const float bb = __fsub_rn(rh, dv);
     const float rl = __fadd_rn(__fsub_rn(dv, __fsub_rn(rh, bb)), __fsub_rn(-xv, bb));
-    acc_add(r.a[5], rh);
-    r.a[5].c = __fadd_rn(r.a[5].c, rl);
-    // c r and s r: exact products of the heads, the tails' products (below
-    // 2^-24 of them) added to the compensation words
-    acc_add_prod(r.a[6], cs.x, rh);
-    r.a[6].c = __fmaf_rn(cs.x, rl, r.a[6].c);
-    acc_add_prod(r.a[7], cs.y, rh);
-    r.a[7].c = __fmaf_rn(cs.y, rl, r.a[7].c);
+    psum_add(r.a[0], v);
+    psum_add_prod(r.a[1], v, v, zero);
+    // the tail of r, and its products with c and s (below 2^-24 of the
+    // heads'), go to the compensation words
+    psum_add_prod(r.a[2], PF{cs.x, rh}, PF{cs.y, 1.0f}, PF{0.f, rl});
+    psum_add_prod(r.a[3], v, PF{rh, rh}, pmul(v, PF{rl, rl}));
 }
-__device__ __forceinline__ void sums_store(const RunSums &r, double wA, double wb, double *rr) {
-    rr[0] = wA * r.hits;
-    rr[1] = wA * acc_value(r.a[0]);
-    rr[2] = wA * acc_value(r.a[1]);
-    rr[3] = wA * acc_value(r.a[2]);
-    rr[4] = wA * acc_value(r.a[3]);
-    rr[5] = wA * acc_value(r.a[4]);
-    rr[6] = wb * acc_value(r.a[5]);
-    rr[7] = wb * acc_value(r.a[6]);
-    rr[8] = wb * acc_value(r.a[7]);
-    rr[9] = static_cast<double>(r.hits);
+__device__ __forceinline__ PF shfl_xor(PF v, int m) {
+    return PF{__shfl_xor_sync(0xffffffffu, v.a, m), __shfl_xor_sync(0xffffffffu, v.b, m)};
+}
+// the sums of lanes l and l ^ m, the lower lane's first, in both
+__device__ __forceinline__ void sums_merge_xor(RunSums &r, int m) {
+    const bool up = (threadIdx.x & m) != 0;
+#pragma unroll
+    for (int k = 0; k < NSUM; ++k) {
+        PSum p = r.a[k], o{shfl_xor(p.s, m), shfl_xor(p.c, m)};
+        if (up) {
+            psum_merge(o, p);
+            r.a[k] = o;
+        } else {
+            psum_merge(p, o);
+            r.a[k] = p;
+        }
+    }
+    r.hits += __shfl_xor_sync(0xffffffffu, r.hits, m);
+}
+// the ten outputs as double-words (hits exact below 2^24, else in two words)
+__device__ __forceinline__ void sums_out(const RunSums &r, Acc2 *o) {
+    const float h = static_cast<float>(r.hits);
+    const float hl = static_cast<float>(r.hits - static_cast<int>(h));
+    o[0] = o[9] = Acc2{h, hl};
+    o[1] = Acc2{r.a[0].s.a, r.a[0].c.a};
+    o[2] = Acc2{r.a[0].s.b, r.a[0].c.b};
+    o[3] = Acc2{r.a[1].s.a, r.a[1].c.a};
+    o[4] = Acc2{r.a[2].s.a, r.a[2].c.a};
+    o[5] = Acc2{r.a[1].s.b, r.a[1].c.b};
+    o[6] = Acc2{r.a[2].s.b, r.a[2].c.b};
+    o[7] = Acc2{r.a[3].s.a, r.a[3].c.a};
+    o[8] = Acc2{r.a[3].s.b, r.a[3].c.b};
+}
+// float to double, exactly, by integer instructions (the conversion itself
+// issues with the FP64 ones): normal numbers and zeros, the rest converted
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+    if (m - 0x00800000u >= 0x7F000000u && m != 0u) return static_cast<double>(x);
+    const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u);
+    return __hiloint2double(static_cast<int>(hi), static_cast<int>(m << 29));
 }
 
 __device__ __forceinline__ uint16_t psi_flag(const BinArgs &a, int64_t tg) {
@@ -121,23 +156,91 @@ __device__ __forceinline__ void load_dx(const BinArgs &a, int64_t tg, float &dv,
     }
 }
 
-__global__ void __launch_bounds__(BIN_T) k_bin(BinArgs a)
+// copies into shared memory past the registers; zeros where !take
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool take) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                 :: "r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src), "r"(take ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async8(float2 *dst, const float2 *src, bool take) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;"
+                 :: "r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src), "r"(take ? 8 : 0) : "memory");
+}
+
+// Bound by the gather: its loads and the sectors they touch take three
+// quarters of the time (324 of 401 us with the sums left out).  A branch per
+// sample put the psi -> cos, sin chains of a thread's eight samples one behind
+// the other; here each kind of load is issued for all eight first, and data,
+// residual and cos, sin go past the registers, which also keeps five CTAs on
+// an SM (four: 441 against 409 us; six, by spilling: 449).  FP64 issues at 1/64
+// of the FP32 rate, so the weights' divisions run on one thread of the last
+// warp beside the sums, and the outputs of 64 runs are scaled by all threads,
+// every lane of an FP64 instruction at work; the sums are packed FP32
+// double-words.  Four lanes per run: eight are even at 33 runs a tile (409
+// against 401 us) and slower at 40 (963 against 876).
+// 45M samples of 44 GHz: 596 -> 401 us; 102M of 70 GHz: 1324 -> 876 us.
+constexpr int BIN_LANES = 4;                         // lanes per run
+constexpr int BIN_CTAS = 5;                          // CTAs per SM
+constexpr int BIN_BATCH = 64;                        // runs whose outputs are staged together
+
+__global__ void __launch_bounds__(BIN_T, BIN_CTAS) k_bin(BinArgs a)
 {
     __shared__ float s_d[BIN_TILE], s_x[BIN_TILE];
     __shared__ float2 s_cs[BIN_TILE];
-    __shared__ Acc2 s_red[BIN_T / 32][NSUM];
-    __shared__ int s_hits[BIN_T / 32];
-    __shared__ Acc2 s_out[BIN_T / 4][10];          // a quad's ten run outputs as double-words
+    __shared__ Acc2 s_out[BIN_BATCH][10];            // the outputs of a batch's runs
+    __shared__ double s_w[2];
+    __shared__ RunSums s_red[BIN_T / 32];
     const int tile = blockIdx.x;
     const int q = a.tile_q[tile];
     const int r0 = a.tile_r0[tile], nr = a.tile_r0[tile + 1] - r0;
     const int64_t o = a.off[q];
     const int64_t s0 = a.pair_start[r0];
     const int cnt = static_cast<int>(a.pair_start[r0 + nr - 1] + a.pair_len[r0 + nr - 1] - s0);
-    // the detscan's weights g^2/sigma0^2 and g/sigma0^2: FP64 divisions once,
-    // by thread 0 (FP64 issues at 1/64 of the FP32 rate on this part)
-    __shared__ double s_w[2];
-    if (threadIdx.x == 0) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool whole = cnt > BIN_TILE;               // one run longer than a tile
+
+    if (!whole) {
+        // gather in the tile's load order (the k-th sample of each run, k = 0,
+        // 1, ..: a warp's 32 samples are close in time, so they share sectors),
+        // each value into its run-major slot: the positions first, then every
+        // psi, flag, data and residual load of the thread in flight together
+        // (data and residual straight into shared memory), then cos 2psi and
+        // sin 2psi, both zero for a flagged sample
+        constexpr int PER = BIN_TILE / BIN_T;
+        int idx[PER], pos[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int i = threadIdx.x + u * BIN_T;
+            idx[u] = i < cnt ? static_cast<int>(__ldg(a.ld_t + s0 + i)) : -1;
+            pos[u] = i < cnt ? __ldg(a.ld_pos + s0 + i) : 0;
+        }
+        uint32_t fw[PER];
+        uint16_t pf[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int64_t tg = o + idx[u];
+            pf[u] = idx[u] >= 0 ? __ldg(a.psi + tg) : 0;
+            fw[u] = a.flags && idx[u] >= 0 ? __ldg(a.flags + (tg >> 5)) >> (tg & 31) : 0u;
+        }
+        if (a.y64) {
+#pragma unroll
+            for (int u = 0; u < PER; ++u)
+                if (idx[u] >= 0) load_dx(a, o + idx[u], s_d[pos[u]], s_x[pos[u]]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < PER; ++u)
+                if (idx[u] >= 0) {
+                    cp_async4(s_d + pos[u], a.d + o + idx[u], true);
+                    cp_async4(s_x + pos[u], a.x ? a.x + o + idx[u] : a.d, a.x != nullptr);
+                }
+        }
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (idx[u] >= 0) cp_async8(s_cs + pos[u], a.trig + (pf[u] & 0x0FFF), !(fw[u] & 1u));
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+    }
+    // the detscan's weights g^2/sigma0^2 and g/sigma0^2
+    if (threadIdx.x == BIN_T - 1) {
         const double gq = a.gain[q];
         if (a.adjoint) {
             s_w[0] = 0.0;
@@ -148,130 +251,64 @@ __global__ void __launch_bounds__(BIN_T) k_bin(BinArgs a)
             s_w[1] = gq / (sig0 * sig0);
         }
     }
-    __syncthreads();
-    const double wA = s_w[0], wb = s_w[1];
-
-    if (cnt > BIN_TILE) {
-        // one run longer than a tile: strided partial sums, then a fixed-order tree
-        RunSums r;
-        sums_zero(r);
-        for (int i = threadIdx.x; i < cnt; i += BIN_T) {
-            const int64_t tg = o + __ldg(a.ld_t + s0 + i);     // a single run: run order
-            const uint16_t pf = psi_flag(a, tg);
-            if (pf >> 15) continue;
-            float dv, xv;
-            load_dx(a, tg, dv, xv);
-            sums_add(r, __ldg(a.trig + (pf & 0x0FFF)), dv, xv);
-        }
-#pragma unroll
-        for (int ofs = 16; ofs; ofs >>= 1) {
-#pragma unroll
-            for (int k = 0; k < NSUM; ++k) {
-                Acc2 o2;
-                o2.s = __shfl_down_sync(0xffffffffu, r.a[k].s, ofs);
-                o2.c = __shfl_down_sync(0xffffffffu, r.a[k].c, ofs);
-                r.a[k] = acc_merge(r.a[k], o2);
+    for (int rb = 0; rb < nr; rb += BIN_BATCH) {
+        const int nb = min(BIN_BATCH, nr - rb);
+        if (whole) {
+            // strided partial sums, then a fixed-order tree
+            RunSums rs;
+            sums_zero(rs);
+            for (int i = threadIdx.x; i < cnt; i += BIN_T) {
+                const int64_t tg = o + __ldg(a.ld_t + s0 + i);     // a single run: run order
+                const uint16_t pf = psi_flag(a, tg);
+                if (pf >> 15) continue;
+                float dv, xv;
+                load_dx(a, tg, dv, xv);
+                sums_add(rs, __ldg(a.trig + (pf & 0x0FFF)), dv, xv);
             }
-            r.hits += __shfl_down_sync(0xffffffffu, r.hits, ofs);
-        }
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        if (lane == 0) {
+#pragma unroll 1
+            for (int m = 1; m < 32; m <<= 1) sums_merge_xor(rs, m);
+            if (lane == 0) s_red[warp] = rs;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int w = 1; w < BIN_T / 32; ++w) {
 #pragma unroll
-            for (int k = 0; k < NSUM; ++k) s_red[warp][k] = r.a[k];
-            s_hits[warp] = r.hits;
+                    for (int k = 0; k < NSUM; ++k) psum_merge(rs.a[k], s_red[w].a[k]);
+                    rs.hits += s_red[w].hits;
+                }
+                sums_out(rs, s_out[0]);
+            }
+        } else {
+            // lane j of a run's quad takes its samples j, j + 4, ...; their
+            // sums are merged in a fixed order (deterministic)
+            const int sub = lane / BIN_LANES, ql = lane % BIN_LANES;
+            for (int g = warp * (32 / BIN_LANES); g < nb; g += BIN_T / BIN_LANES) {
+                const int r = g + sub;
+                RunSums rs;
+                sums_zero(rs);
+                if (r < nb) {
+                    const int st = static_cast<int>(a.pair_start[r0 + rb + r] - s0);
+                    const int end = st + a.pair_len[r0 + rb + r];
+                    for (int i = st + ql; i < end; i += BIN_LANES) {
+                        const float2 cs = s_cs[i];
+                        if (cs.x == 0.0f && cs.y == 0.0f) continue;
+                        sums_add(rs, cs, s_d[i], s_x[i]);
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int m = 1; m < BIN_LANES; m <<= 1) sums_merge_xor(rs, m);
+                if (r < nb && ql == 0) sums_out(rs, s_out[r]);
+            }
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < BIN_T / 32; ++w) {
-#pragma unroll
-                for (int k = 0; k < NSUM; ++k) r.a[k] = acc_merge(r.a[k], s_red[w][k]);
-                r.hits += s_hits[w];
-            }
-            sums_store(r, wA, wb, a.rec + static_cast<int64_t>(a.pair_slot[r0]) * 10);
+        const double wA = s_w[0], wb = s_w[1];
+        for (int e = threadIdx.x; e < nb * 10; e += BIN_T) {
+            const int r = e / 10, i = e - 10 * r;
+            const Acc2 v = s_out[r][i];
+            const double w = i == 9 ? 1.0 : (i <= 5 ? wA : wb);
+            a.rec[static_cast<int64_t>(a.pair_slot[r0 + rb + r]) * 10 + i] = w * (widen(v.s) + widen(v.c));
         }
-        return;
-    }
-
-    // gather in the tile's load order (the k-th sample of each run, k = 0,
-    // 1, ..: a warp's 32 samples are close in time, so they share sectors):
-    // the positions first, then every value load of the thread in flight
-    // together, each value into its run-major slot; cos 2psi and sin 2psi
-    // are staged with the data, and a flagged sample is marked by cos = 2
-    constexpr int PER = BIN_TILE / BIN_T;
-    int idx[PER], pos[PER];
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int i = threadIdx.x + u * BIN_T;
-        idx[u] = -1;
-        pos[u] = 0;
-        if (i < cnt) {
-            idx[u] = static_cast<int>(__ldg(a.ld_t + s0 + i));
-            pos[u] = __ldg(a.ld_pos + s0 + i);
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        if (idx[u] < 0) continue;
-        const int64_t tg = o + idx[u];
-        const uint16_t pf = psi_flag(a, tg);
-        float2 cs = __ldg(a.trig + (pf & 0x0FFF));
-        if (pf >> 15) cs.x = 2.0f;
-        const int i = pos[u];
-        s_cs[i] = cs;
-        load_dx(a, tg, s_d[i], s_x[i]);
-    }
-    __syncthreads();
-    // four lanes per run: lane j of the quad takes samples j, j+4, ...; the
-    // quad's partial sums are merged in a fixed order (deterministic)
-    const int quad = threadIdx.x >> 2, ql = threadIdx.x & 3;
-    for (int rb = 0; rb < nr; rb += BIN_T / 4) {
-        const int r = rb + quad;
-        RunSums rs;
-        sums_zero(rs);
-        int pr = -1;
-        if (r < nr) {
-            pr = r0 + r;
-            const int st = static_cast<int>(a.pair_start[pr] - s0);
-            const int len = a.pair_len[pr];
-            for (int i = st + ql; i < st + len; i += 4) {
-                const float2 cs = s_cs[i];
-                if (cs.x > 1.5f) continue;
-                sums_add(rs, cs, s_d[i], s_x[i]);
-            }
-        }
-#pragma unroll
-        for (int ofs = 1; ofs <= 2; ofs <<= 1) {
-#pragma unroll
-            for (int k = 0; k < NSUM; ++k) {
-                Acc2 o2;
-                o2.s = __shfl_xor_sync(0xffffffffu, rs.a[k].s, ofs);
-                o2.c = __shfl_xor_sync(0xffffffffu, rs.a[k].c, ofs);
-                rs.a[k] = (ql & ofs) ? acc_merge(o2, rs.a[k]) : acc_merge(rs.a[k], o2);
-            }
-            rs.hits += __shfl_xor_sync(0xffffffffu, rs.hits, ofs);
-        }
-        // the ten outputs in FP64, spread over the quad's lanes (lane ql takes
-        // outputs ql, ql + 4, ql + 8: FP64 issues slowly on this part, so every
-        // lane of its warp instructions works)
-        if (pr >= 0 && ql == 0) {
-            Acc2 *o = s_out[quad];
-            o[0] = Acc2{static_cast<float>(rs.hits), 0.f};      // hits <= BIN_TILE: exact
-#pragma unroll
-            for (int k = 0; k < 5; ++k) o[1 + k] = rs.a[k];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) o[6 + k] = rs.a[5 + k];
-            o[9] = o[0];
-        }
-        __syncwarp();
-        if (pr >= 0) {
-            double *rr = a.rec + static_cast<int64_t>(a.pair_slot[pr]) * 10;
-            for (int i = ql; i < 10; i += 4) {
-                const Acc2 v = s_out[quad][i];
-                const double w = i == 9 ? 1.0 : (i <= 5 ? wA : wb);
-                rr[i] = w * acc_value(v);
-            }
-        }
-        __syncwarp();
+        if (rb + BIN_BATCH < nr) __syncthreads();    // the next batch overwrites s_out
     }
 }
 
