@@ -38,18 +38,73 @@ struct TxCtx {
     int64_t o;                                   // first sample of the detscan
     int64_t yb;                                  // first complex value of its Y block
     int64_t koff;                                // first flagged rank (n_corr)
+    int2 fw[3];                                  // ItemFeed: items by turn, and their length indices
+    int fl[3];
 };
 
-// Copy the length plan of item (q, blk) into shared memory (skipped when the
-// previous item had the same length) and set the detscan scalars.  All
-// threads call it; it ends with a barrier.
-__device__ __forceinline__ void tx_begin(TxCtx &X, const TxLen *__restrict__ txl, const int32_t *__restrict__ q_tx,
-                                         const int64_t *__restrict__ off, int q, int blk, int64_t obase, int ndet,
-                                         double fsamp, const double *psd, const double *gain, int &cur,
-                                         const float4 *__restrict__ qsc = nullptr)
+__device__ __forceinline__ void cp_async_bytes4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n"
+                 ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_bytes8(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n"
+                 ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+}
+
+// A CTA's share of a list of n items, i0, i0 + stride, ..: the items (detscan,
+// tile) and the detscans' length indices, fetched by thread 0 two tiles and
+// one tile ahead of their use into a ring in shared memory (two dependent
+// loads, about a microsecond, in front of every tile otherwise; in registers
+// the row passes spilled more).  n_corr draw of 6 x 45 detscans at 44 GHz, this
+// and the single round of loads in tx_begin: 2335 -> 2196 us; chi^2 of 52M
+// samples, with the spectrum's logarithm once per detscan: 2336 -> 2240 us.
+struct ItemFeed {
+    const int2 *__restrict__ items;
+    const int32_t *__restrict__ q_tx;
+    int last, k;
+    __device__ __forceinline__ ItemFeed(TxCtx &X, const int2 *items_, const int32_t *q_tx_, int i0, int n)
+        : items(items_), q_tx(q_tx_), last(n - 1), k(0) {
+        if (threadIdx.x == 0 && i0 <= last) {
+            X.fw[0] = items[i0];
+            if (i0 + static_cast<int>(gridDim.x) <= last) X.fw[1] = items[i0 + static_cast<int>(gridDim.x)];
+            X.fl[0] = q_tx[X.fw[0].x];
+        }
+    }
+    // by thread 0 alone, ahead of the barrier that the others read the turn's
+    // slot behind: waits for it, and fetches for the turns to come (none is
+    // left in flight after the last)
+    __device__ __forceinline__ void fetch(TxCtx &X, int it) const {
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        const int k1 = k == 2 ? 0 : k + 1, k2 = k1 == 2 ? 0 : k1 + 1;
+        const int st = static_cast<int>(gridDim.x);
+        if (it + st <= last) cp_async_bytes4(&X.fl[k1], q_tx + X.fw[k1].x);
+        if (it + 2 * st <= last) cp_async_bytes8(&X.fw[k2], items + it + 2 * st);
+    }
+    __device__ __forceinline__ void next() { k = k == 2 ? 0 : k + 1; }
+};
+
+// The item (q, blk) set up: the length plan li copied into shared memory
+// (skipped when the previous item had the same length) and the detscan's
+// scalars, from qsc those of the call, from cgs its CG mode and first rank.
+// All threads call it; it ends with a barrier.  A tile takes 5 to 20 us, and
+// its FFT waits for all of this: the loads go out together, ahead of the first
+// barrier.
+struct TxItem { int64_t o, koff; float4 a0, a1; int mode; };
+__device__ __forceinline__ TxItem tx_load(const int64_t *__restrict__ off, int q, const float4 *__restrict__ qsc,
+                                          const CgState *cgs)
 {
-    __syncthreads();                 // earlier readers of X are done
-    const int li = q_tx[q];
+    TxItem t;
+    t.a0 = t.a1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    t.mode = 0;
+    t.koff = 0;
+    t.o = off[q];
+    if (qsc) { t.a0 = qsc[2 * q]; t.a1 = qsc[2 * q + 1]; }
+    if (cgs) { t.mode = cgs[q].mode; t.koff = cgs[q].koff; }
+    return t;
+}
+__device__ __forceinline__ void tx_set(TxCtx &X, const TxLen *__restrict__ txl, const TxItem &t, int q, int blk, int li,
+                                       int64_t obase, int ndet, int &cur)
+{
     if (li != cur) {
         const int4 *src = reinterpret_cast<const int4 *>(txl + li);
         int4 *dst = reinterpret_cast<int4 *>(&X.L);
@@ -59,26 +114,41 @@ __device__ __forceinline__ void tx_begin(TxCtx &X, const TxLen *__restrict__ txl
         X.q = q;
         X.blk = blk;
         X.det = q % ndet;
-        X.o = off[q];
-        X.yb = (off[q] - obase) >> 1;
-        if (qsc) {          // precomputed for this call: (s2, 1/s2, 1/s, fscale), (alpha, g, -, -)
-            const float4 a0 = qsc[2 * q], a1 = qsc[2 * q + 1];
-            X.s2 = a0.x; X.inv_s2 = a0.y; X.inv_s = a0.z; X.fscale = a0.w;
-            X.alpha = a1.x;
-            X.g = a1.y;
-        } else if (psd) {
-            const double sig0 = psd[3 * X.det], fk = psd[3 * X.det + 1], al = psd[3 * X.det + 2];
-            const int n = static_cast<int>(off[q + 1] - off[q]);
-            X.s2 = static_cast<float>(sig0 * sig0);
-            X.inv_s2 = static_cast<float>(1.0 / (sig0 * sig0));
-            X.inv_s = static_cast<float>(1.0 / sig0);
-            X.fscale = static_cast<float>(fsamp / (2.0 * n * fk));
-            X.alpha = static_cast<float>(al);
-        }
-        if (!qsc) X.g = gain ? static_cast<float>(gain[q]) : 1.0f;
+        X.o = t.o;
+        X.yb = (t.o - obase) >> 1;
+        X.s2 = t.a0.x; X.inv_s2 = t.a0.y; X.inv_s = t.a0.z; X.fscale = t.a0.w;
+        X.alpha = t.a1.x;
+        X.g = t.a1.y;
+        X.mode = t.mode;
+        X.koff = t.koff;
     }
     cur = li;
     __syncthreads();
+}
+__device__ __forceinline__ void tx_begin(TxCtx &X, const TxLen *__restrict__ txl, int li,
+                                         const int64_t *__restrict__ off, int q, int blk, int64_t obase, int ndet,
+                                         int &cur, const float4 *__restrict__ qsc = nullptr,
+                                         const CgState *cgs = nullptr)
+{
+    TxItem t{};
+    if (threadIdx.x == 0) t = tx_load(off, q, qsc, cgs);
+    __syncthreads();                 // earlier readers of X are done
+    tx_set(X, txl, t, q, blk, li, obase, ndet, cur);
+}
+// the feed's next item
+__device__ __forceinline__ void tx_begin(TxCtx &X, ItemFeed &feed, int it, const TxLen *__restrict__ txl,
+                                         const int64_t *__restrict__ off, int64_t obase, int ndet, int &cur,
+                                         const float4 *__restrict__ qsc = nullptr, const CgState *cgs = nullptr)
+{
+    TxItem t{};
+    if (threadIdx.x == 0) {
+        feed.fetch(X, it);
+        t = tx_load(off, X.fw[feed.k].x, qsc, cgs);
+    }
+    __syncthreads();                 // earlier readers of X are done, the turn's slot is there
+    const int2 w = X.fw[feed.k];
+    tx_set(X, txl, t, w.x, w.y, X.fl[feed.k], obase, ndet, cur);
+    feed.next();
 }
 
 // The FP32 scalars of every detscan of a call, from the FP64 noise
@@ -689,9 +759,9 @@ __global__ void __launch_bounds__(TX_T, TX_CTAS_COL) k_gain_cols(GainTx a)
     __shared__ TxCtx X;
     CF2 *b0 = tx_smem, *b1 = tx_smem + TX_PAIRS;
     int cur = -1;
+    ItemFeed feed(X, a.items + a.item0, a.q_tx, blockIdx.x, a.nitems);
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const int2 w = a.items[a.item0 + it];
-        tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
+        tx_begin(X, feed, it, a.txl, a.off, a.obase, a.ndet, cur);
         const float *sq = a.s + X.o;
         col_forward<false, 4>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](CF2 *) {},
                     [&](int j, bool ctr, uint32_t) { return ld4(sq, 4 * static_cast<int64_t>(j), ctr); },
@@ -711,9 +781,9 @@ __global__ void __launch_bounds__(TX_T, 3) k_gain_rows(GainTx a)
     __shared__ double s_red[TX_T / 32], s_out[1];
     CF2 *b0 = tx_smem, *b1 = tx_smem + TX_PAIRS;
     int cur = -1;
+    ItemFeed feed(X, a.items + a.item0, a.q_tx, blockIdx.x, a.nitems);
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const int2 w = a.items[a.item0 + it];
-        tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, a.psd, nullptr, cur, a.qsc);
+        tx_begin(X, feed, it, a.txl, a.off, a.obase, a.ndet, cur, a.qsc);
         const float fscale = X.fscale, alpha = X.alpha, s2 = X.s2;
         const int n = X.L.n, m = X.L.m;
         PAcc sum = pacc_zero();
@@ -740,9 +810,9 @@ __global__ void __launch_bounds__(TX_T, TX_CTAS_COL) k_gain_colsinv(GainTx a)
     __shared__ double s_red[TX_T / 32], s_out[1];
     CF2 *b0 = tx_smem, *b1 = tx_smem + TX_PAIRS;
     int cur = -1;
+    ItemFeed feed(X, a.items + a.item0, a.q_tx, blockIdx.x, a.nitems);
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const int2 w = a.items[a.item0 + it];
-        tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
+        tx_begin(X, feed, it, a.txl, a.off, a.obase, a.ndet, cur);
         const float *dq = a.d + X.o;
         PAcc sum = pacc_zero();
         col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
@@ -847,6 +917,7 @@ template <class V> struct Chi2Tx {
     int64_t obase;
     Z *Y;
     double *part;                 // [item][4]
+    double2 *par;                 // [nq][2] (sigma0, ln(fsamp/(2 n f_knee))), (alpha, f_knee): the row pass's
     void *v_out;                  // float or double [N] (global sample index), or null
     bool v_al;                    // v_out aligned to two values
 };
@@ -876,10 +947,11 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
     __shared__ TxCtx X;
     V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_PAIRS;
     int cur = -1;
+    ItemFeed feed(X, a.items + a.item0, a.q_tx, blockIdx.x, a.nitems);
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const int2 w = a.items[a.item0 + it];
-        tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
-        const S g = static_cast<S>(a.gain[X.q]);
+        tx_begin(X, feed, it, a.txl, a.off, a.obase, a.ndet, cur);
+        const double gq = a.gain[X.q];
+        const S g = static_cast<S>(gq);
         const float *dq = a.d + X.o;
         const int64_t o = X.o;
         struct U4 { float4 dv; S sx[4]; };
@@ -897,6 +969,11 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
                         v[2] = (fb & 4) ? S(0) : static_cast<S>(D.dv.z) - g * D.sx[2];
                         v[3] = (fb & 8) ? S(0) : static_cast<S>(D.dv.w) - g * D.sx[3];
                     });
+        if (X.blk == 0 && threadIdx.x == 0) {      // once per detscan: a chain of FP64 operations, 40 ns each
+            const double *ps = a.psd + 3 * X.det;
+            a.par[2 * X.q] = make_double2(ps[0], log(a.fsamp / (2.0 * X.L.n * ps[1])));
+            a.par[2 * X.q + 1] = make_double2(ps[2], ps[1]);
+        }
     }
 }
 
@@ -910,22 +987,15 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
     extern __shared__ __align__(16) CD2 tx_smem64[];
     __shared__ TxCtx X;
     __shared__ double s_red[4 * (TX_T / 32)], s_out[4];
-    __shared__ double s_par[4];       // sigma0, ln(fsamp/(2 n f_knee)), alpha, f_knee
     V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_PAIRS;
     int cur = -1;
+    ItemFeed feed(X, a.items + a.item0, a.q_tx, blockIdx.x, a.nitems);
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const int2 w = a.items[a.item0 + it];
-        tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, a.psd, nullptr, cur);
-        if (threadIdx.x == 0) {
-            const double sig0 = a.psd[3 * X.det], fk = a.psd[3 * X.det + 1], al = a.psd[3 * X.det + 2];
-            s_par[0] = sig0;
-            s_par[1] = log(a.fsamp / (2.0 * X.L.n * fk));
-            s_par[2] = al;
-            s_par[3] = fk;
-        }
-        __syncthreads();
-        const S sig0 = static_cast<S>(s_par[0]), lfs = static_cast<S>(s_par[1]), al = static_cast<S>(s_par[2]);
-        const S fk = static_cast<S>(s_par[3]);
+        tx_begin(X, feed, it, a.txl, a.off, a.obase, a.ndet, cur);
+        const double2 *par = a.par + 2 * X.q;                        // written by k_chi2_cols
+        const double2 pa = __ldg(par), pb = __ldg(par + 1);
+        const S sig0 = static_cast<S>(pa.x), lfs = static_cast<S>(pa.y), al = static_cast<S>(pb.x);
+        const S fk = static_cast<S>(pb.y);
         const S s2 = sig0 * sig0;
         const S d1 = S(2) / sig0, d2 = -s2 * al / fk;
         const int n = X.L.n, m = X.L.m;
@@ -994,9 +1064,9 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
     __shared__ double s_red[TX_T / 32], s_out[1];
     V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_PAIRS;
     int cur = -1;
+    ItemFeed feed(X, a.items + a.item0, a.q_tx, blockIdx.x, a.nitems);
     for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const int2 w = a.items[a.item0 + it];
-        tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.obase, a.ndet, a.fsamp, nullptr, nullptr, cur);
+        tx_begin(X, feed, it, a.txl, a.off, a.obase, a.ndet, cur);
         const int64_t o = X.o;
         LaneSum<C> sum;
         struct U4 { S sx[4]; };
@@ -2172,11 +2242,10 @@ __device__ __forceinline__ void nc_items(const NcorrTx &a, TxCtx &X, bool rows, 
     const int2 *items = rows ? a.rowitems : a.colitems;
     const int j0 = rows ? a.row_off[a.q0] : a.col_off[a.q0];
     const int j1 = rows ? a.row_off[a.q1] : a.col_off[a.q1];
+    const int64_t obase = a.off[a.q0];
+    ItemFeed feed(X, items, a.q_tx, j0 + blockIdx.x, j1);
     for (int it = j0 + blockIdx.x; it < j1; it += gridDim.x) {
-        const int2 w = items[it];
-        tx_begin(X, a.txl, a.q_tx, a.off, w.x, w.y, a.off[a.q0], a.ndet, a.fsamp, a.psd, a.gain, cur, a.qsc);
-        if (threadIdx.x == 0) { X.mode = a.cgs[w.x].mode; X.koff = a.cgs[w.x].koff; }
-        __syncthreads();
+        tx_begin(X, feed, it, a.txl, a.off, obase, a.ndet, cur, a.qsc, a.cgs);
         fn();
     }
 }
@@ -2258,6 +2327,7 @@ __device__ __forceinline__ void nc_list_items(const NcorrTx &a, TxCtx &X, bool r
     const int32_t *lq = nl_q(a), *lo = rows ? nl_row(a) : nl_col(a);
     const int i0 = blockIdx.x, i1 = lo[n];
     if (i0 >= i1) return;
+    const int64_t obase = a.off[a.q0];
     int pos = 0, hi = n - 1;                      // last detscan whose items start at or before i0
     while (pos < hi) {
         const int mid = (pos + hi + 1) >> 1;
@@ -2266,9 +2336,7 @@ __device__ __forceinline__ void nc_list_items(const NcorrTx &a, TxCtx &X, bool r
     for (int ii = i0; ii < i1; ii += gridDim.x) {
         while (lo[pos + 1] <= ii) ++pos;
         const int q = lq[pos];
-        tx_begin(X, a.txl, a.q_tx, a.off, q, ii - lo[pos], a.off[a.q0], a.ndet, a.fsamp, a.psd, a.gain, cur, a.qsc);
-        if (threadIdx.x == 0) { X.mode = a.cgs[q].mode; X.koff = a.cgs[q].koff; }
-        __syncthreads();
+        tx_begin(X, a.txl, a.q_tx[q], a.off, q, ii - lo[pos], obase, a.ndet, cur, a.qsc, a.cgs);
         fn();
     }
 }
@@ -2523,6 +2591,7 @@ static cudaError_t chi2_range(const Plan &p, const float *d, const void *s, cons
     constexpr bool f32 = sizeof(Z) == sizeof(float2);
     a.tw = reinterpret_cast<const Z *>(f32 ? static_cast<const void *>(p.txtw) : static_cast<const void *>(p.txtw64));
     a.ndet = p.ndet; a.fsamp = p.fsamp; a.obase = p.h_off[q0];
+    a.par = reinterpret_cast<double2 *>(p.qsc);
     a.Y = reinterpret_cast<Z *>(p.ybuf);
     a.v_out = v_out;
     a.v_al = (reinterpret_cast<uintptr_t>(v_out) & (sizeof(Z) - 1)) == 0;
