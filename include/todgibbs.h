@@ -387,7 +387,7 @@ tod_status tod_sample_ncorr(tod_plan *p, const float *d, const float *s,
  *   per-detector gap preconditioner tables the plan holds (the Toeplitz
  *   autocovariance of the CG operator at every lag of a power-of-two
  *   reference length, by one FFT per two detectors, its prefix sums for the
- *   coarse correction, and the Durbin solutions of its first 512 lags),
+ *   coarse correction, and T_L^-1 e_1 of its first 512 lags),
  *   overwriting the previous ones.
  *   tod_sample_ncorr_prepared is tod_sample_ncorr (same arguments, results
  *   and errors) using those tables; psd must be the array they were built
