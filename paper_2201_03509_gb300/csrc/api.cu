@@ -916,6 +916,7 @@ tod_status tod_plan_create(tod_plan **out, const tod_band_desc *band)
         const size_t M2 = 2 * static_cast<size_t>(p->cz_href);
         if ((e = dev_upload(*p, p->czfft, static_cast<float2 *>(nullptr), 2 * static_cast<size_t>((p->ndet + 1) / 2) * M2)))
             return fail(e);
+        if ((e = dev_upload(*p, p->czscale, static_cast<float *>(nullptr), static_cast<size_t>(p->ndet)))) return fail(e);
         if ((e = dev_upload(*p, p->cztab, static_cast<float4 *>(nullptr),
                             static_cast<size_t>(p->ndet) * (static_cast<size_t>(p->cz_href) + 1))))
             return fail(e);

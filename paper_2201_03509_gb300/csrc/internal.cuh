@@ -128,6 +128,7 @@ struct Plan {
     // two detectors, and its prefix sums
     int32_t cz_href = 0;
     float2 *czfft = nullptr;         // [2][(ndet + 1)/2][2 cz_href] FFT work, then the kernels
+    float *czscale = nullptr;        // [ndet] factor of a detector's part of the transform
     float4 *cztab = nullptr;         // [ndet][cz_href + 1] (H, G) as FP32 pairs: H(x) = sum_{d<x} h(d), G: d h(d)
     int32_t *gbpos = nullptr;        // [nq][TX_GBMAX] first sample (within the detscan) of each block
     float *czsz = nullptr;           // [czcap][TX_CZJ] S Z entries by flagged rank

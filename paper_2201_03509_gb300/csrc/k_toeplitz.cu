@@ -11,7 +11,10 @@
 // part of the length-2H DFT of the even sequence a_k = gamma_k (k < H),
 // a_{2H-k} = gamma_k, a_H = 0, divided by 2H.  The transform of a real even
 // sequence is real, so one complex FP32 FFT serves two detectors (one in the
-// real, one in the imaginary part).  A scan then stores, for the coarse
+// real, one in the imaginary part), each brought to a peak between 1 and 2 by
+// a power of two first: the rounding of the transform goes by the larger of
+// the two, and a detector far below its partner, or beside one whose noise
+// parameters are not finite, keeps its own kernel.  A scan then stores, for the coarse
 // correction, the prefix sums H(x) = sum_{d<x} h(d) and G(x) = sum_{d<x} d h(d)
 // (FP32 double-words); the gap blocks take the first TOEP_LMAX lags.
 // A second kernel finds, for every order L, the first column
@@ -67,13 +70,35 @@ __device__ __forceinline__ DW dw_div(DW a, DW b) {
     return dw_renorm(q, __fmul_rn(r, inv));
 }
 
-// gamma at mode k of the length-2H sequence (f_k = k f_samp / (2H); a_0 = a_H = 0)
-struct CzDet { float s2, fscale, mal; };
+// A detector's sequence: gamma_k / sigma0^2 = r / (1 + r) at mode k of the
+// length-2H sequence (f_k = k f_samp / (2H); a_0 = a_H = 0), in units of the
+// power of two `unit` at or below its largest value (the first or the last:
+// it is monotone in k).
+struct CzDet { float unit, fscale, mal; };
+__device__ __forceinline__ float cz_ratio(const CzDet &c, int kk) {
+    const float r = exp2f(c.mal * log2f(static_cast<float>(kk) * c.fscale));
+    return 1.0f / (1.0f + 1.0f / r);          // r / (1 + r), also for r = 0 or inf
+}
+__device__ __forceinline__ CzDet cz_det(const double *__restrict__ psd, int det, int href, double fsamp, float &peak) {
+    CzDet c{1.0f, static_cast<float>(fsamp / (2.0 * href * psd[3 * det + 1])), static_cast<float>(-psd[3 * det + 2])};
+    const float lo = cz_ratio(c, 1), hi = cz_ratio(c, href - 1);
+    peak = lo + hi >= 0.f ? fmaxf(lo, hi) : lo + hi;                   // NaN where one of them is
+    c.unit = __uint_as_float(max(__float_as_uint(peak >= 0.f ? peak : 0.f) & 0x7f800000u, 0x00800000u));
+    return c;
+}
+// in units; a value that is not a number would spread to the partner: zero
+// (the detector's kernel is marked by cz_scale)
 __device__ __forceinline__ float cz_gamma(const CzDet &c, int k, int href) {
     const int kk = k <= href ? k : 2 * href - k;
     if (kk == 0 || kk >= href) return 0.f;
-    const float r = exp2f(c.mal * log2f(static_cast<float>(kk) * c.fscale));
-    return c.s2 / (1.0f + 1.0f / r);          // sigma0^2 r / (1 + r), also for r = 0 or inf
+    const float g = cz_ratio(c, kk) * __uint_as_float(0x7f000000u - __float_as_uint(c.unit));
+    return g >= 0.f ? g : 0.f;
+}
+// what the transform's output is multiplied by: NaN for parameters that give
+// no kernel (the tables then end at order 0 and the detector goes without)
+__device__ __forceinline__ float cz_scale(const CzDet &c, float peak, double sig0) {
+    const float s2 = static_cast<float>(sig0 * sig0);
+    return peak >= 0.f && s2 < __int_as_float(0x7f800000) ? s2 * c.unit : __int_as_float(0x7fffffff);
 }
 
 // One radix-R Stockham pass (R = 8 A, forward DFT) over the length-M sequence
@@ -84,8 +109,9 @@ __device__ __forceinline__ float cz_gamma(const CzDet &c, int k, int href) {
 // rows r = 8 n1 + n2 in registers, a table twiddle, one exchange through
 // shared memory, and 8-point DFTs over n2.  FIRST evaluates gamma in place
 // of a load (and writes through shared memory, since its outputs of one j
-// are consecutive); LAST keeps the lags d < H only, real part to the first
-// detector's kernel, imaginary part to the second's.
+// are consecutive), and leaves the detectors' scales; LAST keeps the lags
+// d < H only, real part to the first detector's kernel, imaginary part to the
+// second's, each times its scale.
 // Every radix-R pass reads and writes the sequence once, so R up to 128
 // takes three passes where radix 4 took ten; per point one sincospif in
 // eight instead of three in four.  Bound: L2 bandwidth and the gamma
@@ -95,7 +121,7 @@ __device__ __forceinline__ float cz_gamma(const CzDet &c, int k, int href) {
 template <int A, bool FIRST, bool LAST>
 __global__ void __launch_bounds__(CZ_T)
 k_cz_fft(const float2 *__restrict__ src, float2 *__restrict__ dst, const double *__restrict__ psd, int ndet, int href,
-         double fsamp, int Ns, float *__restrict__ hout)
+         double fsamp, int Ns, float *__restrict__ scale, float *__restrict__ hout)
 {
     constexpr int R = 8 * A;
     constexpr int IT = (A * CZ_C + CZ_T - 1) / CZ_T;
@@ -112,9 +138,10 @@ k_cz_fft(const float2 *__restrict__ src, float2 *__restrict__ dst, const double 
     }
     if (FIRST && threadIdx.x < 2) {
         const int det = min(2 * pair + static_cast<int>(threadIdx.x), ndet - 1);
-        const double sig0 = psd[3 * det], fk = psd[3 * det + 1];
-        s_det[threadIdx.x] = CzDet{static_cast<float>(sig0 * sig0), static_cast<float>(fsamp / (2.0 * href * fk)),
-                                   static_cast<float>(-psd[3 * det + 2])};
+        float peak;
+        const CzDet c = cz_det(psd, det, href, fsamp, peak);
+        s_det[threadIdx.x] = c;
+        if (blockIdx.x == 0) scale[det] = cz_scale(c, peak, psd[3 * det]);
     }
     __syncthreads();
     {
@@ -167,6 +194,7 @@ k_cz_fft(const float2 *__restrict__ src, float2 *__restrict__ dst, const double 
         RDft<8, false, float2>::run(u[i]);
     }
     if (FIRST) __syncthreads();                // t is reused for the outputs
+    const float sc0 = LAST ? scale[2 * pair] : 0.f, sc1 = LAST ? scale[min(2 * pair + 1, ndet - 1)] : 0.f;
     float2 *y = dst + static_cast<int64_t>(pair) * M;
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
@@ -182,8 +210,8 @@ k_cz_fft(const float2 *__restrict__ src, float2 *__restrict__ dst, const double 
                 const int d = j + r * Ns;      // Ns = M/R: j < Ns
                 if (d < href) {
                     const float inv = 1.0f / static_cast<float>(M);              // a power of two
-                    hout[static_cast<int64_t>(2 * pair) * href + d] = u[i][k2].x * inv;
-                    if (2 * pair + 1 < ndet) hout[static_cast<int64_t>(2 * pair + 1) * href + d] = u[i][k2].y * inv;
+                    hout[static_cast<int64_t>(2 * pair) * href + d] = u[i][k2].x * inv * sc0;
+                    if (2 * pair + 1 < ndet) hout[static_cast<int64_t>(2 * pair + 1) * href + d] = u[i][k2].y * inv * sc1;
                 }
             } else {
                 y[(j - k) * R + k + r * Ns] = u[i][k2];
@@ -437,9 +465,15 @@ static void cz_fft_pass(const Plan &p, int lgR, const float2 *src, float2 *dst, 
     static_assert(CZ_C == 32, "grid");
     KTIME(TOD_KT_TOEP_KERNEL);
     switch (lgR) {
-    case 5: k_cz_fft<4, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, h); break;
-    case 6: k_cz_fft<8, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, h); break;
-    default: k_cz_fft<16, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, h); break;
+    case 5:
+        k_cz_fft<4, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, p.czscale, h);
+        break;
+    case 6:
+        k_cz_fft<8, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, p.czscale, h);
+        break;
+    default:
+        k_cz_fft<16, FIRST, LAST><<<grid, CZ_T, 0, st>>>(src, dst, psd, p.ndet, p.cz_href, p.fsamp, Ns, p.czscale, h);
+        break;
     }
 }
 
