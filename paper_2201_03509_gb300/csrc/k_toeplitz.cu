@@ -523,14 +523,20 @@ cudaError_t launch_toeplitz_prep(const Plan &p, const double *psd, cudaStream_t 
 // of the preparation's chain (0.2 to 0.3 ms) is hidden.  Every later kernel of
 // the caller's stream waits for it (the draw waits for prep_done), so nothing
 // on the side stream outlives the call's work there, and psd may be freed in
-// stream order as before.
+// stream order as before.  After an error there is no draw to wait: the
+// caller's stream is joined here (a capture keeps no loose branch; by the host
+// if even the event fails), and the first error returned.
 cudaError_t fork_toeplitz_prep(const Plan &p, const double *psd, cudaStream_t st)
 {
     cudaError_t e = cudaEventRecord(p.prep_fork, st);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(p.prep_stream, p.prep_fork, 0);
-    if (e == cudaSuccess) e = launch_toeplitz_prep(p, psd, p.prep_stream);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(p.prep_stream, p.prep_fork, 0)) != cudaSuccess) return e;
+    e = launch_toeplitz_prep(p, psd, p.prep_stream);
     const cudaError_t e2 = cudaEventRecord(p.prep_done, p.prep_stream);
-    return e == cudaSuccess ? e2 : e;
+    if (e == cudaSuccess) e = e2;
+    if (e != cudaSuccess && (e2 != cudaSuccess || cudaStreamWaitEvent(st, p.prep_done, 0) != cudaSuccess))
+        cudaStreamSynchronize(p.prep_stream);
+    return e;
 }
 
 }  // namespace tg
