@@ -21,6 +21,7 @@
 // a CTA holds one tile in shared memory, passes are separate grid-wide
 // phases, and the intermediate goes through L2/HBM.
 #include <cooperative_groups.h>
+#include <type_traits>
 #include "fft_reg.cuh"
 
 namespace cgrp = cooperative_groups;
@@ -419,12 +420,17 @@ __device__ __forceinline__ void col_forward(const TxCtx &X, V *b0, V *b1, typena
 // Inverse column pass: the tile's Y values (every load of a thread in
 // flight), the conjugate twiddle, inverse FFT of the columns; then for every
 // unit out(D, j, centre, v, fb) with v its samples, D = ld(j, centre, fb) issued
-// ahead of the transform (the flag bits are read while the tile loads).
-template <class V, class Ld, class Out>
+// ahead of the transform (the flag bits are read while the tile loads).  Where
+// again() then asks for it, the thread's units are gone through once more, as
+// redo(D, j, centre, v, fb).
+struct NoRedo {
+    __device__ __forceinline__ bool again() const { return false; }
+};
+template <class V, class Ld, class Out, class Redo = NoRedo>
 __device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
                                             const typename PairOf<V>::Z *__restrict__ Y,
                                             const typename PairOf<V>::Z *__restrict__ twb,
-                                            const uint32_t *__restrict__ fl, Ld ld, Out out)
+                                            const uint32_t *__restrict__ fl, Ld ld, Out out, Redo redo = Redo())
 {
     typedef typename PairOf<V>::Z Z;
     typedef typename VecT<V>::S S;
@@ -490,22 +496,35 @@ __device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
     __syncthreads();
     V *R = sp_transform<true, TX_T, true>(b0, b1, m1, X.L.s1, X.L.nr1, X.L.lgW, 0, T.tw1);
     if (C.c < 0) return;
-#pragma unroll
-    for (int r = 0; r < TX_ROWS; ++r) {
+    // the units of the thread's r-th row
+    const auto units = [&](int r, const auto &Da, const auto &Db, auto &fn) {
         const int j1 = C.row(r);
-        if (j1 >= C.m1h) continue;
         const uint32_t fb = fnib >> (8 * r);
         const V ea = sld(R + j1 * TP + C.i), eb = sld(R + (m1 - 1 - j1) * TP + C.i);
         if (C.centre(j1)) {
             const S v[4] = {ea.x.a, ea.y.a, S(0), S(0)};
-            out(D[r][0], j1 * m2 + C.c, true, v, fb & 15u);
+            fn(Da, j1 * m2 + C.c, true, v, fb & 15u);
         } else {
             const S v[4] = {ea.x.a, eb.y.b, ea.y.a, eb.x.b};
-            out(D[r][0], j1 * m2 + C.c, false, v, fb & 15u);
+            fn(Da, j1 * m2 + C.c, false, v, fb & 15u);
         }
         if (C.second(j1)) {
             const S v[4] = {ea.x.b, eb.y.a, ea.y.b, eb.x.a};
-            out(D[r][1], j1 * m2 + C.c2, false, v, (fb >> 4) & 15u);
+            fn(Db, j1 * m2 + C.c2, false, v, (fb >> 4) & 15u);
+        }
+    };
+#pragma unroll
+    for (int r = 0; r < TX_ROWS; ++r)
+        if (C.row(r) < C.m1h) units(r, D[r][0], D[r][1], out);
+    if constexpr (!std::is_same<Redo, NoRedo>::value) {
+        if (!redo.again()) return;
+#pragma unroll 1
+        for (int r = 0; C.row(r) < C.m1h; ++r) {
+            const int j1 = C.row(r);
+            const uint32_t fb = fnib >> (8 * r);
+            const auto Da = ld(j1 * m2 + C.c, C.centre(j1), fb & 15u);
+            const auto Db = C.second(j1) ? ld(j1 * m2 + C.c2, false, (fb >> 4) & 15u) : Da;
+            units(r, Da, Db, redo);
         }
     }
 }
@@ -531,10 +550,15 @@ __device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
 // takes elements k2 and m2 - 1 - k2 together: lane a the pair based in row p,
 // lane b the pair based in row m1 - p.  Rows 0 and m1/2 pair with themselves
 // (p = 0).  The conjugates of P and Q are carried, so no sign is flipped.
+//
+// stop(), asked of every thread after the modes: where one says so the pass
+// ends there, Y as it was, and returns false.
 // ---------------------------------------------------------------------------
-template <bool NORM, class V, class Pre, class F>
-__device__ __forceinline__ void row_pass(const TxCtx &X, V *b0, V *b1, typename PairOf<V>::Z *__restrict__ Y,
-                                         const typename PairOf<V>::Z *__restrict__ twb, Pre pre, F f)
+struct NeverStop {};
+template <bool NORM, class V, class Pre, class F, class Stop = NeverStop>
+__device__ __forceinline__ bool row_pass(const TxCtx &X, V *b0, V *b1, typename PairOf<V>::Z *__restrict__ Y,
+                                         const typename PairOf<V>::Z *__restrict__ twb, Pre pre, F f,
+                                         Stop stop = Stop())
 {
     typedef typename PairOf<V>::Z Z;
     typedef typename VecT<V>::S S;
@@ -634,7 +658,8 @@ __device__ __forceinline__ void row_pass(const TxCtx &X, V *b0, V *b1, typename 
             }
         }
     }
-    __syncthreads();
+    if constexpr (std::is_same<Stop, NeverStop>::value) __syncthreads();
+    else if (__syncthreads_or(stop())) return false;
     const V *Ri = sp_transform<true, TX_T, false>(R, Fr, m2, X.L.s2, X.L.nr2, X.L.lgS, m2p, T.tw2);
     for (int pl = 0; pl < nr; ++pl) {
         const int p = p0 + pl;
@@ -651,6 +676,7 @@ __device__ __forceinline__ void row_pass(const TxCtx &X, V *b0, V *b1, typename 
             }
         }
     }
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -923,13 +949,20 @@ template <class V> struct Chi2Tx {
 };
 
 // Sums over a CTA's modes or samples, one per lane: FP32 double-words (2^-44
-// relative; FP64 adds issue at 1/64 of the FP32 rate) or FP64
+// relative; FP64 adds issue at 1/64 of the FP32 rate) or FP64.  A double-word
+// sum reaches 3.4e38, and an infinite term leaves NaN in its tail: what is
+// not finite the caller adds up again in FP64.
 template <class C> struct LaneSum;
 template <> struct LaneSum<PF> {
     PAcc a = pacc_zero();
     __device__ __forceinline__ void add(PF v) { pacc_add(a, v); }
     __device__ __forceinline__ void add_prod(PF x, PF y) { pacc_add_prod(a, x, y); }
     __device__ __forceinline__ double total() const { return acc_value(pacc_total(a)); }
+};
+struct WideSum {                          // FP32 terms added in FP64
+    double a = 0.0;
+    __device__ __forceinline__ void add(PF v) { a += static_cast<double>(v.a) + static_cast<double>(v.b); }
+    __device__ __forceinline__ double total() const { return a; }
 };
 template <> struct LaneSum<PD> {
     double a = 0.0;
@@ -986,6 +1019,7 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
     typedef typename VecT<V>::C C;
     extern __shared__ __align__(16) CD2 tx_smem64[];
     __shared__ TxCtx X;
+    constexpr bool kF64 = sizeof(S) == sizeof(double);
     __shared__ double s_red[4 * (TX_T / 32)], s_out[4];
     V *b0 = reinterpret_cast<V *>(tx_smem64), *b1 = b0 + TX_PAIRS;
     int cur = -1;
@@ -999,11 +1033,10 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
         const S s2 = sig0 * sig0;
         const S d1 = S(2) / sig0, d2 = -s2 * al / fk;
         const int n = X.L.n, m = X.L.m;
-        LaneSum<C> sum[4];            // 2 L, dL/dsigma0, dL/dfknee, dL/dalpha
         // the modes k0, k1 of coefficients r: r / P, their terms added; in
-        // FP64 all but ln P (P in the mask's lanes, 1 elsewhere, left in Pm)
-        constexpr bool kF64 = sizeof(S) == sizeof(double);
-        const auto mode_terms = [&](int k0, int k1, int mask, C r, C &Pm) -> C {
+        // FP64 all but ln P (P in the mask's lanes, 1 elsewhere, left in Pm).  The
+        // sums: 2 L, dL/dsigma0, dL/dfknee, dL/dalpha
+        const auto mode_terms = [&](auto &sum, int k0, int k1, int mask, C r, C &Pm) -> C {
             // ln(f/fk) = ln k + ln(fsamp/(2 n fk)); P = s2 (1 + e^{alpha ln(f/fk)})
             const C lr = pset(log(static_cast<S>(max(k0, 1))) + lfs, log(static_cast<S>(max(k1, 1))) + lfs);
             const C pw = pset(exp(al * lr.a), exp(al * lr.b));
@@ -1028,11 +1061,11 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
             sum[3].add(t3);
             return rP;
         };
-        row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, [](V *) {}, [&](int k0, int k1, int mask, V Rv, V) {
+        const auto modes = [&](auto &sum, int k0, int k1, int mask, V Rv) {
             const int on = (k0 ? 1 : 0) | (k1 ? 2 : 0);         // the offset mode does not enter
             C P0, P1;
-            const C x = mode_terms(k0, k1, mask & on, Rv.x, P0);
-            const C y = mode_terms(k0 ? n - k0 : m, k1 ? n - k1 : m, mask, Rv.y, P1);
+            const C x = mode_terms(sum, k0, k1, mask & on, Rv.x, P0);
+            const C y = mode_terms(sum, k0 ? n - k0 : m, k1 ? n - k1 : m, mask, Rv.y, P1);
             if constexpr (kF64) {
                 // one logarithm for the four modes (an FP64 one takes about 30
                 // operations, at 1/64 of the FP32 rate: 25 scans of 4 x 65536,
@@ -1047,8 +1080,32 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
                 }
             }
             return vmake<V>(on == 3 ? x : pmask(x, on), y);
-        });
-        const double acc[4] = {0.5 * sum[0].total(), sum[1].total(), sum[2].total(), sum[3].total()};
+        };
+        double acc[4];
+        const auto totals = [&](auto &sum) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[k] = (k == 0 ? 0.5 : 1.0) * sum[k].total();
+        };
+        const auto none = [](V *) {};
+        LaneSum<C> sum[4];
+        const auto pass = [&](int k0, int k1, int mask, V Rv, V) { return modes(sum, k0, k1, mask, Rv); };
+        if constexpr (kF64) {
+            row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, none, pass);
+            totals(sum);
+        } else {
+            // a sum past FP32's range, or an infinite term: the tile once more,
+            // its terms added in FP64
+            const auto stop = [&] {
+                totals(sum);
+                return !(isfinite(acc[0]) && isfinite(acc[1]) && isfinite(acc[2]) && isfinite(acc[3]));
+            };
+            if (!row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, none, pass, stop)) {
+                WideSum wide[4];
+                row_pass<false>(X, b0, b1, a.Y, a.tw + X.L.twb, none,
+                                [&](int k0, int k1, int mask, V Rv, V) { return modes(wide, k0, k1, mask, Rv); });
+                totals(wide);
+            }
+        }
         block_sums_d<4>(acc, s_red, s_out);
         if (threadIdx.x < 4) a.part[4 * static_cast<int64_t>(a.item0 + it) + threadIdx.x] = s_out[threadIdx.x];
     }
@@ -1070,11 +1127,12 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
         const int64_t o = X.o;
         LaneSum<C> sum;
         struct U4 { S sx[4]; };
-        col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [&](int j, bool ctr, uint32_t) {
+        const auto load = [&](int j, bool ctr, uint32_t) {
             U4 D;
             ld4s<S>(a.s, o + 4 * static_cast<int64_t>(j), ctr, D.sx);
             return D;
-        }, [&](const U4 &D, int j, bool ctr, const S (&u)[4], uint32_t fb) {
+        };
+        const auto unit = [&](const U4 &D, int j, bool ctr, const S (&u)[4], uint32_t fb) {
             const S v[4] = {(fb & 1) ? S(0) : u[0], (fb & 2) ? S(0) : u[1], (fb & 4) ? S(0) : u[2],
                             (fb & 8) ? S(0) : u[3]};
             // at the centre the last two samples are zero
@@ -1091,8 +1149,30 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
                     for (int s = 0; s < (ctr ? 2 : 4); ++s) vs[s] = v[s];
                 }
             }
-        });
-        const double acc[1] = {-sum.total()};
+        };
+        double total;
+        if constexpr (sizeof(S) == sizeof(float)) {
+            // a sum past FP32's range, or with a product past it: formed again in FP64
+            struct Again {
+                LaneSum<C> *sum;
+                double *t;
+                __device__ __forceinline__ bool again() const {
+                    *t = sum->total();
+                    if (isfinite(*t)) return false;
+                    *t = 0.0;
+                    return true;
+                }
+                __device__ __forceinline__ void operator()(const U4 &D, int, bool, const S (&u)[4], uint32_t fb) const {
+                    for (int s = 0; s < 4; ++s) *t += static_cast<double>(D.sx[s]) * ((fb >> s & 1) ? 0.0 : u[s]);
+                }
+            };
+            total = 0.0;                              // threads without a column add nothing
+            col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, load, unit, Again{&sum, &total});
+        } else {
+            col_inverse(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, load, unit);
+            total = sum.total();
+        }
+        const double acc[1] = {-total};
         block_sums_d<1>(acc, s_red, s_out);
         if (threadIdx.x == 0) a.part[4 * static_cast<int64_t>(a.item0 + it) + 1] = s_out[0];
     }
