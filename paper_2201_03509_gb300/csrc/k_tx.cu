@@ -555,6 +555,25 @@ __device__ __forceinline__ void col_inverse(const TxCtx &X, V *b0, V *b1,
 // ends there, Y as it was, and returns false.
 // ---------------------------------------------------------------------------
 struct NeverStop {};
+// A CTA's threads as groups of whole warps, a power of two of threads at least
+// n wide: a loop over the n elements of each of several rows takes the rows by
+// groups, so that short rows keep the CTA at work (one row after the other left
+// seven of eight warps idle in the split at m2 = 64: FP64 chi^2 of 16 x 4096
+// samples 955 us, 432 so; the gain of 800 x 2000 89 us, 74 so).  A warp has one
+// row: groups of fewer threads than a warp cost the long rows registers (gain of
+// 72 x 225k samples 325 us, 308 so, 311 with one row after the other).
+struct RowGroups {
+    int first, step, row, nrow;
+    __device__ __forceinline__ explicit RowGroups(int n) {
+        const int lg = min(8, max(5, 32 - __clz(n - 1)));
+        first = threadIdx.x & ((1 << lg) - 1);
+        step = 1 << lg;
+        row = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> lg), 0);      // uniform, and known to be
+        nrow = __shfl_sync(0xffffffffu, TX_T >> lg, 0);
+    }
+};
+static_assert(TX_T == 256, "a group is at most the CTA");
+
 template <bool NORM, class V, class Pre, class F, class Stop = NeverStop>
 __device__ __forceinline__ bool row_pass(const TxCtx &X, V *b0, V *b1, typename PairOf<V>::Z *__restrict__ Y,
                                          const typename PairOf<V>::Z *__restrict__ twb, Pre pre, F f,
@@ -566,22 +585,22 @@ __device__ __forceinline__ bool row_pass(const TxCtx &X, V *b0, V *b1, typename 
     const int m = X.L.m, m1 = X.L.m1, m2 = X.L.m2, m2p = X.L.m2p, TR = X.L.TR;
     const int p0 = X.blk * TR, nr = min(TR, X.L.P1 - p0);
     const bool odd = m1 & 1;
-    const int tid = threadIdx.x;
+    const RowGroups W(m2), H((m2 + 1) >> 1);
     Z *Yq = Y + X.yb;
-    for (int pl = 0; pl < TR; ++pl) {
+    for (int pl = W.row; pl < TR; pl += W.nrow) {
         const int p = p0 + pl;
         V *dst = b0 + pl * m2p;
         if (pl >= nr) {
-            for (int k2 = tid; k2 < m2; k2 += TX_T) sst(dst + k2, vzero<V>());
+            for (int k2 = W.first; k2 < m2; k2 += W.step) sst(dst + k2, vzero<V>());
         } else if (odd && p == 0) {
             const Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
-            for (int k2 = tid; k2 < m2; k2 += TX_T) {
+            for (int k2 = W.first; k2 < m2; k2 += W.step) {
                 const Z z = y[k2];
                 sst(dst + k2, vmake<V>(pset(z.x, S(0)), pset(z.y, S(0))));
             }
         } else {
             const Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
-            for (int k2 = tid; k2 < m2; k2 += TX_T) {
+            for (int k2 = W.first; k2 < m2; k2 += W.step) {
                 cp_async(&dst[k2].x, y + k2);
                 cp_async(&dst[k2].y, y + m2 + k2);
             }
@@ -597,13 +616,13 @@ __device__ __forceinline__ bool row_pass(const TxCtx &X, V *b0, V *b1, typename 
         __syncthreads();
     }
     const C h = pdup<C>(static_cast<S>(0.70710678118654752440));
-    for (int pl = 0; pl < nr; ++pl) {
+    for (int pl = H.row; pl < nr; pl += H.nrow) {
         const int p = p0 + pl;
         const int ra = p, rb = p ? m1 - p : (odd ? 0 : m1 >> 1);
         V *t = R + pl * m2p, *nt = Fr + pl * m2p;
         const V A1 = vtwo<V>(vld(T.sa1 + ra), vld(T.sa1 + rb)), A5 = vtwo<V>(vld(T.sa5 + ra), vld(T.sa5 + rb));
         const int cnt = p ? (m2 + 1) >> 1 : (m2 >> 1) + 1;
-        for (int k2 = tid; k2 < cnt; k2 += TX_T) {
+        for (int k2 = H.first; k2 < cnt; k2 += H.step) {
             const int q = m2 - 1 - k2;                       // partner element (p = 0: lane b)
             const int q0 = k2 ? m2 - k2 : 0;                 // p = 0: lane a's partner
             int mb = 3, mp = 3;
@@ -661,15 +680,15 @@ __device__ __forceinline__ bool row_pass(const TxCtx &X, V *b0, V *b1, typename 
     if constexpr (std::is_same<Stop, NeverStop>::value) __syncthreads();
     else if (__syncthreads_or(stop())) return false;
     const V *Ri = sp_transform<true, TX_T, false>(R, Fr, m2, X.L.s2, X.L.nr2, X.L.lgS, m2p, T.tw2);
-    for (int pl = 0; pl < nr; ++pl) {
+    for (int pl = W.row; pl < nr; pl += W.nrow) {
         const int p = p0 + pl;
         const V *src = Ri + pl * m2p;
         if (odd && p == 0) {
             Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
-            for (int k2 = tid; k2 < m2; k2 += TX_T) y[k2] = Z{src[k2].x.a, src[k2].y.a};
+            for (int k2 = W.first; k2 < m2; k2 += W.step) y[k2] = Z{src[k2].x.a, src[k2].y.a};
         } else {
             Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
-            for (int k2 = tid; k2 < m2; k2 += TX_T) {
+            for (int k2 = W.first; k2 < m2; k2 += W.step) {
                 const V v = sld(src + k2);
                 y[k2] = Z{v.x.a, v.x.b};
                 y[m2 + k2] = Z{v.y.a, v.y.b};
