@@ -283,9 +283,11 @@ __device__ __forceinline__ int y_plane(int m1, int p) { return (m1 & 1) ? 2 * (p
 constexpr int TX_ROWS = 4;
 // CTAs per SM of the column passes and the chi^2 passes: at three (80
 // registers) the four rows of loads that a thread keeps in flight spill; two
-// at 128 registers are faster but for the scatter, which loads only flags
-// (82M samples: k_gain_cols 359 -> 343 us, k_nc_gather_final 476 -> 418; chi^2 rows of 52M
-// 1093 -> 840 us, there with a grid that is resident at once).
+// at 128 registers are faster (82M samples: k_gain_cols 359 -> 343 us,
+// k_nc_gather_final 476 -> 418; chi^2 rows of 52M 1093 -> 840 us, there with a
+// grid that is resident at once).  The scatter, which holds no samples, keeps
+// three (the draw of 72 x 225k samples without its preparation 2009 us; 2102
+// with two).
 constexpr int TX_CTAS_COL = 2;
 struct ColThread {
     int m, m1, m2, TP, np, i, c, c2, r0, rstep, m1h;
@@ -324,12 +326,55 @@ __device__ __forceinline__ uint32_t unit_flags(const ColThread &C, const uint32_
     return nib;
 }
 
+// The second half of a forward column pass, the tile in b0: the column FFTs,
+// the four-step twiddle W_m^{c k1}, and the tile out to Y.
+template <class V>
+__device__ __forceinline__ void col_forward_out(const TxCtx &X, const ColThread &C, V *b0, V *b1,
+                                                typename PairOf<V>::Z *__restrict__ Y,
+                                                const typename PairOf<V>::Z *__restrict__ twb)
+{
+    typedef typename PairOf<V>::Z Z;
+    const int m1 = C.m1, m2 = C.m2, TP = C.TP;
+    __syncthreads();
+    const TwB<V> T(twb, X.L);
+    V *R = sp_transform<false, TX_T, true>(b0, b1, m1, X.L.s1, X.L.nr1, X.L.lgW, 0, T.tw1);
+    if (C.c < 0) return;
+    Z *Yq = Y + X.yb;
+    // W_m^{c p} from the table at the thread's first row, then by steps of
+    // W_m^{c rstep} (at most three products); row m1 - p takes W_m2^c conj(W_m^{c p})
+    const V wc = vtwo<V>(Z{vld(T.tw2 + C.c).x.a, vld(T.tw2 + C.c).y.a}, Z{vld(T.tw2 + C.c2).x.a, vld(T.tw2 + C.c2).y.a});
+    V w = C.r0 < m1 ? vtwo<V>(T.w4(C.c * C.r0), T.w4(C.c2 * C.r0)) : vzero<V>();
+    const V wstep = C.rstep < m1 ? vtwo<V>(T.w4(C.c * C.rstep), T.w4(C.c2 * C.rstep)) : vzero<V>();
+#pragma unroll
+    for (int r = 0; r < TX_ROWS; ++r) {
+        const int p = C.row(r);
+        if (p >= C.m1h) break;
+        const V za = vmul(sld(R + p * TP + C.i), w);
+        if (p == 0 && (m1 & 1)) {
+            Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
+            y[C.c] = Z{za.x.a, za.y.a};
+            if (C.c2 != C.c) y[C.c2] = Z{za.x.b, za.y.b};
+        } else {
+            const int pr = p ? m1 - p : m1 >> 1;
+            const V wr = p ? vmul<true>(wc, w) : vtwo<V>(T.w4(C.c * pr), T.w4(C.c2 * pr));
+            const V zb = vmul(sld(R + pr * TP + C.i), wr);
+            Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
+            y[C.c] = Z{za.x.a, zb.x.a};
+            y[m2 + C.c] = Z{za.y.a, zb.y.a};
+            if (C.c2 != C.c) {
+                y[C.c2] = Z{za.x.b, zb.x.b};
+                y[m2 + C.c2] = Z{za.y.b, zb.y.b};
+            }
+        }
+        w = vmul(w, wstep);
+    }
+}
+
 // Forward column pass.  D = ld(j, centre, fb) issues a unit's loads (UNR rows
 // per thread at a time; fb: the unit's flag bits, from fl at sample o + 4j,
 // read ahead), val(D, j, centre, fb, wa, wb, v) gives its samples
 // v[0..3] (two at the centre).  With NORM, pre(tile) first fills the tile
-// and wa, wb are the tile's values at z_j and z_{m-1-j}.  Then the column
-// FFTs, the four-step twiddle W_m^{c k1}, and the tile out to Y.
+// and wa, wb are the tile's values at z_j and z_{m-1-j}.
 template <bool NORM, int UNR, class V, class Pre, class Ld, class Val>
 __device__ __forceinline__ void col_forward(const TxCtx &X, V *b0, V *b1, typename PairOf<V>::Z *__restrict__ Y,
                                             const typename PairOf<V>::Z *__restrict__ twb,
@@ -382,39 +427,7 @@ __device__ __forceinline__ void col_forward(const TxCtx &X, V *b0, V *b1, typena
             }
         }
     }
-    __syncthreads();
-    const TwB<V> T(twb, X.L);
-    V *R = sp_transform<false, TX_T, true>(b0, b1, m1, X.L.s1, X.L.nr1, X.L.lgW, 0, T.tw1);
-    if (C.c < 0) return;
-    Z *Yq = Y + X.yb;
-    // W_m^{c p} from the table at the thread's first row, then by steps of
-    // W_m^{c rstep} (at most three products); row m1 - p takes W_m2^c conj(W_m^{c p})
-    const V wc = vtwo<V>(Z{vld(T.tw2 + C.c).x.a, vld(T.tw2 + C.c).y.a}, Z{vld(T.tw2 + C.c2).x.a, vld(T.tw2 + C.c2).y.a});
-    V w = C.r0 < m1 ? vtwo<V>(T.w4(C.c * C.r0), T.w4(C.c2 * C.r0)) : vzero<V>();
-    const V wstep = C.rstep < m1 ? vtwo<V>(T.w4(C.c * C.rstep), T.w4(C.c2 * C.rstep)) : vzero<V>();
-#pragma unroll
-    for (int r = 0; r < TX_ROWS; ++r) {
-        const int p = C.row(r);
-        if (p >= C.m1h) break;
-        const V za = vmul(sld(R + p * TP + C.i), w);
-        if (p == 0 && (m1 & 1)) {
-            Z *y = Yq + static_cast<int64_t>(m1 - 1) * m2;
-            y[C.c] = Z{za.x.a, za.y.a};
-            if (C.c2 != C.c) y[C.c2] = Z{za.x.b, za.y.b};
-        } else {
-            const int pr = p ? m1 - p : m1 >> 1;
-            const V wr = p ? vmul<true>(wc, w) : vtwo<V>(T.w4(C.c * pr), T.w4(C.c2 * pr));
-            const V zb = vmul(sld(R + pr * TP + C.i), wr);
-            Z *y = Yq + static_cast<int64_t>(y_plane(m1, p)) * m2;
-            y[C.c] = Z{za.x.a, zb.x.a};
-            y[m2 + C.c] = Z{za.y.a, zb.y.a};
-            if (C.c2 != C.c) {
-                y[C.c2] = Z{za.x.b, zb.x.b};
-                y[m2 + C.c2] = Z{za.y.b, zb.y.b};
-            }
-        }
-        w = vmul(w, wstep);
-    }
+    col_forward_out(X, C, b0, b1, Y, twb);
 }
 
 // Inverse column pass: the tile's Y values (every load of a thread in
@@ -1679,26 +1692,43 @@ __device__ void nc_x0_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1)
 }
 
 // CG column pass: z = E vec (the flagged samples' entries of vec, zero
-// elsewhere), forward columns.
+// elsewhere), forward columns.  The thread zeroes its tile elements and places
+// the entries of its flagged units, about one sample in fifty: no value is held
+// for the others (four rows of values, and the lookup of their ranks written out
+// eight times, spilled 412 bytes at 80 registers: the draw of 72 x 225k samples
+// without its preparation 2107 -> 2009 us).
+// Sample s of unit (j1, c): z_j = (x_0, x_2) in lane a of row j1, its mirror
+// z_{m-1-j} = (x_3, x_1) in lane b of row m1-1-j1; of unit (j1, c2) the lanes
+// change places; a column that is its own mirror fills both.
 __device__ void nc_scatter_cols(const NcorrTx &a, const TxCtx &X, CF2 *b0, CF2 *b1, const float *vec)
 {
     const int64_t o = X.o, obase = a.off[a.q0], w_lo = obase >> 5;
-    col_forward<false, 4>(X, b0, b1, a.Y, a.tw + X.L.twb, a.flags, [](CF2 *) {},
-                [&](int j, bool, uint32_t fb) {
-                    // the unit's flagged entries of vec (a rank lookup only where flagged)
-                    const int64_t t = 4 * static_cast<int64_t>(j);
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    while (fb) {
-                        const int u = __ffs(fb) - 1;
-                        fb &= fb - 1;
-                        const float val = vec[flag_rank(a.flags, a.wpre, w_lo, obase, o + t + u)];
-                        if (u == 0) v.x = val; else if (u == 1) v.y = val; else if (u == 2) v.z = val; else v.w = val;
-                    }
-                    return v;
-                },
-                [&](const float4 &D, int, bool, uint32_t, float2, float2, float (&v)[4]) {
-                    v[0] = D.x; v[1] = D.y; v[2] = D.z; v[3] = D.w;
-                });
+    const ColThread C(X.L, X.blk);
+    const int m1 = C.m1, TP = C.TP;
+    uint32_t fnib = unit_flags(C, a.flags, o);
+    for (int j1 = C.r0; j1 < (C.c < 0 ? m1 : C.m1h); j1 += C.rstep) {
+        sst(b0 + j1 * TP + C.i, vzero<CF2>());
+        if (C.c >= 0) sst(b0 + (m1 - 1 - j1) * TP + C.i, vzero<CF2>());
+    }
+#pragma unroll 1
+    for (int k = 0; fnib; ++k, fnib >>= 4) {
+        const uint32_t fb = fnib & 15u;
+        if (!fb) continue;
+        const int j1 = C.row(k >> 1), side = k & 1;
+        const int64_t t = o + 4 * static_cast<int64_t>(j1 * C.m2 + (side ? C.c2 : C.c));
+        const float *v = vec + flag_rank(a.flags, a.wpre, w_lo, obase, t);
+        float *ea = reinterpret_cast<float *>(b0 + j1 * TP + C.i);
+        float *eb = reinterpret_cast<float *>(b0 + (m1 - 1 - j1) * TP + C.i);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (!(fb >> u & 1u)) continue;
+            const float val = v[__popc(fb & ((1u << u) - 1u))];
+            float *e = ((u & 1) ? eb : ea) + ((u == 1 || u == 2) ? 2 : 0);     // x_1, x_2: imaginary parts
+            if (C.c == C.c2) e[0] = e[1] = val;
+            else e[side ^ (u & 1)] = val;
+        }
+    }
+    col_forward_out(X, C, b0, b1, a.Y, a.tw + X.L.twb);
 }
 
 // CG row pass: times gamma (apply S), or times beta (the final B^{-1} E y,
