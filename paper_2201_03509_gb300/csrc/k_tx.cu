@@ -2582,12 +2582,14 @@ __global__ void __launch_bounds__(TX_T, 3) k_nc_update(NcorrTx a, int par)
     nc_update_listed(a, S, reinterpret_cast<float *>(tx_smem), a.count + (par ^ 1));
     nc_list_by_last(a);
 }
-// The iterations left after the launched ones, in one cooperative launch at
-// the passes' own occupancy: the passes over the listed detscans with grid
+// The iterations left after the launched ones, in one cooperative launch, two
+// CTAs per SM (at three, the bodies of all passes in one kernel spill 330 bytes:
+// with PREC_NONE, most of whose iterations run here, the draw of 40 x 115k
+// samples takes 3990 us, 3829 so; 72 x 225k 5312, 5226): the passes over the listed detscans with grid
 // barriers between them, the list rebuilt by CTA 0 after each update.  Then
 // the list of the detscans that ran the CG (for the correction), the
 // iteration counts, and the status of detscans left at x0 for want of CG room.
-__global__ void __launch_bounds__(TX_T, 3) k_nc_tail(NcorrTx a, int par)
+__global__ void __launch_bounds__(TX_T, 2) k_nc_tail(NcorrTx a, int par)
 {
     extern __shared__ __align__(16) CF2 tx_smem[];
     __shared__ NcShared S;
