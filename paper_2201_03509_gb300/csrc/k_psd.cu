@@ -18,6 +18,7 @@
 // the sums' CTAs take none and the
 // step's run on different warps at once.  27M samples: an evaluation 61 ->
 // 50 us, a step 17.7 -> 14.4 us.
+#include <algorithm>
 #include "common.cuh"
 #include "fft_reg.cuh"
 #include "internal.cuh"
@@ -80,13 +81,17 @@ __global__ void __launch_bounds__(PSD_T) k_psd_begin(const double *__restrict__ 
     if (acc_out) acc_out[det] = 0;
 }
 
-// partial S(alpha') of PSD_TILES consecutive element tiles (each one detscan's
-// samples t0..t1).  The tiles' parameters take a chain of three dependent loads,
-// longer than a tile's work: fetched once for all of them by the first lanes.
-constexpr int PSD_TILES = 4;
+// partial S(alpha') of `per` (at most PSD_TILES) consecutive element tiles (each
+// one detscan's samples t0..t1).  The tiles' parameters take a chain of three
+// dependent loads, longer than a tile's work: fetched once for all of them by
+// the first lanes.
+// Several tiles a CTA only once the grid keeps PSD_CTAS CTAs on every SM: below,
+// a tile's work is not shared with anything and the tiles of a CTA just wait for
+// one another.
+constexpr int PSD_TILES = 4, PSD_CTAS = 4;
 __global__ void __launch_bounds__(PSD_T) k_psd_sums(const float *__restrict__ spec, const int64_t *__restrict__ off,
                                                     const int32_t *__restrict__ tile_q,
-                                                    const int64_t *__restrict__ tile_t0, int ntile,
+                                                    const int64_t *__restrict__ tile_t0, int ntile, int per,
                                                     const double *__restrict__ wq, const float2 *__restrict__ lnk,
                                                     const double *__restrict__ state, int ndet,
                                                     double *__restrict__ part)
@@ -94,7 +99,7 @@ __global__ void __launch_bounds__(PSD_T) k_psd_sums(const float *__restrict__ sp
     struct Tile { const float *x; int k0, k1; float na, na_lo; double w; };
     __shared__ Tile s_tile[PSD_TILES];
     __shared__ double s_w[PSD_TILES][PSD_T / 32];
-    const int first = blockIdx.x * PSD_TILES, nt = min(PSD_TILES, ntile - first);
+    const int first = blockIdx.x * per, nt = min(per, ntile - first);
     if (threadIdx.x < nt) {
         const int q = tile_q[first + threadIdx.x];
         const int64_t t0 = tile_t0[first + threadIdx.x];
@@ -261,6 +266,7 @@ cudaError_t launch_noise_psd(const Plan &p, const float *spec, const double *psd
                              double step_lnfk, double step_al, double *psd_out, int32_t *acc_out,
                              double *loglike_out, cudaStream_t st)
 {
+    const int per = std::max(1, std::min(PSD_TILES, p.ntile / (PSD_CTAS * std::max(1, p.sm_count))));
     {
         KTIME(TOD_KT_PSD_STEP);
         k_psd_begin<<<p.ndet, PSD_T, 0, st>>>(psd_in, p.psd_state, p.ndet, p.nq, p.lnfs, p.psd_w, psd_out, acc_out);
@@ -270,9 +276,9 @@ cudaError_t launch_noise_psd(const Plan &p, const float *spec, const double *psd
         if (p.ntile > 0)
             {
                 KTIME(TOD_KT_PSD_SUMS);
-                k_psd_sums<<<(p.ntile + PSD_TILES - 1) / PSD_TILES, PSD_T, 0, st>>>(spec, p.off, p.tile_q, p.tile_t0,
-                                                      p.ntile, p.psd_w, p.lnk, p.psd_state,
-                                                      p.ndet, p.psd_part);
+                k_psd_sums<<<(p.ntile + per - 1) / per, PSD_T, 0, st>>>(spec, p.off, p.tile_q, p.tile_t0, p.ntile, per,
+                                                                        p.psd_w, p.lnk, p.psd_state, p.ndet,
+                                                                        p.psd_part);
             }
         {
             KTIME(TOD_KT_PSD_STEP);
