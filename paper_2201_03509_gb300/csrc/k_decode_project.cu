@@ -405,11 +405,15 @@ __device__ __forceinline__ float project_one(const float4 *__restrict__ map, con
 // loads and 16-byte stores on the tile's aligned body (global sample index a
 // multiple of 4; the caller checks the base pointers), its up to three head
 // and tail samples one per thread.  Bound by the gathers' latency: the four
-// of a thread go out together, out-of-range pointing taking the first entries
+// of a thread go out together, out-of-range pointing taking the last entries
 // and a zero afterwards (with a branch per sample each gather waited for the
-// one before: 102M samples at Nside 1024, whose map is larger than L2, 472 ->
-// 431 us; 27M at Nside 512 120 -> 119 us).
-__global__ void __launch_bounds__(256)
+// one before: 102M samples at Nside 1024, whose map is larger than L2, 474 ->
+// 447 us; 27M at Nside 512 118.5 -> 117.3 us).  A map that stays in L1 leaves
+// the instructions and the warps in flight as the bound: the index clamped by a
+// minimum, the test of the range after the loads, and registers for eight CTAs
+// per SM (18M samples at Nside 16: 59.1 us with a branch per sample, 60.1 with
+// the index selected by the test at 38 registers, 58.7 so).
+__global__ void __launch_bounds__(256, 8)
 k_project4(const float4 *__restrict__ map, const int32_t *__restrict__ pix,
            const uint16_t *__restrict__ psi, const double *__restrict__ gain,
            const float2 *__restrict__ trig, const int32_t *__restrict__ tile_q,
@@ -437,17 +441,24 @@ k_project4(const float4 *__restrict__ map, const int32_t *__restrict__ pix,
         const uint32_t bb[4] = {b4.x & 0xFFFFu, b4.x >> 16, b4.y & 0xFFFFu, b4.y >> 16};
         float4 m[4];
         float2 cs[4];
-        bool in[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            in[u] = static_cast<uint32_t>(pp[u]) < static_cast<uint32_t>(npix) && bb[u] < TOD_N_PSI;
-            m[u] = __ldg(map + (in[u] ? pp[u] : 0));
-            cs[u] = __ldg(trig + (in[u] ? bb[u] : 0u));
+            m[u] = __ldg(map + min(static_cast<uint32_t>(pp[u]), static_cast<uint32_t>(npix) - 1u));
+            cs[u] = __ldg(trig + min(bb[u], static_cast<uint32_t>(TOD_N_PSI) - 1u));
         }
-        if (!(in[0] && in[1] && in[2] && in[3])) set_status(status, q, TOD_ERR_ARG);
         float v[4];
+        bool in = true;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = in[u] ? g * fmaf(m[u].z, cs[u].y, fmaf(m[u].y, cs[u].x, m[u].x)) : 0.0f;
+        for (int u = 0; u < 4; ++u) {
+            v[u] = g * fmaf(m[u].z, cs[u].y, fmaf(m[u].y, cs[u].x, m[u].x));
+            in = in && static_cast<uint32_t>(pp[u]) < static_cast<uint32_t>(npix) && bb[u] < TOD_N_PSI;
+        }
+        if (!in) {
+            set_status(status, q, TOD_ERR_ARG);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (!(static_cast<uint32_t>(pp[u]) < static_cast<uint32_t>(npix) && bb[u] < TOD_N_PSI)) v[u] = 0.0f;
+        }
         const float4 o = make_float4(v[0], v[1], v[2], v[3]);
         *reinterpret_cast<float4 *>(s_out + t) = o;
     }
