@@ -50,7 +50,9 @@ static_assert((1 << DEC_LUTB) % (4 * DEC_T) == 0, "the table is staged 16 bytes 
 // fl32 of the FP64 product c * scale (scale = s1 + s2 + ..., FP32 parts) in
 // FP32: the product as head + tail to about 2^-46, rounded; where that lies
 // too near a rounding boundary to be sure (or out of the easy range), the
-// FP64 product itself (FP64 issues at 1/64 of the FP32 rate here).
+// FP64 product itself (FP64 issues at 1/64 of the FP32 rate here).  A count of
+// zero is zero whatever the scale, which is positive and finite but may lie
+// past FP32's range.
 __device__ __forceinline__ float tod_value(int32_t c, float s1, float s2, double scale) {
     const float fc = static_cast<float>(c);
     const float ph = __fmul_rn(fc, s1);
@@ -61,7 +63,7 @@ __device__ __forceinline__ float tod_value(int32_t c, float s1, float s2, double
     const float half = __uint_as_float(rb & 0x7f800000u) * 5.9604644775390625e-08f;    // half an ulp of r
     const bool sure = c == 0 || (e < 0.9999f * half && (rb & 0x7fffffu) != 0u && abs(c) < (1 << 24) &&
                                  fabsf(r) > 1e-25f && fabsf(r) < 1e25f);
-    return sure ? r : __double2float_rn(static_cast<double>(c) * scale);
+    return !sure ? __double2float_rn(static_cast<double>(c) * scale) : c == 0 ? 0.0f : r;
 }
 
 template <typename OutT, int KIND>
