@@ -1102,9 +1102,10 @@ __global__ void __launch_bounds__(TX_T, sizeof(V) == sizeof(CF2) ? TX_CTAS_COL :
                 // one logarithm for the four modes (an FP64 one takes about 30
                 // operations, at 1/64 of the FP32 rate: 25 scans of 4 x 65536,
                 // rows 2168 -> 1815 us) of the product, which leaves the range
-                // only past 1e72 a mode: then one each
-                const S pr = (P0.a * P0.b) * (P1.a * P1.b);
-                if (pr > S(1e-290) && pr < S(1e290)) {
+                // only past 1e72 a mode: then one each (also where half the
+                // product is below 2^-963, which the other half may hide)
+                const S pa = P0.a * P0.b, pb = P1.a * P1.b, pr = pa * pb;
+                if (min(__double2hiint(pa), __double2hiint(pb)) > 0x03c00000 && pr > S(1e-290) && pr < S(1e290)) {
                     sum[0].add(pset(log(pr), S(0)));
                 } else {
                     sum[0].add(pset(log(P0.a), log(P0.b)));
