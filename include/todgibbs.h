@@ -145,7 +145,8 @@ typedef struct {
                                widest tile that fits, else a cap 1..64 (the tile takes the
                                largest power of two not above it) */
     int32_t device;         /* CUDA device ordinal the plan lives on */
-    int32_t max_radix;      /* largest Stockham radix of the transforms: 0 = 16; else 2..16 */
+    int32_t max_radix;      /* largest Stockham radix of the transforms, 2..16 (10 is the largest there
+                               is: more means 10); 0: no bound */
 } tod_band_desc;
 
 /* Counter-based random streams: Philox4x64-10 (Salmon et al. 2011) with key

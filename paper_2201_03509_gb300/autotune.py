@@ -44,7 +44,7 @@ def autotune(nside: int, ndet: int, nscan: int, fsamp: float, offsets: np.ndarra
     g = torch.zeros(nq, dtype=torch.float64, device=dev)
     its = torch.zeros(nq, dtype=torch.int32, device=dev)
     if candidates is None:
-        candidates = [(t, r) for t in (0, 4, 8) for r in (8, 16)]
+        candidates = [(t, r) for t in (0, 4, 8) for r in (8, 16)]      # 16: no bound, the largest radix there is
     timings = {}
     for (c, r) in candidates:
         try:

@@ -414,7 +414,7 @@ k_reduce(const double *__restrict__ rec, const int64_t *__restrict__ pix_slot_of
 static unsigned reduce_grid(const Plan &p)
 {
     const int64_t ctas = (static_cast<int64_t>(p.npix) + RED_T - 1) / RED_T;
-    return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(ctas, 152 * 8 * 8)));
+    return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(ctas, static_cast<int64_t>(p.sm_count) * 8 * 8)));
 }
 
 // Shards' pairs of pixels [0, np) added in rank order as double-doubles,

@@ -56,7 +56,7 @@ __device__ __forceinline__ void cp_async_bytes8(void *dst, const void *src) {
 // tile) and the detscans' length indices, fetched by thread 0 two tiles and
 // one tile ahead of their use into a ring in shared memory (two dependent
 // loads, about a microsecond, in front of every tile otherwise; in registers
-// the row passes spilled more).  n_corr draw of 6 x 45 detscans at 44 GHz, this
+// the row passes spilled more).  n_corr draw of 6 x 18 detscans at 44 GHz, this
 // and the single round of loads in tx_begin: 2335 -> 2196 us; chi^2 of 52M
 // samples, with the spectrum's logarithm once per detscan: 2336 -> 2240 us.
 struct ItemFeed {
@@ -1261,7 +1261,8 @@ __global__ void __launch_bounds__(256) k_chi2_total(const double *__restrict__ c
 // sample flagged has A = C^T diag(phi) C: x is its exact spectral solution
 // (the offset mode, unconstrained, set to zero).
 //
-// One cooperative launch: phases separated by grid barriers.
+// One launch per pass, and one cooperative launch (grid barriers between its
+// passes) for the CG iterations past the launched ones.
 // ===========================================================================
 struct NcorrTx {
     const float *d, *s;
@@ -1303,7 +1304,7 @@ struct NcorrTx {
     int32_t *gnb;                 // [nq]
     float *cgv;                   // [5][cgcap]
     int64_t cgcap;
-    int32_t *count;               // [2]
+    int32_t *count;               // [3] active detscans (alternating), arrivals at the list
     float4 *qsc;                  // [nq][2] per-detscan FP32 scalars, written in the index phase
     // the detscans a CG pass works on, in order, with the running counts of
     // their column and row items: list[0] = n, then q[nq], col[nq + 1], row[nq + 1]
@@ -2631,7 +2632,10 @@ static_assert(kGbBytes <= sizeof(CF2) * 2 * TX_PAIRS, "the preconditioner stagin
 // the cooperative tail, whose grid barriers cost what a launch does.  Launches
 // past the last iteration return at once but cost 2 us each (four an
 // iteration), and the tail costs as much as they do: three launched
-// iterations leave it the few stragglers.
+// iterations leave it the few stragglers.  With eight the two-level draw of
+// 16 x 4096 samples takes 465 us instead of 383, of 72 x 225k 2228 instead of
+// 2175; without a preconditioner (12 and 21 iterations on average and at most)
+// that of 72 x 225k 5102 instead of 5226, of 40 x 115k 3811 instead of 3829.
 constexpr int NC_LAUNCHED_ITERS = 3;
 
 template <class K>
