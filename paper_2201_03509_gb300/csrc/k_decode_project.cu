@@ -20,7 +20,7 @@
 // branch but those to a refill and to the long codes, whose symbols are staged
 // in shared memory too when a scan has at most DEC_CANON of them (30 % of the
 // 70 GHz pixel symbols are longer than the table).  27M samples of pointing:
-// 474 -> 268 us; of TOD 305 -> 232, of flags 149 -> 73 us; 65k samples 111 -> 63 us
+// 474 -> 268 us; of TOD 305 -> 151, of flags 149 -> 73 us; 65k samples 111 -> 63 us
 // a stream; 102M samples of 70 GHz pointing 1972 -> 784 us.  A symbol's chain of
 // dependent operations is the bound.  (Asking L2 for a block's lines at its
 // start cost 15 %, a ring of eight chunks gained nothing.)
